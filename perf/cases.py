@@ -98,18 +98,34 @@ def _params(case):
     return sd.make_params(case["block"], case["keep"], case["prompt"])
 
 
-def _pattern_from_means(q, k, case, params, ws):
-    """The pattern a loop in its sparse phase has in hand. It is ranked here on block-mean scores taken with plain tensor
-    operations (on these inputs they keep 98-99 % of the blocks the exact scores do), so that it is the same pattern
-    whatever the scoring kernels' rounding is."""
+def _inputs(case, seed):
+    cfg = synthetic.AttnConfig("perf", case["batch"], case["heads_q"], case["heads_kv"], case["tokens"], HEAD_DIM,
+                               case["block"], case["keep"], case["prompt"], seed=seed, plant_norm=case["norm"])
+    q, k, v = synthetic.make_qkv(cfg, torch.device("cuda"))
+    if case["layout"] == "token":
+        q, k, v = (t.transpose(1, 2).contiguous().transpose(1, 2) for t in (q, k, v))
+    return q, k, v
+
+
+def _mean_scores(q, k, block):
+    """Block-mean scores, taken with plain tensor operations. A loop's pattern is ranked on these here (on these inputs
+    they keep 98-99 % of the blocks the exact scores do), so that it is the same pattern whatever the scoring kernels'
+    rounding is."""
     B, H, L, D = q.shape
-    bs, nb, group = case["block"], L // case["block"], H // k.shape[1]
+    bs, nb, group = block, L // block, H // k.shape[1]
     scores = torch.empty(B, H, nb, nb, dtype=torch.float32, device=q.device)
     for b in range(B):
         for h in range(H):
             mq = q[b, h].float().reshape(nb, bs, D).mean(1)
             mk = k[b, h // group].float().reshape(nb, bs, D).mean(1)
             scores[b, h] = torch.softmax(mq @ mk.t() / math.sqrt(D), dim=-1)
+    return scores
+
+
+def _pattern_from_means(q, k, case, params, ws):
+    """The pattern a loop in its sparse phase has in hand."""
+    B, H, L, _ = q.shape
+    nb, scores = L // case["block"], _mean_scores(q, k, case["block"])
     k_pre, k_gen = sd.sparsed_kept_per_row(params, L)
     pat, row_ptr, col_idx = sd.new_pattern(B, H, nb, k_pre + k_gen, q.device)
     sd.sparsed_select_from_scores(scores, params, pat, ws)
@@ -117,12 +133,8 @@ def _pattern_from_means(q, k, case, params, ws):
 
 
 def prepare(case, seed):
-    dev = torch.device("cuda")
-    cfg = synthetic.AttnConfig("perf", case["batch"], case["heads_q"], case["heads_kv"], case["tokens"], HEAD_DIM,
-                               case["block"], case["keep"], case["prompt"], seed=seed, plant_norm=case["norm"])
-    q, k, v = synthetic.make_qkv(cfg, dev)
-    if case["layout"] == "token":
-        q, k, v = (t.transpose(1, 2).contiguous().transpose(1, 2) for t in (q, k, v))
+    q, k, v = _inputs(case, seed)
+    dev = q.device
     state = {"phase": case["phase"], "q": q, "k": k, "v": v, "params": _params(case), "lse": None, "scores": None}
     params, phase = state["params"], case["phase"]
     if phase == "select":
@@ -167,6 +179,57 @@ def run(state):
     if phase == "switch":
         return {"o": state["o"], "row_ptr": state["row_ptr"], "col_idx": state["col_idx"]}
     return {"o": state["o"]}
+
+
+def _kept_blocks(scores, case):
+    """[nb, kept] ids of the blocks that each row of a head's scores keeps: the best of the prompt's blocks and of the
+    others, each ranked by itself, ties to the lower id, in ascending order."""
+    nb, ids, first = scores.shape[-1], [], 0
+    split = case["prompt"] // case["block"]
+    for end in ([split] if 0 < split < nb else []) + [nb]:
+        kept = min(max(math.ceil(case["keep"] * (end - first) - 1e-6), 1), end - first)
+        order = torch.sort(scores[:, first:end], dim=-1, descending=True, stable=True).indices[:, :kept]
+        ids.append(order + first)
+        first = end
+    return torch.cat(ids, dim=-1).sort(dim=-1).values
+
+
+def exact(case, seed):
+    """What run() returns, from plain tensor operations in 64 bits. Lists of blocks that are chosen by exact scores have no
+    such value here: see tolerance()."""
+    if case["phase"] == "select" and not case["scores"]:
+        return None
+    q, k, v = _inputs(case, seed)
+    B, H, L, D = q.shape
+    bs, nb, group = case["block"], L // case["block"], H // k.shape[1]
+    o = torch.empty(B, H, L, D, dtype=torch.float64, device=q.device) if case["phase"] != "select" else None
+    pooled = torch.empty(B, H, nb, nb, dtype=torch.float64, device=q.device) if case["phase"] == "select" else None
+    means = _mean_scores(q, k, bs) if case["phase"] == "sparse" else None
+    for b in range(B):
+        for h in range(H):
+            qh = q[b, h].double() / math.sqrt(D)
+            kh, vh = k[b, h // group].double(), v[b, h // group].double()
+            if case["phase"] == "sparse":
+                ids = _kept_blocks(means[b, h], case)
+                step = max(1, (1 << 25) // (ids.shape[1] * bs * D))
+                kb, vb, qb = kh.reshape(nb, bs, D), vh.reshape(nb, bs, D), qh.reshape(nb, bs, D)
+                for i in range(0, nb, step):
+                    at = ids[i:i + step]
+                    p = torch.softmax(qb[i:i + step] @ kb[at].flatten(1, 2).transpose(1, 2), dim=-1)
+                    o[b, h, i * bs:(i + step) * bs] = (p @ vb[at].flatten(1, 2)).flatten(0, 1)
+                continue
+            step = max(bs, (1 << 27) // L // bs * bs)
+            for i in range(0, L, step):
+                p = torch.softmax(qh[i:i + step] @ kh.t(), dim=-1)
+                if pooled is not None:
+                    pooled[b, h, i // bs:(i + step) // bs] = p.reshape(-1, bs, nb, bs).mean(dim=(1, 3))
+                else:
+                    o[b, h, i:i + step] = p @ vh
+    if case["phase"] == "select":
+        return {"row_ptr": None, "col_idx": None, "scores": pooled}
+    if case["phase"] == "switch":
+        return {"o": o, "row_ptr": None, "col_idx": None}
+    return {"o": o}
 
 
 def work(case):
