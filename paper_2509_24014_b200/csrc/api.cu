@@ -603,11 +603,14 @@ sparsed_status sparsed_select_pattern(const sparsed_shape* shape, const sparsed_
     return st;
   // With few enough blocks per row the pooled-scoring kernel ranks each block-row in its own
   // tail; A' then goes to memory only if the caller asked for it.
-  const bool fused = nb <= kFusedTopkMaxBlocks && params->block_size != 32;
+  const bool fused = score_ranks_in_kernel(nb, params->block_size);
+  // Up to 128 key blocks per row it also needs no log-sum-exp pass before it (one exponential per logit instead of
+  // two). The workspace asked for is that of the longest route either way.
+  const bool one_pass = lse_or_null == nullptr && score_in_one_pass(nb);
   const size_t bh = static_cast<size_t>(shape->batch) * shape->heads_q;
   const size_t score_bytes = round_up(bh * nb * nb * 4, 256);
   const size_t lse_bytes = round_up(bh * static_cast<size_t>(shape->seq_len) * 4, 256);
-  const bool need_score_ws = !fused && scores_out_or_null == nullptr;
+  const bool need_score_ws = (nb > 1024 || params->block_size == 32) && scores_out_or_null == nullptr;
   const size_t required = SPARSED_STATUS_BYTES + (need_score_ws ? score_bytes : 0) + (lse_or_null ? 0 : lse_bytes);
   if ((st = check_ws(ws, ws_bytes, required)) != SPARSED_OK) return st;
   if ((st = check_arch()) != SPARSED_OK) return st;
@@ -621,9 +624,9 @@ sparsed_status sparsed_select_pattern(const sparsed_shape* shape, const sparsed_
   }
   CUtensorMap tq, tk;
   if ((st = make_tensor_map(&tq, q, shape->batch, shape->heads_q, shape->seq_len, rs.q, 128)) != SPARSED_OK) return st;
-  if ((st = make_tensor_map(&tk, k, shape->batch, shape->heads_kv, shape->seq_len, rs.k, 128)) != SPARSED_OK) return st;
+  if ((st = make_tensor_map(&tk, k, shape->batch, shape->heads_kv, shape->seq_len, rs.k, 64)) != SPARSED_OK) return st;
   ScoreParams sp;
-  sp.scores = scores;
+  sp.scores = fused ? scores_out_or_null : scores;
   sp.lse = lse_or_null;
   sp.seq_len = shape->seq_len;
   sp.heads_q = shape->heads_q;
@@ -636,11 +639,12 @@ sparsed_status sparsed_select_pattern(const sparsed_shape* shape, const sparsed_
   sp.pb = pb;
   sp.k_pre = k_pre;
   sp.k_gen = k_gen;
-  if (lse_or_null == nullptr) {
-    float* lse_buf = reinterpret_cast<float*>(base + off);
-    cudaError_t e = launch_row_stats(tq, tk, sp, lse_buf, shape->batch, stream);
+  sp.lse_out = nullptr;
+  if (lse_or_null == nullptr && !one_pass) {
+    sp.lse_out = reinterpret_cast<float*>(base + off);
+    cudaError_t e = launch_row_stats(tq, tk, sp, shape->batch, stream);
     if (e != cudaSuccess) return cuda_fail(e);
-    sp.lse = lse_buf;
+    sp.lse = sp.lse_out;
   }
   cudaError_t e = launch_pooled_scores(tq, tk, sp, shape->batch, stream);
   if (e != cudaSuccess) return cuda_fail(e);

@@ -60,7 +60,8 @@ struct AttnParams {
 // Parameters of the pooled-scoring kernel.
 struct ScoreParams {
   float* scores;           // fp32 [B,Hq,nb,nb], or null when only the pattern is wanted (fused top-k)
-  const float* lse;        // fp32 [B,Hq,L], natural log
+  const float* lse;        // fp32 [B,Hq,L], natural log; null: not known (one pass, few enough key blocks)
+  float* lse_out;          // row-statistics pass: fp32 [B,Hq,L], natural log
   int seq_len;
   int heads_q;
   int group;
@@ -72,9 +73,6 @@ struct ScoreParams {
   int32_t* col_idx;
   int pb, k_pre, k_gen;
 };
-
-// Largest number of key blocks per row the pooled-scoring kernel can rank in its own tail.
-constexpr int kFusedTopkMaxBlocks = 1024;
 
 // Parameters of the kernel that pools per-tile row statistics into A' and ranks it.
 struct PoolParams {
@@ -130,8 +128,11 @@ int attn_sparse_max_blocks(int block_size);   // most key blocks per row the spa
 cudaError_t launch_attn_sparse(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv,
                                const CUtensorMap& to, const AttnParams& p, int batch, int block_size,
                                cudaStream_t stream);
-cudaError_t launch_row_stats(const CUtensorMap& tq, const CUtensorMap& tk, const ScoreParams& p, float* lse_out,
-                             int batch, cudaStream_t stream);
+bool score_ranks_in_kernel(int nb, int block_size);   // the pooled-scoring kernel ranks rows of nb key blocks itself
+bool score_in_one_pass(int nb);                       // ... and needs no log-sum-exp of the rows
+// (K tensor map of both: boxes of 64 x 64 rows)
+cudaError_t launch_row_stats(const CUtensorMap& tq, const CUtensorMap& tk, const ScoreParams& p, int batch,
+                             cudaStream_t stream);
 cudaError_t launch_pooled_scores(const CUtensorMap& tq, const CUtensorMap& tk, const ScoreParams& p, int batch,
                                  cudaStream_t stream);
 cudaError_t launch_topk_csr(const TopkParams& p, cudaStream_t stream);

@@ -1,45 +1,121 @@
-// Block-pooled attention scores A' = avgpool(softmax(Q K^T / sqrt(d)), block_size)
-// ("Isolated Selection"; the avgpool line of Algorithm 1), streamed one 128-row query tile
-// at a time so that the l x l matrix is never stored.
+// Block-pooled attention scores A' = avgpool(softmax(Q K^T / sqrt(d)), block_size) from Q and K alone
+// ("Isolated Selection"; the avgpool line of Algorithm 1), streamed one 128-row query tile at a time so that
+// the l x l matrix is never stored.
 //
-// Two kernels built from one template:
-//   * row statistics : LSE_i = ln sum_j exp(s_ij) by online max/sum (only needed when the
-//                      caller has no LSE from the full-attention pass of the same step);
-//   * pooled scores  : p_ij = exp(s_ij - LSE_i) is the exactly normalised probability, so
-//                      each 128x128 logit tile can be reduced to its block sums at once.
-// Pipeline per CTA: warp 4 streams K tiles by TMA (two stages), warp 5 issues S = Q K^T
-// into one of two tensor-memory buffers, warps 0-3 (one thread per query row) exponentiate
-// and reduce. Sums run in a fixed order, so results are bitwise reproducible.
-// With a pattern to fill (row_ptr != null) warp 0 also keeps the block-row(s) it produced as
-// ordered keys in shared memory and, after the last tile, runs the isolated top-k of Eq. 5/6
-// on them and writes the CSR lists: selection then needs no pass over A' in memory.
+// What bounds it: one exponential per logit. The SM's exponential unit does 16 a clock, so a 128 x 64 tile of
+// logits takes 512 clocks there against 384 on the tensor pipe (eight M128 N64 K16 MMAs at 48 clocks). Every logit
+// is therefore exponentiated ONCE where that is possible:
+//
+//   * kOnePass  the row sums of every key block are kept, relative to a per-row reference that is fixed with the
+//               first tile, until the row's denominator is known; then they are divided by it and summed over the
+//               rows of each query block. One fp32 per row and key block, in the tensor-memory columns that the
+//               two logit buffers leave free: 128 of them, so up to 128 key blocks per row.
+//   * kPooled   the caller (or a kRowStats pass) has the rows' log-sum-exp: p = exp(s - LSE) is the probability
+//               itself, and the block sums are folded into A' whenever 128 of them have come together.
+//   * kRowStats log-sum-exp of every row: the first of the two passes that rows with more than 128 key blocks
+//               take.
+//
+// Pipeline per CTA (320 threads, two CTAs per SM): warp 8 streams 64-key K tiles by TMA into a ring of four, warp 9
+// issues S = Q K^T (one commit per tile: "S ready" for the softmax warps, "slot free" for the producer), warps 0-3 and
+// 4-7 are two groups with one thread per query row each. The groups take turns at 128 keys (two tiles), so that a key
+// block belongs to one of them; each has one S buffer, its own row references and its own denominators, which meet at
+// the end. A thread copies its row of S into registers, hands the buffer back at once, exponentiates and sums. Four
+// such warps per scheduler cover each other's waits: with two (one group per CTA, two S buffers) the first case below
+// took 2.53 ms, with the next tile's copy pipelined into the current one's exponentials as well 2.70 ms.
+// Sums run in a fixed order, so results are bitwise reproducible. When the keys of its block-row(s) fit in shared
+// memory the CTA ranks them itself (warp_select_row) and writes the CSR lists.
+//
+// Measured on B200, from Q and K alone (two passes over the logits before, with two CTAs of four softmax warps):
+//   28 heads x 16384 tokens, block 128   6.21 -> 2.50 ms (kOnePass; exponential unit busy 82 % of the time)
+//   32 heads x 8192 tokens, block 128    1.79 -> 0.73 ms (kOnePass)
+//   8 heads x 65536 tokens, block 128    27.5 -> 22.0 ms (kRowStats + kPooled)
 #include "internal.h"
+#include "softmax_pipeline.cuh"
 #include "topk_device.cuh"
 
 namespace sparsed {
 namespace {
 
 constexpr int kHeadDim = 128;
-constexpr int kTile = 128;
-constexpr int kThreads = 192;
+constexpr int kTileM = 128;     // query rows per CTA
+constexpr int kTileN = 64;      // keys per pipeline step
+constexpr int kThreads = 320;
+constexpr int kSlots = 4;       // 16 KB ring slots, one K tile each
 constexpr int kTmemCols = 256;
-constexpr int kStages = 2;
+constexpr int kColStat = 128;   // columns 0-127: one S buffer per group; 128-255: one block sum per column and row
+constexpr int kChunk = 128;     // block sums held per row
+constexpr int kMaxKeys = 2048;  // ranking keys held in shared memory: (block-rows per tile) x (key blocks per row)
+
+enum ScoreMode { kOnePass, kPooled, kRowStats };
+
+// A row's reference is the maximum of its first 32 logits and stays until a sum outgrows this: only fp32 sums are taken
+// here (no bf16 probabilities), so 2^60 is as safe as 1, and what an outgrown reference would lose at the other end of
+// the fp32 range is below 2^-66 of the row's sum.
+constexpr float kOutgrown = 1152921504606846976.f;   // 2^60
 
 struct ScoreSmem {
-  alignas(1024) __nv_bfloat16 q[2][kTile * 64];
-  alignas(1024) __nv_bfloat16 k[kStages][2][kTile * 64];
-  uint64_t q_full, k_full[kStages], s_full[2], s_empty[2], partial_full[4];
-  float partial[4][4][2];  // [tile % 4][warp][column half]
-  uint32_t keys[2][kFusedTopkMaxBlocks];  // ordered keys of the block-row(s) of this CTA (fused top-k)
-  int hist[256];
+  alignas(1024) __nv_bfloat16 q[2][kTileM * 64];           // two 64-wide halves of head_dim
+  alignas(1024) __nv_bfloat16 k[kSlots][2][kTileN * 64];   // each slot: two 64-wide halves of head_dim
+  uint32_t keys[kMaxKeys];          // ordered keys of this CTA's block-row(s)
+  float quarter[4][kChunk];         // block sums over each 32-row quarter of the tile
+  int hist[4][256];                 // one histogram per ranking warp
+  uint64_t q_full, k_full[kSlots];
+  uint64_t done[kSlots];            // the MMAs that read the slot have completed: S of that tile is ready
+  uint64_t s_free[2];               // every warp of the group has copied its rows of the S buffer into registers
+  float2 ml[2][kTileM];             // each group's (reference, denominator) of each row
   uint32_t tmem_base;
   int abort_flag;
 };
 
-template <bool kStatsOnly>
+// One 32-bit cell per lane, at the warp's lanes of column `taddr`.
+__device__ __forceinline__ void tmem_st1(uint32_t taddr, float v) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x1.b32 [%0], {%1};" ::"r"(taddr), "r"(__float_as_uint(v)) : "memory");
+}
+
+// v[j] of lane i = element (i, j): returns sum over i of element (i, lane), added pairwise in a fixed tree.
+__device__ __forceinline__ float warp_column_sums(float (&v)[32], int lane) {
+#pragma unroll
+  for (int half = 16; half > 0; half >>= 1) {
+    const bool upper = (lane & half) != 0;
+#pragma unroll
+    for (int j = 0; j < half; ++j) {
+      const float keep = upper ? v[j + half] : v[j];
+      const float give = upper ? v[j] : v[j + half];
+      v[j] = keep + __shfl_xor_sync(0xffffffffu, give, half);
+    }
+  }
+  return v[0];
+}
+
+// Block sums of one row in n columns at t_stat times alpha.
+__device__ __noinline__ void rescale_block_sums(uint32_t t_stat, int n, float alpha) {
+  for (int c = 0; c < n; ++c) {
+    uint32_t r;
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(r) : "r"(t_stat + c) : "memory");
+    tmem_wait_ld();
+    tmem_st1(t_stat + c, __uint_as_float(r) * alpha);
+  }
+}
+
+// Sum of 2^(scale * s - m) over 32 columns.
+__device__ __forceinline__ float exp_sum(const uint32_t (&r)[32], float scale_log2, float m) {
+  const float2 sc = make_float2(scale_log2, scale_log2);
+  const float2 nm = make_float2(-m, -m);
+  float2 a0 = make_float2(0.f, 0.f), a1 = make_float2(0.f, 0.f);
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    const float2 x0 = __ffma2_rn(make_float2(__uint_as_float(r[4 * j]), __uint_as_float(r[4 * j + 1])), sc, nm);
+    const float2 x1 = __ffma2_rn(make_float2(__uint_as_float(r[4 * j + 2]), __uint_as_float(r[4 * j + 3])), sc, nm);
+    a0 = __fadd2_rn(a0, make_float2(fast_exp2(x0.x), fast_exp2(x0.y)));
+    a1 = __fadd2_rn(a1, make_float2(fast_exp2(x1.x), fast_exp2(x1.y)));
+  }
+  const float2 a = __fadd2_rn(a0, a1);
+  return a.x + a.y;
+}
+
+template <int kMode>
 __global__ void __launch_bounds__(kThreads, 2)
-score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
-             const ScoreParams p, float* lse_out) {
+score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k, const ScoreParams p) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   ScoreSmem& sm = *reinterpret_cast<ScoreSmem*>(smem_raw);
   if ((smem_u32(smem_raw) & 1023u) != 0u) {
@@ -48,28 +124,56 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
   }
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
-  const int num_q_tiles = (p.seq_len + kTile - 1) / kTile;
-  const int num_tiles = num_q_tiles;
+  const int num_q_tiles = (p.seq_len + kTileM - 1) / kTileM;
+  const int num_tiles = (p.seq_len + kTileN - 1) / kTileN;
   const int q_tile = blockIdx.x % num_q_tiles;
   const int bh = blockIdx.x / num_q_tiles;
   const int head = bh % p.heads_q;
   const int batch = bh / p.heads_q;
   const int kv_head = head / p.group;
-  const int q_row0 = q_tile * kTile;
+  const int q_row0 = q_tile * kTileM;
 
-  if (tid == 0) {
-    mbar_init(&sm.q_full, 1);
-    static_assert(kStages == 2, "K stage and S buffer of a tile share one index and one completion barrier");
-    for (int s = 0; s < kStages; ++s) mbar_init(&sm.k_full[s], 1);
-    for (int s = 0; s < 2; ++s) {
-      mbar_init(&sm.s_full[s], 1);
-      mbar_init(&sm.s_empty[s], 128);
+  // Group g takes tiles 4i + 2g and 4i + 2g + 1. Its j-th tile is key tile tile_of(g, j); counted over both groups it is
+  // number index_of(g, j) in the order in which tiles are loaded and multiplied: the groups alternate as long as both
+  // have tiles left (group 0 has up to two more).
+  const int tiles1 = (num_tiles >> 2) * 2 + max((num_tiles & 3) - 2, 0);
+  const int tiles0 = num_tiles - tiles1;
+  auto tile_of = [&](int g, int j) -> int { return (j >> 1) * 4 + 2 * g + (j & 1); };
+  auto index_of = [&](int g, int j) -> int { return j < tiles1 ? 2 * j + g : tiles1 + j; };
+  auto group_of = [&](int i) -> int { return i < 2 * tiles1 ? (i & 1) : 0; };
+  auto step_of = [&](int i) -> int { return i < 2 * tiles1 ? (i >> 1) : i - tiles1; };   // j of number i
+
+  // ---- set-up (the producer warp owns the barriers of its loads and starts them right away) -------
+  if (warp == 8) {
+    if (lane == 0) {
+      mbar_init(&sm.q_full, 1);
+      for (int s = 0; s < kSlots; ++s) mbar_init(&sm.k_full[s], 1);
+      mbar_fence_init();
     }
-    for (int s = 0; s < 4; ++s) mbar_init(&sm.partial_full[s], 4);
+    __syncwarp();
+  }
+  auto issue_k_load = [&](int i) {
+    const int slot = i % kSlots;
+    const int key0 = tile_of(group_of(i), step_of(i)) * kTileN;
+    mbar_expect_tx(&sm.k_full[slot], kTileN * kHeadDim * 2);   // keys beyond the sequence arrive as zeros
+    tma_load_4d(sm.k[slot][0], &tm_k, &sm.k_full[slot], 0, key0, kv_head, batch);
+    tma_load_4d(sm.k[slot][1], &tm_k, &sm.k_full[slot], 64, key0, kv_head, batch);
+  };
+  if (warp == 8 && elect_one_sync()) {
+    tma_prefetch_desc(&tm_q);
+    tma_prefetch_desc(&tm_k);
+    mbar_expect_tx(&sm.q_full, kTileM * kHeadDim * 2);
+    tma_load_4d(sm.q[0], &tm_q, &sm.q_full, 0, q_row0, head, batch);
+    tma_load_4d(sm.q[1], &tm_q, &sm.q_full, 64, q_row0, head, batch);
+    for (int i = 0; i < min(num_tiles, kSlots); ++i) issue_k_load(i);
+  }
+  if (tid == 0) {
+    for (int s = 0; s < kSlots; ++s) mbar_init(&sm.done[s], 1);
+    for (int s = 0; s < 2; ++s) mbar_init(&sm.s_free[s], 4);
     sm.abort_flag = 0;
     mbar_fence_init();
   }
-  if (warp == 5) {
+  if (warp == 9) {
     tmem_alloc(&sm.tmem_base, kTmemCols);
     tmem_relinquish();
   }
@@ -78,232 +182,237 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
   tc_fence_after();
   const uint32_t tmem = sm.tmem_base;
 
-  if (warp == 4) {
-    if (lane == 0) {
-      tma_prefetch_desc(&tm_q);
-      tma_prefetch_desc(&tm_k);
-      mbar_expect_tx(&sm.q_full, kTile * kHeadDim * 2);
-      tma_load_4d(sm.q[0], &tm_q, &sm.q_full, 0, q_row0, head, batch);
-      tma_load_4d(sm.q[1], &tm_q, &sm.q_full, 64, q_row0, head, batch);
-      for (int it = 0; it < num_tiles; ++it) {
-        const int s = it % kStages;
-        const int use = it / kStages;
-        // the stage's previous K tile has been read once the S buffer of the same index is complete
-        if (use > 0 && !mbar_wait(&sm.s_full[s], (use - 1) & 1, &sm.abort_flag, p.status, 40)) break;
-        mbar_expect_tx(&sm.k_full[s], kTile * kHeadDim * 2);
-        tma_load_4d(sm.k[s][0], &tm_k, &sm.k_full[s], 0, it * kTile, kv_head, batch);
-        tma_load_4d(sm.k[s][1], &tm_k, &sm.k_full[s], 64, it * kTile, kv_head, batch);
-      }
+  if (warp == 8) {
+    // =============================== TMA producer =======================================
+    bool ok = true;
+    for (int i = kSlots; ok && i < num_tiles; ++i) {
+      ok = mbar_wait(&sm.done[i % kSlots], (i / kSlots - 1) & 1, &sm.abort_flag, p.status, 40);
+      ok = __all_sync(0xffffffffu, ok);
+      if (ok && elect_one_sync()) issue_k_load(i);
+      __syncwarp();
     }
-  } else if (warp == 5) {
-    if (lane == 0) {
-      constexpr uint32_t idesc = umma_idesc_bf16(kTile, kTile, false, false);
-      const uint32_t q_addr[2] = {smem_u32(sm.q[0]), smem_u32(sm.q[1])};
-      bool ok = mbar_wait(&sm.q_full, 0, &sm.abort_flag, p.status, 50);
-      for (int it = 0; ok && it < num_tiles; ++it) {
-        const int s = it % kStages;
-        const int buf = it & 1;
-        if (!mbar_wait(&sm.k_full[s], (it / kStages) & 1, &sm.abort_flag, p.status, 51)) break;
-        if (it >= 2 && !mbar_wait(&sm.s_empty[buf], ((it >> 1) - 1) & 1, &sm.abort_flag, p.status, 52)) break;
-        tc_fence_after();
-        const uint32_t k_addr[2] = {smem_u32(sm.k[s][0]), smem_u32(sm.k[s][1])};
-#pragma unroll
-        for (int kk = 0; kk < kHeadDim / 16; ++kk) {
-          const uint32_t off = (kk & 3) * 32;
-          umma_ss(tmem + buf * kTile, umma_smem_desc_sw128(q_addr[kk >> 2] + off, 16, 1024),
-                  umma_smem_desc_sw128(k_addr[kk >> 2] + off, 16, 1024), idesc, kk > 0);
-        }
-        umma_commit(&sm.s_full[buf]);   // one commit: "S ready" for the softmax warps, "K stage free" for the producer
-      }
+  } else if (warp == 9) {
+    // =============================== UMMA issuer ========================================
+    const uint32_t q_lo0 = umma_desc_lo(smem_u32(sm.q[0]), 16);
+    const uint32_t k_lo0 = umma_desc_lo(smem_u32(sm.k[0][0]), 16);
+    constexpr uint32_t slot_step = (2 * kTileN * 64 * 2) >> 4;   // 16 KB per ring slot
+    bool ok = mbar_wait(&sm.q_full, 0, &sm.abort_flag, p.status, 50);
+    ok = __all_sync(0xffffffffu, ok);
+    for (int i = 0; ok && i < num_tiles; ++i) {
+      const int slot = i % kSlots;
+      const int g = group_of(i), j = step_of(i);
+      ok = j == 0 ? mbar_wait(&sm.k_full[slot], (i / kSlots) & 1, &sm.abort_flag, p.status, 51)
+                  : mbar_wait2(&sm.k_full[slot], (i / kSlots) & 1, &sm.s_free[g], (j - 1) & 1, &sm.abort_flag, p.status, 52);
+      ok = __all_sync(0xffffffffu, ok);
+      if (ok) issue_qk64(tmem + g * kTileN, q_lo0, k_lo0 + slot * slot_step, &sm.done[slot]);
     }
   } else {
-    const uint32_t lane_base = static_cast<uint32_t>(warp * 32) << 16;
+    // =============================== exponentials, block sums, ranking ===================
+    const int g = warp >> 2;              // group
+    const int wq = warp & 3;              // 32-row quarter of the tile
+    const int rit = tid & (kTileM - 1);   // row in tile
+    const uint32_t lane_base = static_cast<uint32_t>(wq * 32) << 16;
+    const uint32_t t_stat = tmem + kColStat + lane_base;
     const float scale_log2 = p.scale_log2;
-    const int row = q_row0 + tid;
+    const int row = q_row0 + rit;
     const bool row_valid = row < p.seq_len;
-    // pooled mode: natural-log LSE -> base-2 offset
-    float lse2 = 0.f;
-    if constexpr (!kStatsOnly) {
-      lse2 = row_valid ? p.lse[static_cast<int64_t>(bh) * p.seq_len + row] * 1.44269504088896341f : INFINITY;
+    const int bs = p.block_size;
+    const int nb = kMode == kRowStats ? 0 : p.seq_len / bs;
+    const int rows_here = kTileM / bs;                       // block-rows of A' in this tile: 1, 2 or 4
+    const bool rank_here = kMode != kRowStats && p.row_ptr != nullptr;
+    const float inv_area = 1.f / (static_cast<float>(bs) * static_cast<float>(bs));
+    float m = -INFINITY;   // reference of this row in this group (base-2 logits)
+    float l = 0.f;         // sum of 2^(s - m)
+    float carry = 0.f;     // 128-key blocks: sum over the block's first 64 keys
+    if constexpr (kMode == kPooled) {
+      // natural-log LSE -> base-2 reference: 2^(s - m) is the probability
+      m = row_valid ? p.lse[static_cast<int64_t>(bh) * p.seq_len + row] * 1.44269504088896341f : INFINITY;
     }
-    float m_run = -INFINITY, l_run = 0.f;
-    const int nb = p.seq_len / p.block_size;
-    const bool half_blocks = (p.block_size == 64);
-    const float inv_area = 1.f / (static_cast<float>(p.block_size) * static_cast<float>(p.block_size));
-    const bool fuse_topk = (!kStatsOnly) && (p.row_ptr != nullptr);
-    bool ok = true;
-    for (int it = 0; it < num_tiles; ++it) {
-      const int buf = it & 1;
-      if (!mbar_wait(&sm.s_full[buf], (it >> 1) & 1, &sm.abort_flag, p.status, 60)) {
-        ok = false;
-        break;
-      }
+
+    // Block sums held in tensor memory (columns of key blocks [jb0, jb0 + n)) times the row's weight in the group that
+    // summed them, then summed over the rows of each query block: A' to memory and / or to the ranking keys. All eight
+    // warps, in step.
+    auto fold = [&](int jb0, int n, float w0, float w1) {
+      asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+      tc_fence_before();
+      named_barrier_sync(1, 2 * kTileM);
       tc_fence_after();
-      const uint32_t tS = tmem + buf * kTile + lane_base;
-      const int valid_cols = min(kTile, p.seq_len - it * kTile);
-      if constexpr (kStatsOnly) {
-        float mx = -INFINITY;
+      for (int c = 32 * g; c < n; c += 64) {
+        uint32_t r[32];
+        float v[32];
+        tmem_ld32(t_stat + c, r);
+        tmem_wait_ld();
 #pragma unroll
-        for (int c = 0; c < kTile / 32; ++c) {
-          uint32_t r[32];
-          tmem_ld32(tS + c * 32, r);
-          tmem_wait_ld();
-#pragma unroll
-          for (int j = 0; j < 32; ++j)
-            if (c * 32 + j < valid_cols) mx = fmaxf(mx, __uint_as_float(r[j]));
+        for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]) * ((((c + j) * bs) & 128) != 0 ? w1 : w0);
+        sm.quarter[wq][c + lane] = warp_column_sums(v, lane);   // columns at and beyond n are not used below
+      }
+      tc_fence_before();
+      named_barrier_sync(1, 2 * kTileM);
+      tc_fence_after();
+      if (tid < n) {
+        const float q0 = sm.quarter[0][tid], q1 = sm.quarter[1][tid], q2 = sm.quarter[2][tid], q3 = sm.quarter[3][tid];
+        float score[4] = {q0, q1, q2, q3};
+        if (bs == 128) score[0] = (q0 + q1) + (q2 + q3);
+        if (bs == 64) {
+          score[0] = q0 + q1;
+          score[1] = q2 + q3;
         }
-        const float m_new = fmaxf(m_run, mx * scale_log2);
-        float sum = 0.f;
+        const int jb = jb0 + tid;
 #pragma unroll
-        for (int c = 0; c < kTile / 32; ++c) {
-          uint32_t r[32];
-          tmem_ld32(tS + c * 32, r);
-          tmem_wait_ld();
-#pragma unroll
-          for (int j = 0; j < 32; ++j) {
-            const float e = fast_exp2(fmaf(__uint_as_float(r[j]), scale_log2, -m_new));
-            sum += (c * 32 + j < valid_cols) ? e : 0.f;
+        for (int rh = 0; rh < 4; ++rh) {
+          const int ib = q_tile * rows_here + rh;
+          if (rh < rows_here && ib < nb) {
+            const float a = score[rh] * inv_area;
+            if (p.scores != nullptr) p.scores[(static_cast<int64_t>(bh) * nb + ib) * nb + jb] = a;
+            if (rank_here) sm.keys[rh * nb + jb] = ordered_key(a);
           }
         }
-        l_run = l_run * fast_exp2(m_run - m_new) + sum;
-        m_run = m_new;
-        tc_fence_before();
-        mbar_arrive(&sm.s_empty[buf]);
-      } else {
-        float half_sum[2] = {0.f, 0.f};
-        float quarter[4];
+      }
+    };
+
+    bool ok = true;
+    int jb0 = 0;   // key block of column 0
+    const int my_tiles = g == 0 ? tiles0 : tiles1;
+    for (int j = 0; j < my_tiles; ++j) {
+      const int i = index_of(g, j);
+      const int t = tile_of(g, j);
+      // (after a wait has run out the remaining tiles are walked without waiting, so that all eight warps still meet in
+      // the same barriers; what they hold is not ranked)
+      ok = ok && mbar_wait(&sm.done[i % kSlots], (i / kSlots) & 1, &sm.abort_flag, p.status, 60);
+      ok = __all_sync(0xffffffffu, ok);
+      tc_fence_after();
+      uint32_t r0[32], r1[32];
+      const uint32_t tS = tmem + g * kTileN + lane_base;
+      tmem_ld32(tS, r0);
+      tmem_ld32(tS + 32, r1);
+      tmem_wait_ld();
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&sm.s_free[g]);
+      const int valid_cols = p.seq_len - t * kTileN;   // ragged tail of the sequence
+      if (valid_cols < kTileN) mask_columns_from(r0, r1, valid_cols);
+      float s0 = exp_sum(r0, scale_log2, m);
+      float s1 = exp_sum(r1, scale_log2, m);
+      if constexpr (kMode != kPooled) {
+        const bool outgrown = !(s0 + s1 <= kOutgrown);   // the row's first tile (m = -inf), far larger logits, or NaN
+        if (__any_sync(0xffffffffu, outgrown)) {
+          // take the tile's own maximum as the reference and bring everything summed so far to it
+          float mx = -INFINITY;
 #pragma unroll
-        for (int c = 0; c < kTile / 32; ++c) {
-          uint32_t r[32];
-          tmem_ld32(tS + c * 32, r);
-          tmem_wait_ld();
-          float acc = 0.f;
-#pragma unroll
-          for (int j = 0; j < 32; ++j)
-            acc += fast_exp2(fmaf(__uint_as_float(r[j]), scale_log2, -lse2));
-          half_sum[c >> 1] += acc;
-          quarter[c] = acc;
-        }
-        if (p.block_size == 32) {
-          // 32-key blocks: a warp's 32 rows are one query block and each 32-column chunk one key
-          // block, so every warp finishes its own four scores (scores always go to memory here)
-          tc_fence_before();
-          mbar_arrive(&sm.s_empty[buf]);
-#pragma unroll
-          for (int c = 0; c < 4; ++c) {
-#pragma unroll
-            for (int off = 16; off > 0; off >>= 1) quarter[c] += __shfl_xor_sync(0xffffffffu, quarter[c], off);
+          for (int c = 0; c < 32; ++c) mx = fmaxf(mx, fmaxf(__uint_as_float(r0[c]), __uint_as_float(r1[c])));
+          const float m_new = outgrown ? fmaxf(m, mx * scale_log2) : m;
+          const float alpha = m_new > m ? fast_exp2(m - m_new) : 1.f;
+          m = m_new;
+          l *= alpha;
+          // a row whose logits so far are all -inf: 2^(-inf - 0) = 0, not NaN
+          const float ref = m == -INFINITY ? 0.f : m;
+          s0 = exp_sum(r0, scale_log2, ref);
+          s1 = exp_sum(r1, scale_log2, ref);
+          if constexpr (kMode == kOnePass) {
+            carry *= alpha;
+            // (columns of the other group are left alone; its threads rescale theirs)
+            asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+            for (int s = g; s <= (t >> 1); s += 2) rescale_block_sums(t_stat + (s * 128) / bs, 128 / bs, alpha);
           }
-          const int ib = q_tile * 4 + warp;
-          if (lane < 4 && ib < nb) {
-            const int jb = it * 4 + lane;
-            const float total = lane == 0 ? quarter[0] : (lane == 1 ? quarter[1] : (lane == 2 ? quarter[2] : quarter[3]));
-            if (jb < nb) p.scores[(static_cast<int64_t>(bh) * nb + ib) * nb + jb] = total * inv_area;
-          }
-          continue;
         }
-        tc_fence_before();
-        mbar_arrive(&sm.s_empty[buf]);
-        // reduce over the 32 rows of this warp (fixed butterfly order)
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) {
-          half_sum[0] += __shfl_xor_sync(0xffffffffu, half_sum[0], off);
-          half_sum[1] += __shfl_xor_sync(0xffffffffu, half_sum[1], off);
-        }
-        // Per-warp partial sums go through a 4-deep ring in shared memory; the S buffers keep
-        // every warp within two tiles of the others, so a slot is never rewritten while read.
-        const int slot = it & 3;
-        if (lane == 0) {
-          sm.partial[slot][warp][0] = half_sum[0];
-          sm.partial[slot][warp][1] = half_sum[1];
-          mbar_arrive(&sm.partial_full[slot]);
-        }
-        if (warp == 0 && lane < 4) {
-          if (!mbar_wait(&sm.partial_full[slot], (it >> 2) & 1, &sm.abort_flag, p.status, 61)) {
-            ok = false;
-          } else if (!half_blocks) {
-            if (lane == 0) {
-              const float* pp = &sm.partial[slot][0][0];
-              const float total = ((pp[0] + pp[1]) + (pp[2] + pp[3])) + ((pp[4] + pp[5]) + (pp[6] + pp[7]));
-              const float score = total * inv_area;
-              if (p.scores != nullptr) p.scores[(static_cast<int64_t>(bh) * nb + q_tile) * nb + it] = score;
-              if (fuse_topk) sm.keys[0][it] = ordered_key(score);
-            }
+        l += s0 + s1;
+      }
+      if constexpr (kMode != kRowStats) {
+        const int col = (t * kTileN) / bs - jb0;   // first block of the tile
+        if (bs == 128) {
+          if ((t & 1) == 0) {
+            carry = s0 + s1;
           } else {
-            const int rh = lane >> 1, ch = lane & 1;  // row half (warps 2rh, 2rh+1), column half
-            const int ib = q_tile * 2 + rh, jb = it * 2 + ch;
-            if (ib < nb && jb < nb) {
-              const float total = sm.partial[slot][2 * rh][ch] + sm.partial[slot][2 * rh + 1][ch];
-              const float score = total * inv_area;
-              if (p.scores != nullptr) p.scores[(static_cast<int64_t>(bh) * nb + ib) * nb + jb] = score;
-              if (fuse_topk) sm.keys[rh][jb] = ordered_key(score);
-            }
+            tmem_st1(t_stat + col, carry + (s0 + s1));
+          }
+        } else if (bs == 64) {
+          tmem_st1(t_stat + col, s0 + s1);
+        } else {
+          tmem_st1(t_stat + col, s0);
+          tmem_st1(t_stat + col + 1, s1);   // (beyond the last block if their number is odd: not folded)
+        }
+        if constexpr (kMode == kPooled) {
+          // 128 blocks are bs spans of 128 keys: bs / 2 spans, bs tiles of each group
+          if ((j + 1) % bs == 0) {
+            fold(jb0, min(kChunk, nb - jb0), 1.f, 1.f);
+            jb0 += kChunk;
           }
         }
-        __syncwarp();
       }
     }
-    if constexpr (!kStatsOnly) {
-      if (fuse_topk && warp == 0) {
-        // warp 0 wrote every key of this CTA's block-row(s); rank them now (Eq. 5 / Eq. 6)
-        const bool all_ok = __all_sync(0xffffffffu, ok);
-        __syncwarp();
-        if (all_ok) {
+    if (*reinterpret_cast<volatile int*>(&sm.abort_flag) != 0) ok = false;
+    // the two groups' references and denominators of a row meet
+    float w0 = 1.f, w1 = 1.f;
+    if constexpr (kMode != kPooled) {
+      sm.ml[g][rit] = make_float2(m, l);
+      named_barrier_sync(1, 2 * kTileM);
+      const float2 a = sm.ml[0][rit], b = sm.ml[1][rit];
+      const float top = fmaxf(a.x, b.x);
+      const float f0 = fast_exp2(a.x - top), f1 = fast_exp2(b.x - top);
+      const float denom = a.y * f0 + b.y * f1;
+      if constexpr (kMode == kRowStats) {
+        if (ok && g == 0 && row_valid)
+          p.lse_out[static_cast<int64_t>(bh) * p.seq_len + row] = (top + log2f(denom)) * 0.69314718055994531f;
+      }
+      w0 = row_valid ? f0 / denom : 0.f;
+      w1 = row_valid ? f1 / denom : 0.f;
+    }
+    if constexpr (kMode != kRowStats) {
+      if (nb > jb0) fold(jb0, min(kChunk, nb - jb0), w0, w1);
+      named_barrier_sync(1, 2 * kTileM);   // the ranking keys are complete
+      if (ok && rank_here && warp < rows_here) {
+        // one warp per block-row: isolated top-k (Eq. 5 / Eq. 6) and the CSR list
+        const int ib = q_tile * rows_here + warp;
+        if (ib < nb) {
           const int k_total = p.k_pre + p.k_gen;
-          const int rows_here = half_blocks ? 2 : 1;
-          for (int rh = 0; rh < rows_here; ++rh) {
-            const int ib = half_blocks ? q_tile * 2 + rh : q_tile;
-            if (ib >= nb) break;
-            const int64_t row = static_cast<int64_t>(bh) * nb + ib;
-            warp_select_row(sm.keys[rh], nb, p.pb, p.k_pre, p.k_gen, sm.hist, p.col_idx + row * k_total, lane);
-            if (lane == 0) {
-              p.row_ptr[row] = static_cast<int32_t>(row * k_total);
-              if (row == static_cast<int64_t>(gridDim.x / num_q_tiles) * nb - 1)
-                p.row_ptr[row + 1] = static_cast<int32_t>((row + 1) * k_total);
-            }
-            __syncwarp();
+          const int64_t r = static_cast<int64_t>(bh) * nb + ib;
+          warp_select_row(sm.keys + warp * nb, nb, p.pb, p.k_pre, p.k_gen, sm.hist[warp], p.col_idx + r * k_total, lane);
+          if (lane == 0) {
+            p.row_ptr[r] = static_cast<int32_t>(r * k_total);
+            if (r == static_cast<int64_t>(gridDim.x / num_q_tiles) * nb - 1)
+              p.row_ptr[r + 1] = static_cast<int32_t>((r + 1) * k_total);
           }
         }
       }
-    }
-    if constexpr (kStatsOnly) {
-      if (ok && row_valid) lse_out[static_cast<int64_t>(bh) * p.seq_len + row] = (m_run + log2f(l_run)) * 0.69314718055994531f;
     }
   }
 
   tc_fence_before();
   __syncthreads();
-  if (warp == 5) {
+  if (warp == 9) {
     __syncwarp();
     tmem_dealloc(tmem, kTmemCols);
   }
 }
 
-template <bool kStatsOnly>
-cudaError_t launch(const CUtensorMap& tq, const CUtensorMap& tk, const ScoreParams& p, float* lse_out, int batch,
-                   cudaStream_t stream) {
-  auto kernel = score_kernel<kStatsOnly>;
+template <int kMode>
+cudaError_t launch(const CUtensorMap& tq, const CUtensorMap& tk, const ScoreParams& p, int batch, cudaStream_t stream) {
+  auto kernel = score_kernel<kMode>;
   const int smem = static_cast<int>(sizeof(ScoreSmem));
+  static_assert(sizeof(ScoreSmem) <= 113 * 1024, "two CTAs per SM");
   static SmemLimit limit;  // per template instantiation
   cudaError_t e = ensure_dynamic_smem(kernel, smem, limit);
   if (e != cudaSuccess) return e;
-  const int num_q_tiles = (p.seq_len + kTile - 1) / kTile;
+  const int num_q_tiles = (p.seq_len + kTileM - 1) / kTileM;
   const long long ctas = static_cast<long long>(batch) * p.heads_q * num_q_tiles;
   if (ctas <= 0) return cudaSuccess;
-  kernel<<<static_cast<unsigned>(ctas), kThreads, smem, stream>>>(tq, tk, p, lse_out);
+  kernel<<<static_cast<unsigned>(ctas), kThreads, smem, stream>>>(tq, tk, p);
   return cudaGetLastError();
 }
 
 }  // namespace
 
-cudaError_t launch_row_stats(const CUtensorMap& tq, const CUtensorMap& tk, const ScoreParams& p, float* lse_out,
-                             int batch, cudaStream_t stream) {
-  return launch<true>(tq, tk, p, lse_out, batch, stream);
+bool score_ranks_in_kernel(int nb, int block_size) { return nb * (kTileM / block_size) <= kMaxKeys; }
+bool score_in_one_pass(int nb) { return nb <= kChunk; }
+
+cudaError_t launch_row_stats(const CUtensorMap& tq, const CUtensorMap& tk, const ScoreParams& p, int batch,
+                             cudaStream_t stream) {
+  return launch<kRowStats>(tq, tk, p, batch, stream);
 }
 
 cudaError_t launch_pooled_scores(const CUtensorMap& tq, const CUtensorMap& tk, const ScoreParams& p, int batch,
                                  cudaStream_t stream) {
-  return launch<false>(tq, tk, p, nullptr, batch, stream);
+  return p.lse == nullptr ? launch<kOnePass>(tq, tk, p, batch, stream) : launch<kPooled>(tq, tk, p, batch, stream);
 }
 
 }  // namespace sparsed
