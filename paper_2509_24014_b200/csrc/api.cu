@@ -400,14 +400,14 @@ static sparsed_status attn_full_impl(const sparsed_shape* shape, const void* q, 
   p.num_q_tiles = (shape->seq_len + 127) / 128;
   p.num_blocks = 0;
   p.num_items = shape->batch * shape->heads_q * p.num_q_tiles;
-  p.max_ctas = 0;   // dense: one CTA per query tile (running on into further tiles measured 1-2 % slower here)
+  p.max_ctas = 0;
   p.scale_log2 = rs.scale_log2;
   p.row_ptr = nullptr;
   p.col_idx = nullptr;
   p.col_capacity = 0;
   p.status = static_cast<DeviceStatus*>(ws);
   cudaError_t e = pair ? launch_attn_dense_pair(tq, tk, tv, to, p, static_cast<cudaStream_t>(cuda_stream))
-                      : launch_attn_dense(tq, tk, tv, to, p, shape->batch, static_cast<cudaStream_t>(cuda_stream));
+                      : launch_attn_dense(tq, tk, tv, to, p, static_cast<cudaStream_t>(cuda_stream));
   return e == cudaSuccess ? SPARSED_OK : cuda_fail(e);
 }
 
@@ -557,7 +557,7 @@ sparsed_status sparsed_attn_sparse(const sparsed_shape* shape, const sparsed_pat
   p.num_q_tiles = (shape->seq_len + 127) / 128;
   p.num_blocks = pattern->num_blocks;
   p.num_items = shape->batch * shape->heads_q * p.num_q_tiles;
-  // block lists: as many CTAs as are resident at once, each running through its share of the query tiles, so
+  // 128-key blocks: as many CTAs as are resident at once, each running through its share of the query tiles, so
   // that only a CTA's first tile pays the start-up chain (+16 % at 4 blocks per row, +5 % at 14, +1 % at 52)
   p.max_ctas = attn_max_ctas();
   p.scale_log2 = rs.scale_log2;
@@ -565,7 +565,7 @@ sparsed_status sparsed_attn_sparse(const sparsed_shape* shape, const sparsed_pat
   p.col_idx = pattern->col_idx;
   p.col_capacity = pattern->col_capacity;
   p.status = static_cast<DeviceStatus*>(ws);
-  cudaError_t e = launch_attn_sparse(tq, tk, tv, to, p, shape->batch, bs, static_cast<cudaStream_t>(cuda_stream));
+  cudaError_t e = launch_attn_sparse(tq, tk, tv, to, p, bs, static_cast<cudaStream_t>(cuda_stream));
   return e == cudaSuccess ? SPARSED_OK : cuda_fail(e);
 }
 

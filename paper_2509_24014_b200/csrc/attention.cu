@@ -27,10 +27,9 @@
 //   * 128-key blocks: the 128 query rows are one query block; its CSR list is walked as it is,
 //     two tiles per block.
 //   * 64- and 32-key blocks: the 128 query rows are two / four consecutive query blocks with lists
-//     of their own. The CTA walks the UNION of those lists (built in shared memory at start-up as one
-//     bitmap per query block) and every warp masks, per 32-column chunk of a tile, the key blocks
-//     its own query block did not keep; a tile in which a warp keeps nothing costs it no
-//     exponentials. All 128 rows of every MMA belong to real queries, and neighbouring query blocks
+//     of their own. The CTA walks the UNION of those lists (built in shared memory by the producer warp, one
+//     item ahead, from one bitmap per query block) and every warp skips, per 32-column half of a tile, the key
+//     blocks its own query block did not keep: no copy out of tensor memory and no exponentials, P = 0. All 128 rows of every MMA belong to real queries, and neighbouring query blocks
 //     share the K/V tiles they have in common.
 #include "internal.h"
 #include "softmax_pipeline.cuh"
@@ -71,22 +70,29 @@ struct AttnSmem {
   uint64_t done[kSlots];   // the MMAs that read the slot have completed (Q K^T for a K tile, P V for a V tile)
   uint64_t p_full[2];
   uint64_t q_free;         // an output tile has been read out of the Q buffer (which staged it): the next Q may land
+  uint64_t o_staged;       // every softmax warp has written its rows of the output tile into the Q buffer
   uint32_t tmem_base;
   int abort_flag;
-  int n_union;                                             // packed: key blocks in the union list
-  uint32_t member[kGroups][kWords];                        // packed: bit j of query block g = "g keeps key block j"
-  uint16_t union_ids[kPacked ? kMaxPackedBlocks : 2];      // packed: the union, ascending
+  // Packed walks: the CTA's items, handed by the producer warp to the other roles through two buffers: the query tile
+  // (-1: no more) and the key blocks in the union of its lists ...
+  uint64_t item_full[2], item_free[2];
+  int item[2], item_entries[2];
+  alignas(16) uint32_t control[4];   // (the launch control's answer)
+  uint64_t control_full;
+  // ... and the union itself, ascending, one entry per key block: its id and, from bit kIdBits on, one bit per query block
+  // that keeps it. One per item buffer: the next item's union is built while this one's is walked.
+  alignas(16) uint16_t list[2][kPacked ? kMaxPackedBlocks + 2 : 2];
+  uint32_t member[kGroups][kWords];  // producer only: bit j of query block g = "g keeps key block j"
 };
+constexpr int kIdBits = 11;
+static_assert((1 << kIdBits) == kMaxPackedBlocks, "ids of union entries");
 
 // kDense: walk every key tile of the sequence (kBlock must be 128 then; no block lists are read).
-// kMultiItem: a CTA may be given several query tiles (launched with fewer CTAs than tiles); without it the
-// item loops below run once and their running counters fold to zero at compile time.
-template <int kBlock, bool kDense, bool kMultiItem>
+template <int kBlock, bool kDense>
 __global__ void __launch_bounds__(kThreads, 2)
 attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
             const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_o, const AttnParams p) {
   static_assert(!kDense || kBlock == 128, "the dense walk uses the unpacked layout");
-  static_assert(!kMultiItem || kBlock == 128, "the packed walk prepares its union once per CTA");
   using Smem = AttnSmem<kBlock>;
   constexpr bool kPacked = Smem::kPacked;
   constexpr int kSlots = Smem::kSlots;
@@ -106,20 +112,25 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
   const int lane = tid & 31;
 
   // ---- work items ----------------------------------------------------------------------
-  // An item is one 128-row query tile of one (batch, head). A CTA takes items blockIdx.x,
-  // blockIdx.x + gridDim.x, ... ; the host launches either one CTA per item or (dense and 128-key
-  // blocks only) as many CTAs as fit on the device at once, in which case each role of the pipeline
-  // runs on into its next item on its own: the producer loads the next Q, list and K/V tiles while
-  // the softmax warps are still in the previous item's last tiles and epilogue, so the start-up
-  // chain row_ptr -> col_idx -> first K tile -> first MMA of all but a CTA's first item is hidden.
-  // Every counter below (loads, tiles, Q loads) runs on across items and all roles compute the same
-  // values, so ring slots, S buffers and barrier phases simply continue.
+  // An item is one 128-row query tile of one (batch, head). Dense: one CTA per item, and that is all there is to it.
+  // Block lists: a CTA runs through several items, and each role of the pipeline runs on into the next one on its
+  // own: the producer loads the next Q, list and K/V tiles while the softmax warps are still in the previous item's
+  // last tiles and epilogue, so that the start-up chain row_ptr -> col_idx -> first K tile -> first MMA of all but a
+  // CTA's first item is hidden. Counters of loads, tiles and Q loads run on across items and all roles compute the same
+  // values, so ring slots, S buffers and barrier phases simply continue. Which items those are:
+  //   128-key blocks: blockIdx.x, blockIdx.x + gridDim.x, ...; as many CTAs as fit on the device. A selected
+  //     pattern's lists are equally long, so that is balanced.
+  //   64- and 32-key blocks: unions differ in length by up to 1 : 4, so the grid has one CTA per item and a CTA that
+  //     runs takes over CTAs that have not been launched yet (cluster launch control), one item ahead. Against equal
+  //     shares: 1450 -> 1390 us for 8 x 32 heads x 4096 tokens, block 32, half kept; 8.64 -> 8.06 ms for 32 x 65536,
+  //     block 64. (With 128-key blocks it was 1 % slower than equal shares.)
   struct Item {
     int q_tile, bh, head, batch, kv_head, q_row0, groups_here, r0;
     int list_begin, list_len;   // CSR entries of the item's query blocks; dense: key tiles of the sequence
   };
   const int n_items = p.num_items;
-  auto describe = [&](int item) -> Item {
+  // with_list: read the item's row_ptr entries too
+  auto describe = [&](int item, bool with_list) -> Item {
     Item it;
     it.q_tile = item % p.num_q_tiles;
     it.bh = item / p.num_q_tiles;
@@ -132,7 +143,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
     it.r0 = it.bh * p.num_blocks + qb0;                                    // CSR row of query block qb0
     it.list_begin = 0;
     it.list_len = (p.seq_len + kTileN - 1) / kTileN;
-    if constexpr (!kDense) {
+    if (!kDense && with_list) {
       // adjacent rows are adjacent in col_idx, so the item's lists are one run of entries
       it.list_begin = __ldg(p.row_ptr + it.r0);
       it.list_len = __ldg(p.row_ptr + it.r0 + it.groups_here) - it.list_begin;
@@ -150,7 +161,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
   auto unpacked_tiles = [&](const Item& it) -> int { return kDense ? it.list_len : it.list_len * kTilesPerBlock; };
 
   const int first_item = blockIdx.x;
-  Item cur = describe(first_item);
+  Item cur = describe(first_item, !kPacked || warp == 4);
 
   // ---- set-up --------------------------------------------------------------------------
   // The producer warp owns the barriers of its own loads, so it can start them before the CTA-wide
@@ -159,7 +170,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
   int list_ids = 0;     // unpacked walk: lane i holds the block id of list entry 32 * chunk + i
   int loads_issued = 0; // K/V loads of the first item already issued by the producer before the set-up barrier
   // rows [kv_row0, +64) (or two 32-row blocks at kv_row0 / kv_row1) of K (which = 0) or V into `slot`
-  auto issue_load = [&](const Item& it, int slot, int which, int kv_row0, int kv_row1, int blocks_here) {
+  auto issue_load = [&](const Item& it, int slot, int which, int kv_row0, int kv_row1) {
     if (elect_one_sync()) {
       const CUtensorMap* tm = which == 0 ? &tm_k : &tm_v;
       if constexpr (kBlocksPerTile == 1) {
@@ -168,13 +179,11 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
         tma_load_4d(sm.kv[slot][1], tm, &sm.kv_full[slot], 64, kv_row0, it.kv_head, it.batch);
       } else {
         // tensor-map boxes are 32 rows here; block b of the tile lands at rows 32 b
-        mbar_expect_tx(&sm.kv_full[slot], blocks_here * kBlock * kHeadDim * 2);
+        mbar_expect_tx(&sm.kv_full[slot], kTileN * kHeadDim * 2);
         tma_load_4d(sm.kv[slot][0], tm, &sm.kv_full[slot], 0, kv_row0, it.kv_head, it.batch);
         tma_load_4d(sm.kv[slot][1], tm, &sm.kv_full[slot], 64, kv_row0, it.kv_head, it.batch);
-        if (blocks_here == 2) {
-          tma_load_4d(sm.kv[slot][0] + kBlock * 64, tm, &sm.kv_full[slot], 0, kv_row1, it.kv_head, it.batch);
-          tma_load_4d(sm.kv[slot][1] + kBlock * 64, tm, &sm.kv_full[slot], 64, kv_row1, it.kv_head, it.batch);
-        }
+        tma_load_4d(sm.kv[slot][0] + kBlock * 64, tm, &sm.kv_full[slot], 0, kv_row1, it.kv_head, it.batch);
+        tma_load_4d(sm.kv[slot][1] + kBlock * 64, tm, &sm.kv_full[slot], 64, kv_row1, it.kv_head, it.batch);
       }
     }
     __syncwarp();
@@ -193,10 +202,85 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
     const int e = t / kTilesPerBlock;
     return __shfl_sync(0xffffffffu, list_ids, e & 31) * kBlock + (t % kTilesPerBlock) * kTileN;
   };
+  // Packed walks, producer warp: one bitmap per query block of the item, then their union into list buffer `buf`;
+  // returns its length. The last tile of an odd union of 32-key blocks is filled up with its own last block, which no
+  // query block keeps there.
+  auto build_union = [&](const Item& it, int buf) -> int {
+    const int words = (p.num_blocks + 31) >> 5;
+    for (int i = lane; i < kGroups * Smem::kWords; i += 32) (&sm.member[0][0])[i] = 0u;
+    int bound[kGroups];   // bound[g] = first CSR entry after query block g's list
+#pragma unroll
+    for (int g = 0; g < kGroups; ++g) bound[g] = __ldg(p.row_ptr + it.r0 + min(g + 1, it.groups_here));
+    __syncwarp();
+    const int list_end = it.list_begin + it.list_len;
+    for (int e0 = it.list_begin + lane; e0 < list_end; e0 += 8 * 32) {
+      int id[8];   // eight loads in flight per lane
+#pragma unroll
+      for (int u = 0; u < 8; ++u) id[u] = e0 + 32 * u < list_end ? __ldg(p.col_idx + e0 + 32 * u) : -1;
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        int g = 0;
+#pragma unroll
+        for (int j = 0; j + 1 < kGroups; ++j) g += (e0 + 32 * u >= bound[j]) ? 1 : 0;
+        if (id[u] >= 0 && id[u] < p.num_blocks) atomicOr(&sm.member[g][id[u] >> 5], 1u << (id[u] & 31));
+      }
+    }
+    __syncwarp();
+    uint16_t* list = sm.list[buf];
+    int n = 0;
+    for (int w = 0; w < words; ++w) {   // lane = bit of the word
+      uint32_t mask = 0u;
+#pragma unroll
+      for (int g = 0; g < kGroups; ++g) mask |= ((sm.member[g][w] >> lane) & 1u) << g;
+      const uint32_t any = __ballot_sync(0xffffffffu, mask != 0u);
+      if (mask != 0u)
+        list[n + __popc(any & ((1u << lane) - 1u))] = static_cast<uint16_t>((w * 32 + lane) | (mask << kIdBits));
+      n += __popc(any);
+    }
+    __syncwarp();
+    if (kBlocksPerTile > 1 && (n & 1) != 0 && lane == 0) list[n] = list[n - 1] & ((1u << kIdBits) - 1u);
+    return n;
+  };
+  // the CTA's next item (-1: none), `entries` key blocks long, to the other roles
+  auto publish = [&](int buf, int item, int entries) {
+    __syncwarp();
+    if (lane == 0) {
+      sm.item[buf] = item;
+      sm.item_entries[buf] = entries;
+      mbar_arrive(&sm.item_full[buf]);
+    }
+    __syncwarp();
+  };
+  // ask for the item after the one at hand
+  auto request_item = [&]() {
+    if (elect_one_sync()) {
+      mbar_expect_tx(&sm.control_full, 16);
+      launch_control_request(sm.control, &sm.control_full);
+    }
+    __syncwarp();
+  };
+  // first key rows of tile t of the union in list buffer `buf`: both 32-key blocks side by side, or one 64-key block
+  auto union_rows = [&](int buf, int t) -> int2 {
+    constexpr uint32_t ids = (1u << kIdBits) - 1u;
+    if constexpr (kBlocksPerTile == 1) {
+      return make_int2(static_cast<int>(sm.list[buf][t] & ids) * kBlock, 0);
+    } else {
+      const uint32_t two = *reinterpret_cast<const uint32_t*>(&sm.list[buf][2 * t]);
+      return make_int2(static_cast<int>(two & ids) * kBlock, static_cast<int>((two >> 16) & ids) * kBlock);
+    }
+  };
+  int first_entries = 0;   // packed, producer: entries of the first item's union
   if (warp == 4) {
     if (lane == 0) {
       mbar_init(&sm.q_full, 1);
       for (int s = 0; s < kSlots; ++s) mbar_init(&sm.kv_full[s], 1);
+      if constexpr (kPacked) {
+        for (int b = 0; b < 2; ++b) {
+          mbar_init(&sm.item_full[b], 1);
+          mbar_init(&sm.item_free[b], 5);   // four softmax warps and the issuer
+        }
+        mbar_init(&sm.control_full, 1);
+      }
       mbar_fence_init();
     }
     __syncwarp();
@@ -207,92 +291,45 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
       if constexpr (!kDense) tma_prefetch_desc(&tm_o);
     }
     __syncwarp();
-    if (cur.list_len > 0) {
-      issue_q_load(cur);
-      if constexpr (!kPacked) {
-        if constexpr (!kDense) {
-          if (lane < cur.list_len) list_ids = __ldg(p.col_idx + cur.list_begin + lane);
-        }
-        const int first = min(2 * unpacked_tiles(cur), kSlots);   // list entries 0..2 at most: within the first chunk
-        for (; loads_issued < first; ++loads_issued)
-          issue_load(cur, loads_issued, loads_issued & 1, unpacked_row(loads_issued >> 1), 0, 1);
+    if constexpr (kPacked) {
+      request_item();
+      first_entries = build_union(cur, 0);
+      publish(0, first_item, first_entries);
+      if (first_entries > 0) issue_q_load(cur);
+      const int first = min(2 * ((first_entries + kBlocksPerTile - 1) / kBlocksPerTile), kSlots);
+      for (; loads_issued < first; ++loads_issued) {
+        const int2 rows = union_rows(0, loads_issued >> 1);
+        issue_load(cur, loads_issued, loads_issued & 1, rows.x, rows.y);
       }
+    } else if (cur.list_len > 0) {
+      issue_q_load(cur);
+      if constexpr (!kDense) {
+        if (lane < cur.list_len) list_ids = __ldg(p.col_idx + cur.list_begin + lane);
+      }
+      const int first = min(2 * unpacked_tiles(cur), kSlots);   // list entries 0..2 at most: within the first chunk
+      for (; loads_issued < first; ++loads_issued)
+        issue_load(cur, loads_issued, loads_issued & 1, unpacked_row(loads_issued >> 1), 0);
     }
   }
   if (tid == 0) {
     for (int s = 0; s < kSlots; ++s) mbar_init(&sm.done[s], 1);
     for (int s = 0; s < 2; ++s) mbar_init(&sm.p_full[s], kSoftmaxThreads);
     mbar_init(&sm.q_free, 1);
+    mbar_init(&sm.o_staged, 4);
     sm.abort_flag = 0;
-    sm.n_union = 0;
     mbar_fence_init();
-  }
-  if constexpr (kBlocksPerTile > 1) {
-    // a tile may be half filled (odd union): its other half is multiplied by P = 0, so it has to
-    // hold finite numbers from the start
-    uint4* z = reinterpret_cast<uint4*>(&sm.kv[0][0][0]);
-    constexpr int n16 = kSlots * 2 * kTileN * 64 * 2 / 16;
-    for (int i = tid; i < n16; i += kThreads) z[i] = make_uint4(0, 0, 0, 0);
-    fence_proxy_async_smem();
   }
   if (warp == 5) {
     tmem_alloc(&sm.tmem_base, kTmemCols);
     tmem_relinquish();
-  }
-  if constexpr (kPacked) {
-    // (one item per CTA here) One bitmap per query block, then their union as an ascending list.
-    const int words = (p.num_blocks + 31) >> 5;
-    for (int i = tid; i < kGroups * Smem::kWords; i += kThreads) (&sm.member[0][0])[i] = 0u;
-    __syncthreads();
-    int bound[kGroups];   // bound[g] = first CSR entry after query block g's list
-#pragma unroll
-    for (int g = 0; g < kGroups; ++g) bound[g] = __ldg(p.row_ptr + cur.r0 + min(g + 1, cur.groups_here));
-    for (int e = cur.list_begin + tid; e < cur.list_begin + cur.list_len; e += kThreads) {
-      const int id = __ldg(p.col_idx + e);
-      int g = 0;
-#pragma unroll
-      for (int j = 0; j + 1 < kGroups; ++j) g += (e >= bound[j]) ? 1 : 0;
-      if (id >= 0 && id < p.num_blocks) atomicOr(&sm.member[g][id >> 5], 1u << (id & 31));
-    }
-    __syncthreads();
-    if (warp == 4) {
-      int base = 0;
-      for (int w0 = 0; w0 < words; w0 += 32) {
-        const int w = w0 + lane;
-        uint32_t bits = 0u;
-        if (w < words) {
-#pragma unroll
-          for (int g = 0; g < kGroups; ++g) bits |= sm.member[g][w];
-        }
-        const int cnt = __popc(bits);
-        int incl = cnt;
-#pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-          const int v = __shfl_up_sync(0xffffffffu, incl, off);
-          if (lane >= off) incl += v;
-        }
-        int pos = base + incl - cnt;
-        while (bits != 0u) {
-          const int b = __ffs(bits) - 1;
-          sm.union_ids[pos++] = static_cast<uint16_t>(w * 32 + b);
-          bits &= bits - 1u;
-        }
-        base += __shfl_sync(0xffffffffu, incl, 31);
-      }
-      if (lane == 0) sm.n_union = base;
-    }
   }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = sm.tmem_base;
   const uint32_t tO = tmem + kColO;
-  // key blocks an item walks (dense: key tiles) and its tiles
-  auto entries_of = [&](const Item& it) -> int { return kPacked ? sm.n_union : it.list_len; };
-  auto tiles_of = [&](const Item& it) -> int {
-    const int n = entries_of(it);
-    return kDense ? n : kBlocksPerTile == 1 ? n * kTilesPerBlock : (n + kBlocksPerTile - 1) / kBlocksPerTile;
-  };
+  // 64-key tiles of a union of n key blocks
+  auto union_tiles = [&](int n) -> int { return kBlocksPerTile == 1 ? n : (n + kBlocksPerTile - 1) / kBlocksPerTile; };
 
   // Warps 4 and 5 run their loops with all 32 lanes converged and let one elected lane issue
   // the TMA / UMMA instructions: their operands then stay on the uniform datapath.
@@ -302,7 +339,8 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
     bool ok = true;
     int load0 = 0;       // K/V loads issued for earlier items
     int q_tiles_done = 0;  // earlier items that had keys (each loaded a Q tile and staged an output tile)
-    for (int item = first_item; ok && item < n_items; item += gridDim.x) {
+    [[maybe_unused]] int requests = 0;   // answers of the launch control that have been followed by a request
+    for (int nth = 0; ok; ++nth) {       // the CTA's nth item; packed: in item buffer nth & 1
       // The Q buffer doubles as the staging tile of the previous output: the next Q may land once the softmax
       // warps have had that output read out of it (which is after the item's last MMA). The first ring-full of
       // the new item's K/V loads does not depend on its Q (their slots are freed by the previous item's MMAs),
@@ -310,10 +348,34 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
       // in this (no Q tile, zeros stored straight from registers), so the barrier completes exactly once per Q
       // tile and this warp is never more than one phase away from it.
       bool q_pending = false;
-      if (item != first_item) {
-        cur = describe(item);
-        q_pending = cur.list_len > 0;
-        if constexpr (!kPacked && !kDense) {
+      int n_entries = kPacked ? first_entries : cur.list_len;
+      if constexpr (kPacked) {
+        if (nth > 0) {
+          ok = mbar_wait(&sm.control_full, (nth - 1) & 1, &sm.abort_flag, p.status, 13);
+          // the softmax warps and the issuer have finished with the item that was in this buffer
+          if (nth >= 2) ok = ok && mbar_wait(&sm.item_free[nth & 1], ((nth >> 1) - 1) & 1, &sm.abort_flag, p.status, 12);
+          ok = __all_sync(0xffffffffu, ok);
+          if (!ok) break;
+          const int item = launch_control_answer(sm.control);
+          __syncwarp();
+          if (item < 0) {
+            publish(nth & 1, -1, 0);
+            break;
+          }
+          request_item();
+          ++requests;
+          cur = describe(item, true);
+          n_entries = build_union(cur, nth & 1);
+          publish(nth & 1, item, n_entries);
+          q_pending = n_entries > 0;
+        }
+      } else if constexpr (!kDense) {
+        if (nth > 0) {
+          const int item = first_item + nth * static_cast<int>(gridDim.x);
+          if (item >= n_items) break;
+          cur = describe(item, true);
+          n_entries = cur.list_len;
+          q_pending = n_entries > 0;
           list_ids = (lane < cur.list_len) ? __ldg(p.col_idx + cur.list_begin + lane) : 0;
         }
       }
@@ -327,17 +389,16 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
         q_pending = false;
         return got;
       };
-      const int n_entries = entries_of(cur);
-      const int num_tiles = tiles_of(cur);
+      const int num_tiles = kPacked ? union_tiles(n_entries) : unpacked_tiles(cur);
       const int q_at = min(2 * num_tiles, kSlots);
       // load i: K (even) or V (odd) of tile i / 2; a slot is reused every kSlots loads
-      for (int i = (item == first_item ? loads_issued : 0); ok && i < 2 * num_tiles; ++i) {
+      for (int i = (nth == 0 ? loads_issued : 0); ok && i < 2 * num_tiles; ++i) {
         if (q_pending && i == q_at && !settle_q()) {
           ok = false;
           break;
         }
         const int t = i >> 1;
-        int kv_row0, kv_row1 = 0, blocks_here = 1;
+        int kv_row0, kv_row1 = 0;
         if constexpr (!kPacked) {
           if constexpr (!kDense) {
             // block ids are fetched 32 at a time, one per lane, when the walk enters a new chunk
@@ -347,13 +408,9 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
           }
           kv_row0 = unpacked_row(t);
         } else {
-          const int e = kBlocksPerTile * t;
-          kv_row0 = static_cast<int>(sm.union_ids[e]) * kBlock;
-          if (kBlocksPerTile > 1 && e + 1 < n_entries) {
-            // two 32-key blocks side by side in one 64-key tile; an odd union leaves the last tile half filled
-            kv_row1 = static_cast<int>(sm.union_ids[e + 1]) * kBlock;
-            blocks_here = 2;
-          }
+          const int2 rows = union_rows(nth & 1, t);
+          kv_row0 = rows.x;
+          kv_row1 = rows.y;
         }
         const int g = load0 + i;
         const int slot = g % kSlots;
@@ -363,13 +420,18 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
           ok = __all_sync(0xffffffffu, ok);
           if (!ok) break;
         }
-        issue_load(cur, slot, i & 1, kv_row0, kv_row1, blocks_here);
+        issue_load(cur, slot, i & 1, kv_row0, kv_row1);
         TL(22);
       }
       if (ok && q_pending) ok = settle_q();
-      if constexpr (!kMultiItem) break;
+      if constexpr (kDense) break;
       load0 += 2 * num_tiles;
       if (num_tiles > 0) ++q_tiles_done;
+    }
+    if constexpr (kPacked) {
+      // given up: the launch control's answer must not arrive after the CTA has left (bounded like every wait)
+      for (uint32_t i = 0; !ok && i < kSpinLimit; ++i)
+        if (mbar_try_wait(&sm.control_full, requests & 1)) break;
     }
   } else if (warp == 5) {
     // =============================== UMMA issuer ========================================
@@ -381,13 +443,28 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
     TL_DECL(1)
     bool ok = true;
     int load0 = 0, tile0 = 0, q_loads = 0;   // loads / tiles / Q tiles of earlier items
-    for (int item = first_item; ok && item < n_items; item += gridDim.x) {
-      if (item != first_item) cur = describe(item);
-      const int num_tiles = tiles_of(cur);
-      if (num_tiles == 0) {
-        if constexpr (!kMultiItem) break;
-        continue;
+    for (int nth = 0; ok; ++nth) {
+      int num_tiles;
+      if constexpr (kPacked) {
+        // (the buffer is handed back at once: the issuer needs nothing but the number of tiles)
+        const int buf = nth & 1;
+        ok = mbar_wait(&sm.item_full[buf], (nth >> 1) & 1, &sm.abort_flag, p.status, 23);
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) break;
+        const int item = sm.item[buf];
+        num_tiles = union_tiles(sm.item_entries[buf]);
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&sm.item_free[buf]);
+        if (item < 0) break;
+      } else {
+        if (!kDense && nth > 0) {
+          const int item = first_item + nth * static_cast<int>(gridDim.x);
+          if (item >= n_items) break;
+          cur = describe(item, true);
+        }
+        num_tiles = unpacked_tiles(cur);
       }
+      if (!kDense && num_tiles == 0) continue;
       // S_t = Q K_t^T into S buffer (tile0 + t) & 1
       auto issue_qk = [&](int t) -> bool {
         const int g = load0 + 2 * t;
@@ -426,7 +503,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
         issue_pv64(tO, tmem + kColS + (gt & 1) * kTileN, v_lo0 + slot * slot_step, t > 0, &sm.done[slot]);
         TL(15);
       }
-      if constexpr (!kMultiItem) break;
+      if constexpr (kDense) break;
       load0 += 2 * num_tiles;
       tile0 += num_tiles;
     }
@@ -439,15 +516,28 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
     bool ok = true;
     TL_DECL(0)
     int load0 = 0, tile0 = 0;   // loads / tiles of earlier items
-    [[maybe_unused]] Item nxt = cur;   // multi-item: the next item's row_ptr entries are fetched one item ahead
-    for (int item = first_item; ok && item < n_items; item += gridDim.x) {
-      if constexpr (kMultiItem) {
-        cur = nxt;
-        if (item + static_cast<int>(gridDim.x) < n_items) nxt = describe(item + gridDim.x);
+    [[maybe_unused]] uint32_t out_phase = 0;   // output tiles staged so far, modulo 2
+    [[maybe_unused]] Item nxt = cur;   // 128-key blocks: the next item's row_ptr entries are fetched one item ahead
+    for (int nth = 0; ok; ++nth) {
+      int num_tiles;
+      if constexpr (kPacked) {
+        ok = mbar_wait(&sm.item_full[nth & 1], (nth >> 1) & 1, &sm.abort_flag, p.status, 33);
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) break;
+        const int item = sm.item[nth & 1];
+        if (item < 0) break;
+        num_tiles = union_tiles(sm.item_entries[nth & 1]);
+        cur = describe(item, false);
+      } else {
+        if constexpr (!kDense) {
+          const int item = first_item + nth * static_cast<int>(gridDim.x);
+          if (item >= n_items) break;
+          cur = nxt;
+          if (item + static_cast<int>(gridDim.x) < n_items) nxt = describe(item + static_cast<int>(gridDim.x), true);
+        }
+        num_tiles = unpacked_tiles(cur);
       }
-      const int n_entries = entries_of(cur);
-      const int num_tiles = tiles_of(cur);
-      const bool group_valid = my_group < cur.groups_here;
+      [[maybe_unused]] const uint16_t* list = sm.list[nth & 1];
       RowState st{-INFINITY, 0.f};
       // One 64-key tile of the softmax.
       auto tile_body = [&](int t) -> bool {
@@ -459,27 +549,28 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
         tc_fence_after();
         const int buf = (tile0 + t) & 1;   // S buffer of the tile
         const uint32_t tS = tmem + kColS + buf * kTileN + lane_base;
-        // packed walk: which 32-column chunks of this tile hold key blocks this warp's query block kept
-        bool keep0 = true, keep1 = true;
-        if constexpr (kPacked) {
-          const int e = kBlocksPerTile * t;
-          const int id0 = sm.union_ids[e];
-          keep0 = group_valid && ((sm.member[my_group][id0 >> 5] >> (id0 & 31)) & 1u) != 0u;
-          if constexpr (kBlocksPerTile == 1) {
-            keep1 = keep0;
-          } else {
-            keep1 = false;
-            if (e + 1 < n_entries) {
-              const int id1 = sm.union_ids[e + 1];
-              keep1 = group_valid && ((sm.member[my_group][id1 >> 5] >> (id1 & 31)) & 1u) != 0u;
-            }
-          }
-        }
         uint32_t pk[32];
-        if (kPacked && !keep0 && !keep1) {
-          // nothing of this tile is kept by this warp's query block: P = 0, no exponentials
-#pragma unroll
-          for (int j = 0; j < 32; ++j) pk[j] = 0u;
+        if constexpr (kPacked) {
+          // which 32-column halves of this tile hold key blocks that this warp's query block keeps
+          bool keep0, keep1;
+          if constexpr (kBlocksPerTile == 1) {
+            keep0 = keep1 = ((list[t] >> (kIdBits + my_group)) & 1u) != 0u;
+          } else {
+            const uint32_t two = *reinterpret_cast<const uint32_t*>(list + 2 * t);
+            keep0 = ((two >> (kIdBits + my_group)) & 1u) != 0u;
+            keep1 = ((two >> (16 + kIdBits + my_group)) & 1u) != 0u;
+          }
+          if (!packed_softmax_tile<kBlocksPerTile>(tS, keep0, keep1, scale_log2, st, pk, [&](float alpha) -> bool {
+                if (t == 0) return true;
+                // O must be quiescent: wait until P_{t-1} V_{t-1} (which read ring load 2t-1) has drained
+                const int gp = load0 + 2 * (t - 1) + 1;
+                if (!mbar_wait(&sm.done[gp % kSlots], (gp / kSlots) & 1, &sm.abort_flag, p.status, 32)) return false;
+                tc_fence_after();
+                rescale_accumulator_row(tO + lane_base, alpha);
+                if (p.slow_path_events != nullptr && lane == 0) atomicAdd(p.slow_path_events, 1ull);
+                return true;
+              }))
+            return false;
         } else {
           uint32_t r0[32], r1[32];
           tmem_ld32(tS, r0);
@@ -489,16 +580,6 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
           if constexpr (kDense) {
             const int valid_cols = p.seq_len - t * kTileN;   // ragged tail of the sequence
             if (valid_cols < kTileN) mask_columns_from(r0, r1, valid_cols);
-          }
-          if constexpr (kPacked) {
-            if (!keep0) {
-#pragma unroll
-              for (int j = 0; j < 32; ++j) r0[j] = 0xff800000u;   // -inf
-            }
-            if (!keep1) {
-#pragma unroll
-              for (int j = 0; j < 32; ++j) r1[j] = 0xff800000u;
-            }
           }
           float2 sums;
           bool exact = (st.m == -INFINITY);   // nothing accumulated yet: no reference maximum to try
@@ -528,6 +609,10 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
         return true;
       };
       for (int t = 0; ok && t < num_tiles; ++t) ok = tile_body(t);
+      if constexpr (kPacked) {
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&sm.item_free[nth & 1]);
+      }
       if constexpr (kDense) {
         // ---- epilogue of the dense walk: O / l -> bf16 -> global, each row from its own thread ----------
         // (with the staged epilogue of the other walks its main loop compiled 1-2 % slower, measured, and its
@@ -548,12 +633,12 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
           p.lse[static_cast<int64_t>(cur.bh) * p.seq_len + row] = (st.m + log2f(st.l)) * 0.69314718055994531f;
       } else {
         // ---- epilogue: O / l -> bf16 -> shared memory -> global (an empty list gives zeros) ----------
-        // Every thread goes through the barrier below even after a wait has run out (it then stages zeros), so
-        // that none is left waiting there; what is done after it is decided by the shared flag.
         if (ok && num_tiles > 0) {
           const int gl = load0 + 2 * (num_tiles - 1) + 1;   // the last P V read this load's slot
           ok = mbar_wait(&sm.done[gl % kSlots], (gl / kSlots) & 1, &sm.abort_flag, p.status, 31);
         }
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) break;
         tc_fence_after();
         const float inv_l = st.l > 0.f ? (1.f / st.l) : 0.f;
         if (num_tiles == 0) {
@@ -564,20 +649,27 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
           store_output_row(0u, false, 0.f, o_row, row < p.seq_len);
         } else {
           // The Q tile is dead (the item's last Q K^T completed before its last P V did): it stages the output.
-          stage_output_row(tO + lane_base, ok, inv_l, &sm.q[0][0], tid);
-          named_barrier_sync(1, kSoftmaxThreads);
-          if (*reinterpret_cast<volatile int*>(&sm.abort_flag) != 0) break;
+          // The first warp waits for the others' rows and sends the tile off; the others run on.
+          stage_output_row(tO + lane_base, true, inv_l, &sm.q[0][0], tid);
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&sm.o_staged);
+          if (warp == 0) {
+            ok = mbar_wait(&sm.o_staged, out_phase, &sm.abort_flag, p.status, 34);
+            ok = __all_sync(0xffffffffu, ok);
+            if (!ok) break;
+          }
+          out_phase ^= 1u;
           if (tid == 0) {
             // rows beyond the sequence end are clipped by the tensor map
             tma_store_4d(&tm_o, sm.q[0], 0, cur.q_row0, cur.head, cur.batch);
             tma_store_4d(&tm_o, sm.q[1], 64, cur.q_row0, cur.head, cur.batch);
             tma_store_commit();
             tma_store_wait_read();
-            if constexpr (kMultiItem) mbar_arrive(&sm.q_free);
+            mbar_arrive(&sm.q_free);
           }
         }
       }
-      if constexpr (!kMultiItem) break;
+      if constexpr (kDense) break;
       tc_fence_before();   // the next item's first P V overwrites O: order these reads before its hand-over
       load0 += 2 * num_tiles;
       tile0 += num_tiles;
@@ -593,19 +685,19 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
   }
 }
 
-template <int kBlock, bool kDense, bool kMultiItem>
+template <int kBlock, bool kDense>
 cudaError_t launch(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap& to,
-                   const AttnParams& p, int batch, cudaStream_t stream) {
-  auto kernel = attn_kernel<kBlock, kDense, kMultiItem>;
+                   const AttnParams& p, cudaStream_t stream) {
+  auto kernel = attn_kernel<kBlock, kDense>;
   const int smem = static_cast<int>(sizeof(AttnSmem<kBlock>));
+  static_assert(sizeof(AttnSmem<kBlock>) <= 113 * 1024, "two CTAs per SM");
   static SmemLimit limit;  // per template instantiation
   cudaError_t e = ensure_dynamic_smem(kernel, smem, limit);
   if (e != cudaSuccess) return e;
-  // one CTA per item, or (kMultiItem and p.max_ctas > 0) at most that many CTAs, each running through its
-  // share of the items
   long long ctas = p.num_items;
   if (ctas <= 0) return cudaSuccess;
-  if (kMultiItem && p.max_ctas > 0 && ctas > p.max_ctas) ctas = p.max_ctas;
+  // 128-key blocks: at most as many CTAs as are resident at once, each with its share of the items
+  if (kBlock == 128 && !kDense && p.max_ctas > 0 && ctas > p.max_ctas) ctas = p.max_ctas;
   kernel<<<static_cast<unsigned>(ctas), kThreads, smem, stream>>>(tq, tk, tv, to, p);
   return cudaGetLastError();
 }
@@ -617,17 +709,16 @@ int attn_sparse_max_blocks(int block_size) { return block_size < kTileM ? kMaxPa
 // Tensor maps: Q and O boxes 64 x 128 rows, K and V boxes 64 x min(64, block_size) rows.
 // p.num_q_tiles = ceil(seq_len / 128), p.num_blocks = seq_len / block_size.
 cudaError_t launch_attn_sparse(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv,
-                               const CUtensorMap& to, const AttnParams& p, int batch, int block_size,
-                               cudaStream_t stream) {
-  if (block_size == 128) return launch<128, false, true>(tq, tk, tv, to, p, batch, stream);
-  if (block_size == 64) return launch<64, false, false>(tq, tk, tv, to, p, batch, stream);
-  return launch<32, false, false>(tq, tk, tv, to, p, batch, stream);
+                               const CUtensorMap& to, const AttnParams& p, int block_size, cudaStream_t stream) {
+  if (block_size == 128) return launch<128, false>(tq, tk, tv, to, p, stream);
+  if (block_size == 64) return launch<64, false>(tq, tk, tv, to, p, stream);
+  return launch<32, false>(tq, tk, tv, to, p, stream);
 }
 
 // Tensor maps: Q and O boxes 64 x 128 rows, K and V boxes 64 x 64 rows. p.num_q_tiles = ceil(seq_len / 128).
 cudaError_t launch_attn_dense(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv,
-                              const CUtensorMap& to, const AttnParams& p, int batch, cudaStream_t stream) {
-  return launch<128, true, false>(tq, tk, tv, to, p, batch, stream);
+                              const CUtensorMap& to, const AttnParams& p, cudaStream_t stream) {
+  return launch<128, true>(tq, tk, tv, to, p, stream);
 }
 
 }  // namespace sparsed

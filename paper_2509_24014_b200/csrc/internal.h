@@ -49,7 +49,7 @@ struct AttnParams {
   int num_q_tiles;         // 128-row query tiles per (batch, head)
   int num_blocks;          // sparse only: pattern blocks per row (seq_len / block_size)
   int num_items;           // batch * heads_q * num_q_tiles: 128-row query tiles in all
-  int max_ctas;            // > 0: launch at most this many CTAs and let each run through several items
+  int max_ctas;            // sparse only: CTAs that fit on the device at once (0: not known)
   float scale_log2;        // softmax scale * log2(e)
   const int32_t* row_ptr;  // sparse only
   const int32_t* col_idx;  // sparse only
@@ -120,14 +120,13 @@ size_t pooled_qk_means_bytes(int batch, int heads_q, int heads_kv, int nb);
 cudaError_t launch_pooled_qk_select(const PooledQkParams& p, cudaStream_t stream);
 // (`to`: tensor map of the output, boxes of 64 x 128 rows like Q's; the kernels write O through it)
 cudaError_t launch_attn_dense(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv,
-                              const CUtensorMap& to, const AttnParams& p, int batch, cudaStream_t stream);
+                              const CUtensorMap& to, const AttnParams& p, cudaStream_t stream);
 // The same pass with the MMAs spanning CTA pairs (cta_group::2); K tensor map with 32-row boxes.
 cudaError_t launch_attn_dense_pair(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv,
                                    const CUtensorMap& to, const AttnParams& p, cudaStream_t stream);
 int attn_sparse_max_blocks(int block_size);   // most key blocks per row the sparse kernel handles
 cudaError_t launch_attn_sparse(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv,
-                               const CUtensorMap& to, const AttnParams& p, int batch, int block_size,
-                               cudaStream_t stream);
+                               const CUtensorMap& to, const AttnParams& p, int block_size, cudaStream_t stream);
 bool score_ranks_in_kernel(int nb, int block_size);   // the pooled-scoring kernel ranks rows of nb key blocks itself
 bool score_in_one_pass(int nb);                       // ... and needs no log-sum-exp of the rows
 // (K tensor map of both: boxes of 64 x 64 rows)

@@ -154,6 +154,38 @@ __device__ __forceinline__ void named_barrier_sync(int id, int count) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(count) : "memory");
 }
 
+// ----------------------------------------------------------------------------
+// Cluster launch control: a running CTA takes over a CTA of its own grid that has not been launched yet.
+// The request is answered asynchronously with 16 bytes at `answer` (16-byte aligned shared memory), counted on
+// `bar`; after an answer that says "none left" no further request may be made.
+// ----------------------------------------------------------------------------
+__device__ __forceinline__ void launch_control_request(void* answer, uint64_t* bar) {
+  asm volatile("clusterlaunchcontrol.try_cancel.async.shared::cta.mbarrier::complete_tx::bytes.b128 [%0], [%1];" ::"r"(
+                   smem_u32(answer)),
+               "r"(smem_u32(bar))
+               : "memory");
+}
+// blockIdx.x of the CTA taken over, or -1 if none was left. Once every reader has called this, the buffer may serve
+// another request.
+__device__ __forceinline__ int launch_control_answer(const void* answer) {
+  uint32_t got, x;
+  asm volatile(
+      "{\n"
+      ".reg .pred p1;\n"
+      ".reg .b128 a;\n"
+      "ld.shared.b128 a, [%2];\n"
+      "clusterlaunchcontrol.query_cancel.is_canceled.pred.b128 p1, a;\n"
+      "selp.b32 %0, 1, 0, p1;\n"
+      "mov.b32 %1, 0;\n"
+      "@p1 clusterlaunchcontrol.query_cancel.get_first_ctaid::x.b32.b128 %1, a;\n"
+      "}\n"
+      : "=r"(got), "=r"(x)
+      : "r"(smem_u32(answer))
+      : "memory");
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  return got != 0 ? static_cast<int>(x) : -1;
+}
+
 __device__ __forceinline__ void tma_prefetch_desc(const void* tmap) {
   asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(tmap)) : "memory");
 }

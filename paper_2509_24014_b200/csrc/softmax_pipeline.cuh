@@ -53,6 +53,26 @@ __device__ __forceinline__ float2 softmax_group_fast(const uint32_t (&r0)[32], c
   return make_float2(acc0.x + acc0.y, acc1.x + acc1.y);
 }
 
+// The same over one half of a group: 32 columns, P into 16 registers, returns their sum.
+__device__ __forceinline__ float softmax_half_fast(const uint32_t (&r)[32], float scale_log2, float m, uint32_t (&pk)[16]) {
+  const float2 sc = make_float2(scale_log2, scale_log2);
+  const float2 nm = make_float2(-m, -m);
+  float2 acc0 = make_float2(0.f, 0.f), acc1 = make_float2(0.f, 0.f);
+#pragma unroll
+  for (int j = 0; j < 16; j += 2) {
+    const float2 x0 = __ffma2_rn(make_float2(__uint_as_float(r[2 * j]), __uint_as_float(r[2 * j + 1])), sc, nm);
+    const float2 x1 = __ffma2_rn(make_float2(__uint_as_float(r[2 * j + 2]), __uint_as_float(r[2 * j + 3])), sc, nm);
+    const float2 e0 = make_float2(fast_exp2(x0.x), fast_exp2(x0.y));
+    const float2 e1 = make_float2(fast_exp2(x1.x), fast_exp2(x1.y));
+    acc0 = __fadd2_rn(acc0, e0);
+    acc1 = __fadd2_rn(acc1, e1);
+    pk[j] = pack_bf16x2(e0.x, e0.y);
+    pk[j + 1] = pack_bf16x2(e1.x, e1.y);
+  }
+  const float2 acc = __fadd2_rn(acc0, acc1);
+  return acc.x + acc.y;
+}
+
 // Exact path: adopts the group's true maximum where it exceeds st.m, redoes the group against
 // the (possibly new) st.m and returns the factor by which everything accumulated before this
 // group (st.l, already scaled here, and the caller's output accumulator) has to be multiplied.
@@ -91,6 +111,60 @@ __device__ __forceinline__ float softmax_group_exact(const uint32_t (&r0)[32], c
   }
   sums = make_float2(s0, s1);
   return alpha;
+}
+
+// One 64-key tile of a walk in which a warp's rows may keep both, one or none of the tile's 32-column halves
+// (keep0 / keep1, the same for the whole warp; both alike with kBlocksPerTile = 1). What is not kept is not even copied
+// out of tensor memory: its P is zero. Otherwise as above; `rescale(alpha)` brings the output accumulator to a new
+// reference maximum and returns false if that could not be done.
+template <int kBlocksPerTile, class Rescale>
+__device__ __forceinline__ bool packed_softmax_tile(uint32_t tS, bool keep0, bool keep1, float scale_log2, RowState& st,
+                                                    uint32_t (&pk)[32], Rescale rescale) {
+  if (!keep0 && !keep1) {
+#pragma unroll
+    for (int j = 0; j < 32; ++j) pk[j] = 0u;
+    return true;
+  }
+  float2 sums = make_float2(0.f, 0.f);
+  bool exact = (st.m == -INFINITY);   // nothing accumulated yet: no reference maximum to try
+  if (!__all_sync(0xffffffffu, exact)) {
+    if (kBlocksPerTile == 1 || (keep0 && keep1)) {
+      uint32_t r0[32], r1[32];
+      tmem_ld32(tS, r0);
+      tmem_ld32(tS + 32, r1);
+      tmem_wait_ld();
+      sums = softmax_group_fast(r0, r1, scale_log2, st.m, pk);
+    } else {
+      uint32_t r[32], half[16];
+      tmem_ld32(keep0 ? tS : tS + 32, r);
+      tmem_wait_ld();
+      sums.x = softmax_half_fast(r, scale_log2, st.m, half);
+#pragma unroll
+      for (int j = 0; j < 16; ++j) {
+        pk[j] = keep0 ? half[j] : 0u;
+        pk[16 + j] = keep0 ? 0u : half[j];
+      }
+    }
+    exact = !(sums.x + sums.y <= 256.0f);   // logits outgrew the running maximum (or NaN)
+  }
+  if (__any_sync(0xffffffffu, exact)) {
+    uint32_t r0[32], r1[32];   // (S is still in tensor memory)
+    tmem_ld32(tS, r0);
+    tmem_ld32(tS + 32, r1);
+    tmem_wait_ld();
+    if (!keep0) {
+#pragma unroll
+      for (int j = 0; j < 32; ++j) r0[j] = 0xff800000u;   // -inf
+    }
+    if (!keep1) {
+#pragma unroll
+      for (int j = 0; j < 32; ++j) r1[j] = 0xff800000u;
+    }
+    const float alpha = softmax_group_exact(r0, r1, scale_log2, st, pk, sums);
+    if (!rescale(alpha)) return false;
+  }
+  st.l += sums.x + sums.y;
+  return true;
 }
 
 // Multiplies this thread's row of a 128-column fp32 accumulator in tensor memory by alpha.
