@@ -8,6 +8,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+import struct
 from typing import Optional, Tuple
 
 import torch
@@ -122,25 +123,30 @@ def _check(status: int, what: str) -> None:
 
 
 def _stream(t: torch.Tensor) -> int:
-    return int(torch.cuda.current_stream(t.device).cuda_stream)
+    # the handle itself: torch.cuda.current_stream() builds a Stream object around it first (2.3 us against 0.1)
+    if t.is_cuda:
+        return torch._C._cuda_getCurrentRawStream(t.get_device())
+    return int(torch.cuda.current_stream(t.device).cuda_stream)   # raises
 
 
-def _strides3(t: torch.Tensor):
-    if t.dim() != 4 or t.stride(3) != 1:
-        raise ValueError("tensors must be [batch, heads, seq_len, head_dim] with head_dim contiguous")
-    return (ctypes.c_int64 * 3)(t.stride(0), t.stride(1), t.stride(2))
+# sparsed_shape up to its last field as one packed record (5 int32, 12 int64, native alignment; the scale is 0, its
+# default): filling the ctypes structure field by field took 5.9 us of a call's 20.
+_SHAPE_RECORD = struct.Struct("@5i12q%dx" % (ctypes.sizeof(Shape) - struct.calcsize("@5i12q")))
 
 
 def make_shape(q: torch.Tensor, k: torch.Tensor, v: Optional[torch.Tensor] = None,
                o: Optional[torch.Tensor] = None, softmax_scale: float = 0.0) -> Shape:
-    s = Shape()
-    s.batch, s.heads_q, s.seq_len, s.head_dim = q.shape
-    s.heads_kv = k.shape[1]
-    s.q_strides = _strides3(q)
-    s.k_strides = _strides3(k)
-    s.v_strides = _strides3(v if v is not None else k)
-    s.o_strides = _strides3(o if o is not None else q)
-    s.softmax_scale = softmax_scale
+    batch, heads_q, seq_len, head_dim = q.shape
+    sq, sk = q.stride(), k.stride()
+    sv = v.stride() if v is not None else sk
+    so = o.stride() if o is not None else sq
+    if not (len(sk) == len(sv) == len(so) == 4 and sq[3] == sk[3] == sv[3] == so[3] == 1):
+        raise ValueError("tensors must be [batch, heads, seq_len, head_dim] with head_dim contiguous")
+    s = Shape.from_buffer_copy(_SHAPE_RECORD.pack(
+        batch, heads_q, k.shape[1], seq_len, head_dim, sq[0], sq[1], sq[2], sk[0], sk[1], sk[2], sv[0], sv[1], sv[2],
+        so[0], so[1], so[2]))
+    if softmax_scale != 0.0:
+        s.softmax_scale = softmax_scale
     return s
 
 
