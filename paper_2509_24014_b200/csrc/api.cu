@@ -138,8 +138,9 @@ sparsed_status check_arch() {
   return major == 10 ? SPARSED_OK : SPARSED_ERR_ARCH;
 }
 
-// CTAs of the attention kernel that are resident on the current device at once (two per SM), cached per
-// device; 0 if the SM count cannot be read (the kernel then gets one CTA per query tile).
+// CTAs of the single-CTA attention kernel, or of the scoring kernel, that are resident on the current device at once
+// (two per SM), cached per device; 0 if the SM count cannot be read (the attention kernel then gets one CTA per query
+// tile).
 int attn_max_ctas() {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return 0;
@@ -400,7 +401,7 @@ static sparsed_status attn_full_impl(const sparsed_shape* shape, const void* q, 
   p.num_q_tiles = (shape->seq_len + 127) / 128;
   p.num_blocks = 0;
   p.num_items = shape->batch * shape->heads_q * p.num_q_tiles;
-  p.max_ctas = 0;
+  p.max_ctas = attn_max_ctas();
   p.scale_log2 = rs.scale_log2;
   p.row_ptr = nullptr;
   p.col_idx = nullptr;
@@ -639,6 +640,7 @@ sparsed_status sparsed_select_pattern(const sparsed_shape* shape, const sparsed_
   sp.pb = pb;
   sp.k_pre = k_pre;
   sp.k_gen = k_gen;
+  sp.max_ctas = attn_max_ctas();
   sp.lse_out = nullptr;
   if (lse_or_null == nullptr && !one_pass) {
     sp.lse_out = reinterpret_cast<float*>(base + off);

@@ -88,7 +88,9 @@ constexpr int kIdBits = 11;
 static_assert((1 << kIdBits) == kMaxPackedBlocks, "ids of union entries");
 
 // kDense: walk every key tile of the sequence (kBlock must be 128 then; no block lists are read).
-template <int kBlock, bool kDense>
+// kOverlap: launched with launch_overlapped. (Of the dense walk there are both kinds: with the wait at its start the
+// compiler arranges its main loop differently, and long launches take 1.4 % longer.)
+template <int kBlock, bool kDense, bool kOverlap>
 __global__ void __launch_bounds__(kThreads, 2)
 attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
             const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_o, const AttnParams p) {
@@ -101,6 +103,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
   constexpr int kBlocksPerTile = kBlock >= kTileN ? 1 : kTileN / kBlock;   // 32-key blocks: two per tile
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   Smem& sm = *reinterpret_cast<Smem*>(smem_raw);
+  if constexpr (kOverlap) wait_for_previous_kernel();
   if ((smem_u32(smem_raw) & 1023u) != 0u) {
     // swizzled tiles need a 1024-byte aligned base; never expected, reported instead of trusted
     if (threadIdx.x == 0 && atomicCAS(&p.status->code, 0, 2) == 0) p.status->where = 1;
@@ -145,8 +148,8 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
     it.list_len = (p.seq_len + kTileN - 1) / kTileN;
     if (!kDense && with_list) {
       // adjacent rows are adjacent in col_idx, so the item's lists are one run of entries
-      it.list_begin = __ldg(p.row_ptr + it.r0);
-      it.list_len = __ldg(p.row_ptr + it.r0 + it.groups_here) - it.list_begin;
+      it.list_begin = __ldcg(p.row_ptr + it.r0);
+      it.list_len = __ldcg(p.row_ptr + it.r0 + it.groups_here) - it.list_begin;
       if (it.list_begin < 0 || it.list_len < 0 ||
           static_cast<int64_t>(it.list_begin) + it.list_len > p.col_capacity) {
         // row_ptr points outside col_idx: not followed; the rows get zeros and the status word says why
@@ -210,13 +213,13 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
     for (int i = lane; i < kGroups * Smem::kWords; i += 32) (&sm.member[0][0])[i] = 0u;
     int bound[kGroups];   // bound[g] = first CSR entry after query block g's list
 #pragma unroll
-    for (int g = 0; g < kGroups; ++g) bound[g] = __ldg(p.row_ptr + it.r0 + min(g + 1, it.groups_here));
+    for (int g = 0; g < kGroups; ++g) bound[g] = __ldcg(p.row_ptr + it.r0 + min(g + 1, it.groups_here));
     __syncwarp();
     const int list_end = it.list_begin + it.list_len;
     for (int e0 = it.list_begin + lane; e0 < list_end; e0 += 8 * 32) {
       int id[8];   // eight loads in flight per lane
 #pragma unroll
-      for (int u = 0; u < 8; ++u) id[u] = e0 + 32 * u < list_end ? __ldg(p.col_idx + e0 + 32 * u) : -1;
+      for (int u = 0; u < 8; ++u) id[u] = e0 + 32 * u < list_end ? __ldcg(p.col_idx + e0 + 32 * u) : -1;
 #pragma unroll
       for (int u = 0; u < 8; ++u) {
         int g = 0;
@@ -304,7 +307,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
     } else if (cur.list_len > 0) {
       issue_q_load(cur);
       if constexpr (!kDense) {
-        if (lane < cur.list_len) list_ids = __ldg(p.col_idx + cur.list_begin + lane);
+        if (lane < cur.list_len) list_ids = __ldcg(p.col_idx + cur.list_begin + lane);
       }
       const int first = min(2 * unpacked_tiles(cur), kSlots);   // list entries 0..2 at most: within the first chunk
       for (; loads_issued < first; ++loads_issued)
@@ -376,7 +379,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
           cur = describe(item, true);
           n_entries = cur.list_len;
           q_pending = n_entries > 0;
-          list_ids = (lane < cur.list_len) ? __ldg(p.col_idx + cur.list_begin + lane) : 0;
+          list_ids = (lane < cur.list_len) ? __ldcg(p.col_idx + cur.list_begin + lane) : 0;
         }
       }
       auto settle_q = [&]() -> bool {
@@ -404,7 +407,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
             // block ids are fetched 32 at a time, one per lane, when the walk enters a new chunk
             const int e = t / kTilesPerBlock;
             if ((i & 1) == 0 && e > 0 && (e & 31) == 0 && t % kTilesPerBlock == 0)
-              list_ids = (e + lane < n_entries) ? __ldg(p.col_idx + cur.list_begin + e + lane) : 0;
+              list_ids = (e + lane < n_entries) ? __ldcg(p.col_idx + cur.list_begin + e + lane) : 0;
           }
           kv_row0 = unpacked_row(t);
         } else {
@@ -685,10 +688,10 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
   }
 }
 
-template <int kBlock, bool kDense>
+template <int kBlock, bool kDense, bool kOverlap>
 cudaError_t launch(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap& to,
                    const AttnParams& p, cudaStream_t stream) {
-  auto kernel = attn_kernel<kBlock, kDense>;
+  auto kernel = attn_kernel<kBlock, kDense, kOverlap>;
   const int smem = static_cast<int>(sizeof(AttnSmem<kBlock>));
   static_assert(sizeof(AttnSmem<kBlock>) <= 113 * 1024, "two CTAs per SM");
   static SmemLimit limit;  // per template instantiation
@@ -698,8 +701,7 @@ cudaError_t launch(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorM
   if (ctas <= 0) return cudaSuccess;
   // 128-key blocks: at most as many CTAs as are resident at once, each with its share of the items
   if (kBlock == 128 && !kDense && p.max_ctas > 0 && ctas > p.max_ctas) ctas = p.max_ctas;
-  kernel<<<static_cast<unsigned>(ctas), kThreads, smem, stream>>>(tq, tk, tv, to, p);
-  return cudaGetLastError();
+  return launch_overlapped(kernel, ctas, kOverlap ? p.max_ctas : 0, kThreads, smem, stream, tq, tk, tv, to, p);
 }
 
 }  // namespace
@@ -710,15 +712,16 @@ int attn_sparse_max_blocks(int block_size) { return block_size < kTileM ? kMaxPa
 // p.num_q_tiles = ceil(seq_len / 128), p.num_blocks = seq_len / block_size.
 cudaError_t launch_attn_sparse(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv,
                                const CUtensorMap& to, const AttnParams& p, int block_size, cudaStream_t stream) {
-  if (block_size == 128) return launch<128, false>(tq, tk, tv, to, p, stream);
-  if (block_size == 64) return launch<64, false>(tq, tk, tv, to, p, stream);
-  return launch<32, false>(tq, tk, tv, to, p, stream);
+  if (block_size == 128) return launch<128, false, true>(tq, tk, tv, to, p, stream);
+  if (block_size == 64) return launch<64, false, true>(tq, tk, tv, to, p, stream);
+  return launch<32, false, true>(tq, tk, tv, to, p, stream);
 }
 
 // Tensor maps: Q and O boxes 64 x 128 rows, K and V boxes 64 x 64 rows. p.num_q_tiles = ceil(seq_len / 128).
 cudaError_t launch_attn_dense(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv,
                               const CUtensorMap& to, const AttnParams& p, cudaStream_t stream) {
-  return launch<128, true>(tq, tk, tv, to, p, stream);
+  return p.num_items <= p.max_ctas ? launch<128, true, true>(tq, tk, tv, to, p, stream)
+                                   : launch<128, true, false>(tq, tk, tv, to, p, stream);
 }
 
 }  // namespace sparsed

@@ -34,6 +34,25 @@ inline cudaError_t ensure_dynamic_smem(Kernel kernel, int bytes, SmemLimit& lim)
   return e;
 }
 
+// Launches a kernel that begins with wait_for_previous_kernel(). If the grid fits on the device at once
+// (resident_ctas; 0: not known, or not wanted), its CTAs may be started before the kernel before it in the stream has ended, which takes
+// 1.7 us off a call of 15 (2 heads x 1024 tokens, dense). Larger grids gain nothing from it and are launched as usual.
+template <class... Params, class... Args>
+inline cudaError_t launch_overlapped(void (*kernel)(Params...), long long ctas, int resident_ctas, int threads, size_t smem,
+                                     cudaStream_t stream, const Args&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(static_cast<unsigned>(ctas));
+  cfg.blockDim = dim3(static_cast<unsigned>(threads));
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute attr = {};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = ctas <= resident_ctas ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
 // Parameters shared by the dense and the block-sparse attention kernels.
 struct AttnParams {
   void* o;                 // bf16 [B,Hq,L,D]; used by the plain dense kernel, which stores rows itself (the others
@@ -49,7 +68,7 @@ struct AttnParams {
   int num_q_tiles;         // 128-row query tiles per (batch, head)
   int num_blocks;          // sparse only: pattern blocks per row (seq_len / block_size)
   int num_items;           // batch * heads_q * num_q_tiles: 128-row query tiles in all
-  int max_ctas;            // sparse only: CTAs that fit on the device at once (0: not known)
+  int max_ctas;            // CTAs of the single-CTA kernel that fit on the device at once (0: not known)
   float scale_log2;        // softmax scale * log2(e)
   const int32_t* row_ptr;  // sparse only
   const int32_t* col_idx;  // sparse only
@@ -72,6 +91,7 @@ struct ScoreParams {
   int32_t* row_ptr;
   int32_t* col_idx;
   int pb, k_pre, k_gen;
+  int max_ctas;            // CTAs that fit on the device at once (0: not known)
 };
 
 // Parameters of the kernel that pools per-tile row statistics into A' and ranks it.

@@ -118,6 +118,7 @@ __global__ void __launch_bounds__(kThreads, 2)
 score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k, const ScoreParams p) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   ScoreSmem& sm = *reinterpret_cast<ScoreSmem*>(smem_raw);
+  wait_for_previous_kernel();
   if ((smem_u32(smem_raw) & 1023u) != 0u) {
     if (threadIdx.x == 0 && atomicCAS(&p.status->code, 0, 2) == 0) p.status->where = 2;
     return;
@@ -396,8 +397,7 @@ cudaError_t launch(const CUtensorMap& tq, const CUtensorMap& tk, const ScorePara
   const int num_q_tiles = (p.seq_len + kTileM - 1) / kTileM;
   const long long ctas = static_cast<long long>(batch) * p.heads_q * num_q_tiles;
   if (ctas <= 0) return cudaSuccess;
-  kernel<<<static_cast<unsigned>(ctas), kThreads, smem, stream>>>(tq, tk, p);
-  return cudaGetLastError();
+  return launch_overlapped(kernel, ctas, p.max_ctas, kThreads, smem, stream, tq, tk, p);
 }
 
 }  // namespace

@@ -113,6 +113,17 @@ __device__ __forceinline__ bool mbar_wait2(uint64_t* bar_a, uint32_t parity_a, u
 }
 
 // ----------------------------------------------------------------------------
+// Overlap with the kernel before it in the stream (launch_overlapped in internal.h): a kernel's CTAs may be started
+// while that kernel's last CTAs still run. This, at a kernel's start, returns when that kernel has completed and its
+// writes are visible; only then is the next kernel allowed to start, so that at most two kernels of a stream
+// overlap. Data that an earlier kernel may have written is read with TMA, __ldcg, __ldcs or plain loads, not __ldg.
+// ----------------------------------------------------------------------------
+__device__ __forceinline__ void wait_for_previous_kernel() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+// ----------------------------------------------------------------------------
 // Proxy fences
 // ----------------------------------------------------------------------------
 __device__ __forceinline__ void fence_proxy_async_smem() {
