@@ -15,16 +15,16 @@ PKG_DIR = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(PKG_DIR, "csrc")
 OBJ_DIR = os.path.join(PKG_DIR, "build")
 LIB_PATH = os.path.join(PKG_DIR, "libsparsed.so")
-SOURCES = ["api.cu", "attention.cu", "attention_dense_pair.cu", "scoring.cu", "topk.cu", "pool_select.cu", "patterns.cu",
+SOURCES = ["api.cu", "attention.cu", "attention_dense_pair.cu", "attention_dense_pair_split.cu", "scoring.cu", "topk.cu", "pool_select.cu", "patterns.cu",
            "pooled_qk.cu"]
-HEADERS = ["internal.h", "sm100_primitives.cuh", "sm100_pair_primitives.cuh", "softmax_pipeline.cuh", "topk_device.cuh",
+HEADERS = ["internal.h", "attention_dense_pair.cu", "sm100_primitives.cuh", "sm100_pair_primitives.cuh", "softmax_pipeline.cuh", "topk_device.cuh",
            os.path.join("..", "..", "include", "sparsed.h")]
 ARCH_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a"]
 COMMON_FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC"]
 # Flags of single files. The CTA-pair dense kernel is built with denormals flushed to zero: its softmax handles
 # probabilities, for which a flushed 1e-38 is as good as the number, and the kernel measured 2-4 % faster that way
 # (8k-64k); the other kernels measured the same or slower with it and keep IEEE denormals.
-PER_FILE_FLAGS = {"attention_dense_pair.cu": ["-ftz=true"]}
+PER_FILE_FLAGS = {"attention_dense_pair.cu": ["-ftz=true"], "attention_dense_pair_split.cu": ["-ftz=true"]}
 
 
 def _nvcc() -> str:

@@ -29,6 +29,9 @@
 #include "sm100_pair_primitives.cuh"
 #include "softmax_pipeline.cuh"
 
+// This file is compiled twice: as it is, and (attention_dense_pair_split.cu) with SPARSED_SPLIT_CLUSTERS for grids whose last
+// clusters own one stream each. Not as a template parameter: any change in the text of the kernel, even one that folds
+// away, makes the compiler schedule the softmax warps' loop differently, by -4 to +1 % of the long launches' time.
 namespace sparsed {
 namespace {
 
@@ -88,10 +91,21 @@ attn_dense_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
 
   // ---- which rows ---------------------------------------------------------------------------
   // cluster c of a (batch, head) owns query tiles 4c .. 4c+3: stream s of CTA r has tile 4c + 2s + r
+#ifdef SPARSED_SPLIT_CLUSTERS
+  // beyond the grid's first p.max_ctas clusters two launched ones share one, a stream each
+  const int beyond = static_cast<int>(blockIdx.x >> 1) - p.max_ctas;
+  const bool whole = beyond < 0;
+  const int cluster_id = p.max_ctas + (whole ? beyond : beyond >> 1);
+  const int clusters_per_head = (p.num_q_tiles + 3) >> 2;
+  const int bh = cluster_id / clusters_per_head;
+  const int first_tile = (cluster_id % clusters_per_head) * 4 + (whole ? 0 : 2 * (beyond & 1));
+#else
+  constexpr bool whole = true;
   const int cluster_id = blockIdx.x >> 1;
   const int clusters_per_head = (p.num_q_tiles + 3) >> 2;
   const int bh = cluster_id / clusters_per_head;
   const int first_tile = (cluster_id % clusters_per_head) * 4;
+#endif
   const int head = bh % p.heads_q;
   const int batch = bh / p.heads_q;
   const int kv_head = head / p.group;
@@ -143,7 +157,7 @@ attn_dense_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
   const int q_row0 = q_tile * kTileM;
   // a stream whose leader tile lies beyond the sequence has no rows at all; one whose peer tile does still runs
   // as a pair: the peer's Q arrives as zeros and its rows are not stored
-  const bool active = pair_ok && (first_tile + 2 * s_of_warp) < p.num_q_tiles;
+  const bool active = pair_ok && (first_tile + 2 * s_of_warp) < p.num_q_tiles && (whole || s_of_warp == 0);
   const uint32_t tS0 = tmem + s_of_warp * 256 + kColS;
   const uint32_t tO = tmem + s_of_warp * 256 + kColO;
 
@@ -153,7 +167,7 @@ attn_dense_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
     // (spare warp)
   } else if (warp == 8) {
     // =============================== TMA producer (both streams) =============================
-    const bool two = pair_ok && (first_tile + 2) < p.num_q_tiles;   // stream 1 has rows
+    const bool two = pair_ok && (first_tile + 2) < p.num_q_tiles && whole;   // stream 1 has rows
     if (elect_one_sync()) {
       for (int s = 0; s < (two ? 2 : 1); ++s) {
         PairStream& T = sm.stream[s];
@@ -359,28 +373,51 @@ attn_dense_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
 
 template <int kStatKeys>
 cudaError_t launch_pair(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap& to,
-                        const AttnParams& p, cudaStream_t stream) {
+                        const AttnParams& p, long long clusters, cudaStream_t stream) {
   auto kernel = attn_dense_pair_kernel<kStatKeys>;
   const int smem = static_cast<int>(sizeof(PairSmem));
   static SmemLimit limit;  // per template instantiation
   cudaError_t e = ensure_dynamic_smem(kernel, smem, limit);
   if (e != cudaSuccess) return e;
-  const long long bh = p.num_q_tiles > 0 ? p.num_items / p.num_q_tiles : 0;
-  const long long clusters = bh * ((p.num_q_tiles + 3) / 4);
-  if (clusters <= 0) return cudaSuccess;
   kernel<<<static_cast<unsigned>(2 * clusters), kThreads, smem, stream>>>(tq, tk, tv, to, p);
   return cudaGetLastError();
 }
 
+cudaError_t launch_any(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap& to,
+                       const AttnParams& p, long long clusters, cudaStream_t stream) {
+  if (p.tile_lse == nullptr) return launch_pair<0>(tq, tk, tv, to, p, clusters, stream);
+  if (p.stat_keys == 128) return launch_pair<128>(tq, tk, tv, to, p, clusters, stream);
+  if (p.stat_keys == 64) return launch_pair<64>(tq, tk, tv, to, p, clusters, stream);
+  return launch_pair<32>(tq, tk, tv, to, p, clusters, stream);
+}
+
 }  // namespace
 
+#ifdef SPARSED_SPLIT_CLUSTERS
+cudaError_t launch_attn_dense_pair_split(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv,
+                                         const CUtensorMap& to, const AttnParams& p, long long clusters,
+                                         cudaStream_t stream) {
+  return launch_any(tq, tk, tv, to, p, clusters, stream);
+}
+#else
 // Tensor maps: Q and O boxes 64 x 128 rows, K box 64 x 32 rows, V box 64 x 64 rows. p.num_q_tiles = ceil(seq_len / 128).
+//
+// A cluster with one stream takes 0.65-0.8 of the time of one with two. So a last wave that would leave half of the SM
+// pairs idle or more is launched as clusters of one stream each: 2 heads x 4096 tokens 63.5 -> 47.1 us, 8 x 2048
+// 36.9 -> 28.7, 2 x 1024 22.6 -> 18.4, 16 x 3072 (1.3 waves) 95.0 -> 84.4 (statistics recorded). From two full waves on the
+// launch runs into the power limit, which an emptier last wave only relieves (32 x 4096, 3.46 waves: no gain).
 cudaError_t launch_attn_dense_pair(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv,
                                    const CUtensorMap& to, const AttnParams& p, cudaStream_t stream) {
-  if (p.tile_lse == nullptr) return launch_pair<0>(tq, tk, tv, to, p, stream);
-  if (p.stat_keys == 128) return launch_pair<128>(tq, tk, tv, to, p, stream);
-  if (p.stat_keys == 64) return launch_pair<64>(tq, tk, tv, to, p, stream);
-  return launch_pair<32>(tq, tk, tv, to, p, stream);
+  const long long bh = p.num_q_tiles > 0 ? p.num_items / p.num_q_tiles : 0;
+  const long long clusters = bh * ((p.num_q_tiles + 3) / 4);
+  if (clusters <= 0) return cudaSuccess;
+  const long long pairs = p.max_ctas / 4;   // SM pairs of the device (max_ctas: two CTAs per SM)
+  const long long last = pairs > 0 ? clusters % pairs : 0;
+  if (last == 0 || 2 * last > pairs || clusters >= 2 * pairs) return launch_any(tq, tk, tv, to, p, clusters, stream);
+  AttnParams split = p;
+  split.max_ctas = static_cast<int>(clusters - last);
+  return launch_attn_dense_pair_split(tq, tk, tv, to, split, clusters + last, stream);
 }
+#endif
 
 }  // namespace sparsed

@@ -68,7 +68,8 @@ struct AttnParams {
   int num_q_tiles;         // 128-row query tiles per (batch, head)
   int num_blocks;          // sparse only: pattern blocks per row (seq_len / block_size)
   int num_items;           // batch * heads_q * num_q_tiles: 128-row query tiles in all
-  int max_ctas;            // CTAs of the single-CTA kernel that fit on the device at once (0: not known)
+  int max_ctas;            // CTAs of the single-CTA kernel that fit on the device at once (0: not known); in the split
+                           // launch of the CTA-pair kernel the clusters that own 512 query rows, the rest own 256
   float scale_log2;        // softmax scale * log2(e)
   const int32_t* row_ptr;  // sparse only
   const int32_t* col_idx;  // sparse only
@@ -144,6 +145,10 @@ cudaError_t launch_attn_dense(const CUtensorMap& tq, const CUtensorMap& tk, cons
 // The same pass with the MMAs spanning CTA pairs (cta_group::2); K tensor map with 32-row boxes.
 cudaError_t launch_attn_dense_pair(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv,
                                    const CUtensorMap& to, const AttnParams& p, cudaStream_t stream);
+// ... in `clusters` clusters, of which those beyond the first p.max_ctas own one stream
+cudaError_t launch_attn_dense_pair_split(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv,
+                                         const CUtensorMap& to, const AttnParams& p, long long clusters,
+                                         cudaStream_t stream);
 int attn_sparse_max_blocks(int block_size);   // most key blocks per row the sparse kernel handles
 cudaError_t launch_attn_sparse(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv,
                                const CUtensorMap& to, const AttnParams& p, int block_size, cudaStream_t stream);

@@ -1,0 +1,23 @@
+"""The CTA-pair dense kernel on grids whose last clusters (or all of them) own one stream of 256 query rows: the same
+bits as the single-CTA kernel gives, for query tiles that fill clusters wholly, half and by one tile."""
+import pytest
+import torch
+
+import paper_2509_24014_b200 as sd
+from paper_2509_24014_b200 import synthetic as syn
+from tests.parity_util import gpu_full
+from tests.test_gpu_switch_step_stats import gpu_switch_step
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("Hq,Hkv,L,bs", [
+    (1, 1, 128, 64), (2, 1, 640, 128), (37, 37, 512, 64),    # all clusters split (37 of them: the most on 74 SM pairs)
+    (38, 38, 512, 64),                                        # none split
+    (16, 4, 2944, 128), (19, 19, 2080, 32), (37, 37, 1536, 64)])   # a wave of whole clusters, then split ones
+def test_same_bits_as_the_single_cta_kernel(Hq, Hkv, L, bs):
+    q, k, v = syn.make_qkv(syn.AttnConfig("split", 1, Hq, Hkv, L, 128, bs, 0.3, 0, seed=95, plant_norm=6.0), "cuda")
+    o, lse, _, _, _, scores = gpu_switch_step(q, k, v, bs, 0.3, 0)
+    o_plain, lse_plain = gpu_full(q, k, v)
+    assert torch.equal(o, o_plain) and torch.equal(lse, lse_plain)
+    assert torch.allclose(scores.double().sum(-1), torch.full_like(scores[..., 0], 1.0 / bs).double(), rtol=2e-5)
