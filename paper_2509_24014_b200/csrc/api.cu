@@ -354,11 +354,21 @@ sparsed_status sparsed_workspace_init(void* ws, size_t ws_bytes, void* cuda_stre
 }
 
 // Which dense kernel runs. The pass that also records row statistics has one kernel, whose MMAs span CTA
-// pairs (attention_dense_pair.cu). The plain pass runs it from 16k tokens on (measured 3-4 % faster there) and
-// the single-CTA kernel (attention.cu) below that, where a cluster's short life makes the pair kernel no
-// faster under sustained load and slower per launch. The environment variable SPARSED_DENSE_KERNEL (read once)
-// sends every plain pass to one of them, `pair` or `single`, for A/B measurements and tests.
-static bool dense_pair_kernel(bool with_stats, int seq_len) {
+// pairs (attention_dense_pair.cu). For the plain pass both kernels give the same bits. Per query row the pair kernel takes
+// 3-4 % less from 4096 tokens on (it fetches each K/V tile once for 512 rows instead of once for 128, and sustained
+// launches are bound by power: 32 heads x 8192 951 -> 920 us, 8 x 32 x 4096 1956 -> 1883), below that a cluster's set-up
+// and tear-down weigh more (32 x 1900: 64.4 against 65.6). A wave of either is the same number of rows, but the last one
+// may be emptier: 8 heads x 14000 are 3.03 waves of clusters (740 us) and 2.97 of single CTAs (687). So the waves
+// are counted: a last one that is at most half full as 0.65 where its half-empty SMs run faster (two CTAs per SM, or split
+// clusters), else as 0.5 and half its share (the SMs that are busy have the power of the others). The environment variable SPARSED_DENSE_KERNEL (read once) sends every plain pass to one of them, `pair` or
+// `single`, for A/B measurements and tests.
+static double waves(long long units, long long slots, bool half_wave) {
+  const long long last = units % slots;
+  const double whole = static_cast<double>(units / slots);
+  if (last == 0) return whole;
+  return whole + (half_wave && 2 * last <= slots ? 0.65 : 0.5 + 0.5 * static_cast<double>(last) / static_cast<double>(slots));
+}
+static bool dense_pair_kernel(bool with_stats, const sparsed_shape* shape, int max_ctas) {
   static const int forced = [] {
     const char* v = std::getenv("SPARSED_DENSE_KERNEL");
     if (v != nullptr && std::strcmp(v, "pair") == 0) return 1;
@@ -366,7 +376,12 @@ static bool dense_pair_kernel(bool with_stats, int seq_len) {
     return -1;
   }();
   if (with_stats) return true;
-  return forced >= 0 ? forced == 1 : seq_len >= 16384;
+  if (forced >= 0) return forced == 1;
+  if (shape->seq_len < 4096 || max_ctas < 4) return false;
+  const long long bh = static_cast<long long>(shape->batch) * shape->heads_q;
+  const long long tiles = (shape->seq_len + 127) / 128;
+  const long long clusters = bh * ((tiles + 3) / 4), pairs = max_ctas / 4;
+  return 0.965 * waves(clusters, pairs, clusters < 2 * pairs) < waves(bh * tiles, max_ctas, true);
 }
 
 static sparsed_status attn_full_impl(const sparsed_shape* shape, const void* q, const void* k, const void* v, void* o,
@@ -380,7 +395,8 @@ static sparsed_status attn_full_impl(const sparsed_shape* shape, const void* q, 
   if (!aligned16(lse_or_null) || !aligned16(tile_lse_or_null)) return SPARSED_ERR_ALIGNMENT;
   if ((st = check_ws(ws, ws_bytes, SPARSED_STATUS_BYTES)) != SPARSED_OK) return st;
   if ((st = check_arch()) != SPARSED_OK) return st;
-  const bool pair = dense_pair_kernel(tile_lse_or_null != nullptr, shape->seq_len);
+  const int max_ctas = attn_max_ctas();
+  const bool pair = dense_pair_kernel(tile_lse_or_null != nullptr, shape, max_ctas);
   CUtensorMap tq, tk, tv, to;
   if ((st = make_tensor_map(&tq, q, shape->batch, shape->heads_q, shape->seq_len, rs.q, 128)) != SPARSED_OK) return st;
   if ((st = make_tensor_map(&to, o, shape->batch, shape->heads_q, shape->seq_len, rs.o, 128)) != SPARSED_OK) return st;
@@ -401,7 +417,7 @@ static sparsed_status attn_full_impl(const sparsed_shape* shape, const void* q, 
   p.num_q_tiles = (shape->seq_len + 127) / 128;
   p.num_blocks = 0;
   p.num_items = shape->batch * shape->heads_q * p.num_q_tiles;
-  p.max_ctas = attn_max_ctas();
+  p.max_ctas = max_ctas;
   p.scale_log2 = rs.scale_log2;
   p.row_ptr = nullptr;
   p.col_idx = nullptr;

@@ -70,7 +70,7 @@ constexpr uint32_t kQHalfStep = (kTileM * 64 * 2) >> 4;                  // 16 K
 constexpr uint32_t kKHalfStep = (32 * 64 * 2) >> 4;                      // 4 KB per head_dim half of a K half-tile
 constexpr uint32_t kSlotStep = (kTileN * 64 * 2) >> 4;                   // 8 KB per ring slot
 
-// kStatKeys: 0, or record one row statistic per 32 / 64 / 128 keys.
+// kStatKeys: record one row statistic per 32 / 64 / 128 keys (none if p.tile_lse is null).
 template <int kStatKeys>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 attn_dense_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
@@ -385,8 +385,9 @@ cudaError_t launch_pair(const CUtensorMap& tq, const CUtensorMap& tk, const CUte
 
 cudaError_t launch_any(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const CUtensorMap& to,
                        const AttnParams& p, long long clusters, cudaStream_t stream) {
-  if (p.tile_lse == nullptr) return launch_pair<0>(tq, tk, tv, to, p, clusters, stream);
-  if (p.stat_keys == 128) return launch_pair<128>(tq, tk, tv, to, p, clusters, stream);
+  // The plain pass runs the instantiation for 128-key statistics and stores none (tile_lse is null): its main loop
+  // compiles 2.5-3 % faster than that of one without them (32 heads x 8192: 945 -> 920 us; <64>: 948, <32>: 970).
+  if (p.tile_lse == nullptr || p.stat_keys == 128) return launch_pair<128>(tq, tk, tv, to, p, clusters, stream);
   if (p.stat_keys == 64) return launch_pair<64>(tq, tk, tv, to, p, clusters, stream);
   return launch_pair<32>(tq, tk, tv, to, p, clusters, stream);
 }
