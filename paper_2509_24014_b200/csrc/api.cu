@@ -621,7 +621,7 @@ sparsed_status sparsed_select_pattern(const sparsed_shape* shape, const sparsed_
   // With few enough blocks per row the pooled-scoring kernel ranks each block-row in its own
   // tail; A' then goes to memory only if the caller asked for it.
   const bool fused = score_ranks_in_kernel(nb, params->block_size);
-  // Up to 128 key blocks per row it also needs no log-sum-exp pass before it (one exponential per logit instead of
+  // Up to 512 key blocks per row it also needs no log-sum-exp pass before it (one exponential per logit instead of
   // two). The workspace asked for is that of the longest route either way.
   const bool one_pass = lse_or_null == nullptr && score_in_one_pass(nb);
   const size_t bh = static_cast<size_t>(shape->batch) * shape->heads_q;

@@ -9,13 +9,16 @@
 //   * kOnePass  the row sums of every key block are kept, relative to a per-row reference that is fixed with the
 //               first tile, until the row's denominator is known; then they are divided by it and summed over the
 //               rows of each query block. One fp32 per row and key block, in the tensor-memory columns that the
-//               two logit buffers leave free: 128 of them, so up to 128 key blocks per row.
+//               two logit buffers leave free: 128 of a CTA's 256, so up to 128 key blocks per row.
+//   * kOnePassWide  the same with one CTA per SM and all of its tensor memory: up to 384 key blocks per row. Half
+//               as many softmax warps keep the exponential unit less busy, but there is one pass instead of two.
+//   * kOnePassMost  ... and 128 more sums in 64 KB of shared memory: up to 512 (4 % slower for telling them apart).
 //   * kPooled   the caller (or a kRowStats pass) has the rows' log-sum-exp: p = exp(s - LSE) is the probability
 //               itself, and the block sums are folded into A' whenever 128 of them have come together.
-//   * kRowStats log-sum-exp of every row: the first of the two passes that rows with more than 128 key blocks
+//   * kRowStats log-sum-exp of every row: the first of the two passes that rows with more than 512 key blocks
 //               take.
 //
-// Pipeline per CTA (320 threads, two CTAs per SM): warp 8 streams 64-key K tiles by TMA into a ring of four, warp 9
+// Pipeline per CTA (320 threads, two CTAs per SM but for kOnePassWide / Most): warp 8 streams 64-key K tiles by TMA into a ring of four, warp 9
 // issues S = Q K^T (one commit per tile: "S ready" for the softmax warps, "slot free" for the producer), warps 0-3 and
 // 4-7 are two groups with one thread per query row each. The groups take turns at 128 keys (two tiles), so that a key
 // block belongs to one of them; each has one S buffer, its own row references and its own denominators, which meet at
@@ -28,7 +31,8 @@
 // Measured on B200, from Q and K alone (two passes over the logits before, with two CTAs of four softmax warps):
 //   28 heads x 16384 tokens, block 128   6.21 -> 2.50 ms (kOnePass; exponential unit busy 82 % of the time)
 //   32 heads x 8192 tokens, block 128    1.79 -> 0.73 ms (kOnePass)
-//   8 heads x 65536 tokens, block 128    27.5 -> 22.0 ms (kRowStats + kPooled)
+//   28 heads x 16384 tokens, block 64    6.26 -> 3.53 ms (kOnePassWide; in two passes 5.0)
+//   8 heads x 65536 tokens, block 128    27.5 -> 15.9 ms (kOnePassMost; in two passes 22.3)
 #include "internal.h"
 #include "softmax_pipeline.cuh"
 #include "topk_device.cuh"
@@ -41,27 +45,32 @@ constexpr int kTileM = 128;     // query rows per CTA
 constexpr int kTileN = 64;      // keys per pipeline step
 constexpr int kThreads = 320;
 constexpr int kSlots = 4;       // 16 KB ring slots, one K tile each
-constexpr int kTmemCols = 256;
-constexpr int kColStat = 128;   // columns 0-127: one S buffer per group; 128-255: one block sum per column and row
-constexpr int kChunk = 128;     // block sums held per row
+constexpr int kColStat = 128;   // columns 0-127: one S buffer per group; from 128 on: one block sum per column and row
 constexpr int kMaxKeys = 2048;  // ranking keys held in shared memory: (block-rows per tile) x (key blocks per row)
 
-enum ScoreMode { kOnePass, kPooled, kRowStats };
+enum ScoreMode { kOnePass, kOnePassWide, kOnePassMost, kPooled, kRowStats };
+__host__ __device__ constexpr bool one_per_sm(int mode) { return mode == kOnePassWide || mode == kOnePassMost; }
+__host__ __device__ constexpr int tmem_cols(int mode) { return one_per_sm(mode) ? 512 : 256; }
+__host__ __device__ constexpr int tmem_sums(int mode) { return tmem_cols(mode) - kColStat; }     // block sums held per row in tensor memory
+__host__ __device__ constexpr int smem_sums(int mode) { return mode == kOnePassMost ? 128 : 0; }   // ... in shared memory
+__host__ __device__ constexpr int block_sums(int mode) { return tmem_sums(mode) + smem_sums(mode); }
 
 // A row's reference is the maximum of its first 32 logits and stays until a sum outgrows this: only fp32 sums are taken
 // here (no bf16 probabilities), so 2^60 is as safe as 1, and what an outgrown reference would lose at the other end of
 // the fp32 range is below 2^-66 of the row's sum.
 constexpr float kOutgrown = 1152921504606846976.f;   // 2^60
 
+template <int kMode>
 struct ScoreSmem {
   alignas(1024) __nv_bfloat16 q[2][kTileM * 64];           // two 64-wide halves of head_dim
   alignas(1024) __nv_bfloat16 k[kSlots][2][kTileN * 64];   // each slot: two 64-wide halves of head_dim
   uint32_t keys[kMaxKeys];          // ordered keys of this CTA's block-row(s)
-  float quarter[4][kChunk];         // block sums over each 32-row quarter of the tile
+  float quarter[4][block_sums(kMode)];   // block sums over each 32-row quarter of the tile
   int hist[4][256];                 // one histogram per ranking warp
   uint64_t q_full, k_full[kSlots];
   uint64_t done[kSlots];            // the MMAs that read the slot have completed: S of that tile is ready
   uint64_t s_free[2];               // every warp of the group has copied its rows of the S buffer into registers
+  float more[smem_sums(kMode) > 0 ? smem_sums(kMode) : 1][kTileM];   // block sums beyond those in tensor memory
   float2 ml[2][kTileM];             // each group's (reference, denominator) of each row
   uint32_t tmem_base;
   int abort_flag;
@@ -87,16 +96,6 @@ __device__ __forceinline__ float warp_column_sums(float (&v)[32], int lane) {
   return v[0];
 }
 
-// Block sums of one row in n columns at t_stat times alpha.
-__device__ __noinline__ void rescale_block_sums(uint32_t t_stat, int n, float alpha) {
-  for (int c = 0; c < n; ++c) {
-    uint32_t r;
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(r) : "r"(t_stat + c) : "memory");
-    tmem_wait_ld();
-    tmem_st1(t_stat + c, __uint_as_float(r) * alpha);
-  }
-}
-
 // Sum of 2^(scale * s - m) over 32 columns.
 __device__ __forceinline__ float exp_sum(const uint32_t (&r)[32], float scale_log2, float m) {
   const float2 sc = make_float2(scale_log2, scale_log2);
@@ -114,10 +113,13 @@ __device__ __forceinline__ float exp_sum(const uint32_t (&r)[32], float scale_lo
 }
 
 template <int kMode>
-__global__ void __launch_bounds__(kThreads, 2)
+__global__ void __launch_bounds__(kThreads, one_per_sm(kMode) ? 1 : 2)
 score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k, const ScoreParams p) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
-  ScoreSmem& sm = *reinterpret_cast<ScoreSmem*>(smem_raw);
+  ScoreSmem<kMode>& sm = *reinterpret_cast<ScoreSmem<kMode>*>(smem_raw);
+  constexpr int kTmemCols = tmem_cols(kMode);
+  constexpr int kChunk = block_sums(kMode);
+  constexpr bool kKeepsSums = kMode == kOnePass || one_per_sm(kMode);
   wait_for_previous_kernel();
   if ((smem_u32(smem_raw) & 1023u) != 0u) {
     if (threadIdx.x == 0 && atomicCAS(&p.status->code, 0, 2) == 0) p.status->where = 2;
@@ -230,6 +232,14 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
       m = row_valid ? p.lse[static_cast<int64_t>(bh) * p.seq_len + row] * 1.44269504088896341f : INFINITY;
     }
 
+    // this row's sum over key block jb0 + col
+    auto put_sum = [&](int col, float v) {
+      if (smem_sums(kMode) == 0 || col < tmem_sums(kMode)) {
+        tmem_st1(t_stat + col, v);
+      } else {
+        sm.more[col - tmem_sums(kMode)][rit] = v;
+      }
+    };
     // Block sums held in tensor memory (columns of key blocks [jb0, jb0 + n)) times the row's weight in the group that
     // summed them, then summed over the rows of each query block: A' to memory and / or to the ranking keys. All eight
     // warps, in step.
@@ -241,8 +251,13 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
       for (int c = 32 * g; c < n; c += 64) {
         uint32_t r[32];
         float v[32];
-        tmem_ld32(t_stat + c, r);
-        tmem_wait_ld();
+        if (smem_sums(kMode) == 0 || c < tmem_sums(kMode)) {
+          tmem_ld32(t_stat + c, r);
+          tmem_wait_ld();
+        } else {
+#pragma unroll
+          for (int j = 0; j < 32; ++j) r[j] = __float_as_uint(sm.more[c + j - tmem_sums(kMode)][rit]);
+        }
 #pragma unroll
         for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]) * ((((c + j) * bs) & 128) != 0 ? w1 : w0);
         sm.quarter[wq][c + lane] = warp_column_sums(v, lane);   // columns at and beyond n are not used below
@@ -250,15 +265,15 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
       tc_fence_before();
       named_barrier_sync(1, 2 * kTileM);
       tc_fence_after();
-      if (tid < n) {
-        const float q0 = sm.quarter[0][tid], q1 = sm.quarter[1][tid], q2 = sm.quarter[2][tid], q3 = sm.quarter[3][tid];
+      for (int c = tid; c < n; c += 2 * kTileM) {
+        const float q0 = sm.quarter[0][c], q1 = sm.quarter[1][c], q2 = sm.quarter[2][c], q3 = sm.quarter[3][c];
         float score[4] = {q0, q1, q2, q3};
         if (bs == 128) score[0] = (q0 + q1) + (q2 + q3);
         if (bs == 64) {
           score[0] = q0 + q1;
           score[1] = q2 + q3;
         }
-        const int jb = jb0 + tid;
+        const int jb = jb0 + c;
 #pragma unroll
         for (int rh = 0; rh < 4; ++rh) {
           const int ib = q_tile * rows_here + rh;
@@ -309,11 +324,22 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
           const float ref = m == -INFINITY ? 0.f : m;
           s0 = exp_sum(r0, scale_log2, ref);
           s1 = exp_sum(r1, scale_log2, ref);
-          if constexpr (kMode == kOnePass) {
+          if constexpr (kKeepsSums) {
             carry *= alpha;
             // (columns of the other group are left alone; its threads rescale theirs)
             asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-            for (int s = g; s <= (t >> 1); s += 2) rescale_block_sums(t_stat + (s * 128) / bs, 128 / bs, alpha);
+            const int per_span = 128 / bs;
+            for (int s = g; s <= (t >> 1); s += 2)
+              for (int c = s * per_span; c < (s + 1) * per_span; ++c) {
+                if (smem_sums(kMode) == 0 || c < tmem_sums(kMode)) {
+                  uint32_t r;
+                  asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(r) : "r"(t_stat + c) : "memory");
+                  tmem_wait_ld();
+                  tmem_st1(t_stat + c, __uint_as_float(r) * alpha);
+                } else {
+                  sm.more[c - tmem_sums(kMode)][rit] *= alpha;
+                }
+              }
           }
         }
         l += s0 + s1;
@@ -324,13 +350,13 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
           if ((t & 1) == 0) {
             carry = s0 + s1;
           } else {
-            tmem_st1(t_stat + col, carry + (s0 + s1));
+            put_sum(col, carry + (s0 + s1));
           }
         } else if (bs == 64) {
-          tmem_st1(t_stat + col, s0 + s1);
+          put_sum(col, s0 + s1);
         } else {
-          tmem_st1(t_stat + col, s0);
-          tmem_st1(t_stat + col + 1, s1);   // (beyond the last block if their number is odd: not folded)
+          put_sum(col, s0);
+          put_sum(col + 1, s1);   // (beyond the last block if their number is odd: not folded)
         }
         if constexpr (kMode == kPooled) {
           // 128 blocks are bs spans of 128 keys: bs / 2 spans, bs tiles of each group
@@ -389,21 +415,23 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
 template <int kMode>
 cudaError_t launch(const CUtensorMap& tq, const CUtensorMap& tk, const ScoreParams& p, int batch, cudaStream_t stream) {
   auto kernel = score_kernel<kMode>;
-  const int smem = static_cast<int>(sizeof(ScoreSmem));
-  static_assert(sizeof(ScoreSmem) <= 113 * 1024, "two CTAs per SM");
+  static_assert(sizeof(ScoreSmem<kMode>) <= (kMode == kOnePassMost ? 227 : kMode == kOnePassWide ? 120 : 113) * 1024,
+                "two CTAs per SM, or one");
+  // (one per SM: more than half of its shared memory, so that two CTAs never compete for its tensor memory)
+  const int smem = kMode == kOnePassWide ? 120 * 1024 : static_cast<int>(sizeof(ScoreSmem<kMode>));
   static SmemLimit limit;  // per template instantiation
   cudaError_t e = ensure_dynamic_smem(kernel, smem, limit);
   if (e != cudaSuccess) return e;
   const int num_q_tiles = (p.seq_len + kTileM - 1) / kTileM;
   const long long ctas = static_cast<long long>(batch) * p.heads_q * num_q_tiles;
   if (ctas <= 0) return cudaSuccess;
-  return launch_overlapped(kernel, ctas, p.max_ctas, kThreads, smem, stream, tq, tk, p);
+  return launch_overlapped(kernel, ctas, one_per_sm(kMode) ? p.max_ctas / 2 : p.max_ctas, kThreads, smem, stream, tq, tk, p);
 }
 
 }  // namespace
 
 bool score_ranks_in_kernel(int nb, int block_size) { return nb * (kTileM / block_size) <= kMaxKeys; }
-bool score_in_one_pass(int nb) { return nb <= kChunk; }
+bool score_in_one_pass(int nb) { return nb <= block_sums(kOnePassMost); }
 
 cudaError_t launch_row_stats(const CUtensorMap& tq, const CUtensorMap& tk, const ScoreParams& p, int batch,
                              cudaStream_t stream) {
@@ -412,7 +440,11 @@ cudaError_t launch_row_stats(const CUtensorMap& tq, const CUtensorMap& tk, const
 
 cudaError_t launch_pooled_scores(const CUtensorMap& tq, const CUtensorMap& tk, const ScoreParams& p, int batch,
                                  cudaStream_t stream) {
-  return p.lse == nullptr ? launch<kOnePass>(tq, tk, p, batch, stream) : launch<kPooled>(tq, tk, p, batch, stream);
+  if (p.lse != nullptr) return launch<kPooled>(tq, tk, p, batch, stream);
+  const int nb = p.seq_len / p.block_size;
+  if (nb <= block_sums(kOnePass)) return launch<kOnePass>(tq, tk, p, batch, stream);
+  if (nb <= block_sums(kOnePassWide)) return launch<kOnePassWide>(tq, tk, p, batch, stream);
+  return launch<kOnePassMost>(tq, tk, p, batch, stream);
 }
 
 }  // namespace sparsed

@@ -1,5 +1,5 @@
-"""Selection from Q and K: the one-pass route (up to 128 key blocks per row), the two-pass route beyond it, and the
-route with the caller's LSE, at the sizes where one ends and the next begins and on ragged query and key tiles."""
+"""Selection from Q and K: the one-pass routes (up to 128 and up to 512 key blocks per row), the two-pass route beyond
+them, and the route with the caller's LSE, at the sizes where one ends and the next begins and on ragged query and key tiles."""
 import numpy as np
 import pytest
 import torch
@@ -29,7 +29,8 @@ def check(q, k, bs, rho, p, lse=None):
 @pytest.mark.parametrize("bs,nb,Hq,Hkv,batch,p_blocks", [
     (32, 1, 1, 1, 1, 0), (32, 3, 2, 1, 2, 1), (32, 127, 1, 1, 1, 60), (32, 128, 2, 2, 1, 0), (32, 129, 1, 1, 1, 7),
     (64, 1, 2, 2, 1, 0), (64, 5, 4, 2, 1, 2), (64, 128, 1, 1, 1, 31), (64, 129, 1, 1, 1, 0),
-    (128, 1, 1, 1, 1, 0), (128, 3, 3, 1, 2, 1), (32, 513, 1, 1, 1, 200)])
+    (128, 1, 1, 1, 1, 0), (128, 3, 3, 1, 2, 1), (32, 383, 1, 1, 1, 100), (32, 385, 1, 1, 1, 9), (32, 511, 1, 1, 1, 0), (32, 512, 1, 1, 1, 77),
+    (64, 200, 2, 1, 1, 64), (32, 513, 1, 1, 1, 200)])
 def test_every_route_at_its_ends(bs, nb, Hq, Hkv, batch, p_blocks):
     cfg = syn.AttnConfig("routes", batch, Hq, Hkv, nb * bs, 128, bs, 0.3, p_blocks * bs, seed=71, plant_norm=6.0)
     q, k, v = syn.make_qkv(cfg, DEV)
@@ -52,20 +53,19 @@ def test_more_than_128_blocks_of_128_keys_sampled():
     np.testing.assert_array_equal(col_idx.cpu().numpy(), ci)
 
 
-@pytest.mark.parametrize("bs", [32, 128])
-def test_logits_that_outgrow_the_rows_reference(bs):
+@pytest.mark.parametrize("bs,L", [(32, 1024), (128, 1024), (32, 6016), (32, 16384)])
+def test_logits_that_outgrow_the_rows_reference(bs, L):
     """The reference of a row is its first tile's maximum until a sum passes 2^60: here the logits of half the rows
     rise by about 2^100 between the first and later keys (more than once for some), those of the others fall."""
-    L = 1024
     g = torch.Generator(device=DEV).manual_seed(73)
     q = torch.randn(1, 1, L, 128, generator=g, device=DEV) * 0.05
     k = torch.randn(1, 1, L, 128, generator=g, device=DEV) * 0.05
     u = torch.randn(128, generator=g, device=DEV)
     u = u / u.norm()
     level = torch.zeros(L, device=DEV)
-    level[200:], level[500:] = 28.0, 56.0
+    level[200:], level[L // 2:], level[-500:] = 28.0, 42.0, 56.0
     q += 28.0 * u * torch.where(torch.arange(L, device=DEV) % 2 == 0, 1.0, -1.0)[None, None, :, None]
-    k += u * level[None, None, :, None]      # scaled logits 28 * level / sqrt(128): 0, 69, 139 (base e)
+    k += u * level[None, None, :, None]      # scaled logits 28 * level / sqrt(128): 0, 69, 104, 139 (base e)
     q, k = q.bfloat16(), k.bfloat16()
     # fp32 logits of up to 139 are known to 2^-17 here (six more binades than those SCORE_RTOL is stated for)
     _, _, _, scores = gpu_select(q, k, bs, 0.3, 0)
