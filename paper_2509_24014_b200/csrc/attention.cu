@@ -88,8 +88,8 @@ constexpr int kIdBits = 11;
 static_assert((1 << kIdBits) == kMaxPackedBlocks, "ids of union entries");
 
 // kDense: walk every key tile of the sequence (kBlock must be 128 then; no block lists are read).
-// kOverlap: launched with launch_overlapped. (Of the dense walk there are both kinds: with the wait at its start the
-// compiler arranges its main loop differently, and long launches take 1.4 % longer.)
+// kOverlap: launched with launch_overlapped. (Of the unpacked walks there are both kinds: with the wait at its start the
+// compiler arranges the main loop differently, and long launches take 1.4 % longer, dense, or 0.4 %, 128-key blocks.)
 template <int kBlock, bool kDense, bool kOverlap>
 __global__ void __launch_bounds__(kThreads, 2)
 attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
@@ -124,8 +124,8 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
   //   128-key blocks: blockIdx.x, blockIdx.x + gridDim.x, ...; as many CTAs as fit on the device. A selected
   //     pattern's lists are equally long, so that is balanced.
   //   64- and 32-key blocks: unions differ in length by up to 1 : 4, so the grid has one CTA per item and a CTA that
-  //     runs takes over CTAs that have not been launched yet (cluster launch control), one item ahead. Against equal
-  //     shares: 1450 -> 1390 us for 8 x 32 heads x 4096 tokens, block 32, half kept; 8.64 -> 8.06 ms for 32 x 65536,
+  //     runs takes over CTAs that have not been launched yet (cluster launch control), late in the
+  //     item before. Against equal shares: 1450 -> 1390 us for 8 x 32 heads x 4096 tokens, block 32, half kept; 8.64 -> 8.06 ms for 32 x 65536,
   //     block 64. (With 128-key blocks it was 1 % slower than equal shares.)
   struct Item {
     int q_tile, bh, head, batch, kv_head, q_row0, groups_here, r0;
@@ -295,7 +295,6 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
     }
     __syncwarp();
     if constexpr (kPacked) {
-      request_item();
       first_entries = build_union(cur, 0);
       publish(0, first_item, first_entries);
       if (first_entries > 0) issue_q_load(cur);
@@ -342,7 +341,7 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
     bool ok = true;
     int load0 = 0;       // K/V loads issued for earlier items
     int q_tiles_done = 0;  // earlier items that had keys (each loaded a Q tile and staged an output tile)
-    [[maybe_unused]] int requests = 0;   // answers of the launch control that have been followed by a request
+    [[maybe_unused]] int requests = 0;   // made to the launch control
     for (int nth = 0; ok; ++nth) {       // the CTA's nth item; packed: in item buffer nth & 1
       // The Q buffer doubles as the staging tile of the previous output: the next Q may land once the softmax
       // warps have had that output read out of it (which is after the item's last MMA). The first ring-full of
@@ -365,8 +364,6 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
             publish(nth & 1, -1, 0);
             break;
           }
-          request_item();
-          ++requests;
           cur = describe(item, true);
           n_entries = build_union(cur, nth & 1);
           publish(nth & 1, item, n_entries);
@@ -394,11 +391,27 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
       };
       const int num_tiles = kPacked ? union_tiles(n_entries) : unpacked_tiles(cur);
       const int q_at = min(2 * num_tiles, kSlots);
+      // The next item is asked for two tiles before this one's last load: late enough that a CTA with a long union does
+      // not hold an item that another could have started (asked for at once, 1.7 items per CTA took 12 % longer than
+      // with one item per CTA), early enough for the answer to be there.
+      [[maybe_unused]] const int request_at = max(2 * num_tiles - 4, nth == 0 ? loads_issued : 0);
+      if constexpr (kPacked) {
+        if (request_at >= 2 * num_tiles) {
+          request_item();
+          ++requests;
+        }
+      }
       // load i: K (even) or V (odd) of tile i / 2; a slot is reused every kSlots loads
       for (int i = (nth == 0 ? loads_issued : 0); ok && i < 2 * num_tiles; ++i) {
         if (q_pending && i == q_at && !settle_q()) {
           ok = false;
           break;
+        }
+        if constexpr (kPacked) {
+          if (i == request_at) {
+            request_item();
+            ++requests;
+          }
         }
         const int t = i >> 1;
         int kv_row0, kv_row1 = 0;
@@ -433,8 +446,8 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
     }
     if constexpr (kPacked) {
       // given up: the launch control's answer must not arrive after the CTA has left (bounded like every wait)
-      for (uint32_t i = 0; !ok && i < kSpinLimit; ++i)
-        if (mbar_try_wait(&sm.control_full, requests & 1)) break;
+      for (uint32_t i = 0; !ok && requests > 0 && i < kSpinLimit; ++i)
+        if (mbar_try_wait(&sm.control_full, (requests - 1) & 1)) break;
     }
   } else if (warp == 5) {
     // =============================== UMMA issuer ========================================
@@ -712,7 +725,9 @@ int attn_sparse_max_blocks(int block_size) { return block_size < kTileM ? kMaxPa
 // p.num_q_tiles = ceil(seq_len / 128), p.num_blocks = seq_len / block_size.
 cudaError_t launch_attn_sparse(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv,
                                const CUtensorMap& to, const AttnParams& p, int block_size, cudaStream_t stream) {
-  if (block_size == 128) return launch<128, false, true>(tq, tk, tv, to, p, stream);
+  if (block_size == 128)
+    return p.num_items <= p.max_ctas ? launch<128, false, true>(tq, tk, tv, to, p, stream)
+                                     : launch<128, false, false>(tq, tk, tv, to, p, stream);
   if (block_size == 64) return launch<64, false, true>(tq, tk, tv, to, p, stream);
   return launch<32, false, true>(tq, tk, tv, to, p, stream);
 }
