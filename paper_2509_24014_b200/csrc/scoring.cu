@@ -55,10 +55,20 @@ __host__ __device__ constexpr int tmem_sums(int mode) { return tmem_cols(mode) -
 __host__ __device__ constexpr int smem_sums(int mode) { return mode == kOnePassMost ? 128 : 0; }   // ... in shared memory
 __host__ __device__ constexpr int block_sums(int mode) { return tmem_sums(mode) + smem_sums(mode); }
 
-// A row's reference is the maximum of its first 32 logits and stays until a sum outgrows this: only fp32 sums are taken
-// here (no bf16 probabilities), so 2^60 is as safe as 1, and what an outgrown reference would lose at the other end of
-// the fp32 range is below 2^-66 of the row's sum.
+// A row's reference, one in each group, is the maximum of the group's first 64-key tile and stays until the sum of a later
+// tile outgrows this: only fp32 sums are taken here (no bf16 probabilities), so 2^60 is as safe as 1. Sums may thus stand
+// up to 2^66 above their reference, which is why they are brought to another one in two steps (PowerOfTwo).
 constexpr float kOutgrown = 1152921504606846976.f;   // 2^60
+
+// 2^e as a product of two factors, each well inside the fp32 range: a sum of 2^60 brought down by 2^-150 is 2^-90, while
+// 2^-150 by itself is zero. far is 1 or 2^-64, so that nothing is rounded by applying it.
+struct PowerOfTwo {
+  float far, near;
+};
+__device__ __forceinline__ PowerOfTwo power_of_two(float e) {
+  const bool low = e < -32.f;   // (2^-32 divided by the largest denominator, 2^76, is still a normal number)
+  return {low ? 0x1p-64f : 1.f, fast_exp2(low ? e + 64.f : e)};
+}
 
 template <int kMode>
 struct ScoreSmem {
@@ -240,10 +250,10 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
         sm.more[col - tmem_sums(kMode)][rit] = v;
       }
     };
-    // Block sums held in tensor memory (columns of key blocks [jb0, jb0 + n)) times the row's weight in the group that
-    // summed them, then summed over the rows of each query block: A' to memory and / or to the ranking keys. All eight
-    // warps, in step.
-    auto fold = [&](int jb0, int n, float w0, float w1) {
+    // Block sums held in tensor memory (columns of key blocks [jb0, jb0 + n)) times the row's weight (both factors) in the
+    // group that summed them, then summed over the rows of each query block: A' to memory and / or to the ranking keys. All
+    // eight warps, in step.
+    auto fold = [&](int jb0, int n, PowerOfTwo w0, PowerOfTwo w1) {
       asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
       tc_fence_before();
       named_barrier_sync(1, 2 * kTileM);
@@ -259,7 +269,10 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
           for (int j = 0; j < 32; ++j) r[j] = __float_as_uint(sm.more[c + j - tmem_sums(kMode)][rit]);
         }
 #pragma unroll
-        for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]) * ((((c + j) * bs) & 128) != 0 ? w1 : w0);
+        for (int j = 0; j < 32; ++j) {
+          const bool second = (((c + j) * bs) & 128) != 0;
+          v[j] = __uint_as_float(r[j]) * (second ? w1.far : w0.far) * (second ? w1.near : w0.near);
+        }
         sm.quarter[wq][c + lane] = warp_column_sums(v, lane);   // columns at and beyond n are not used below
       }
       tc_fence_before();
@@ -317,15 +330,15 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
 #pragma unroll
           for (int c = 0; c < 32; ++c) mx = fmaxf(mx, fmaxf(__uint_as_float(r0[c]), __uint_as_float(r1[c])));
           const float m_new = outgrown ? fmaxf(m, mx * scale_log2) : m;
-          const float alpha = m_new > m ? fast_exp2(m - m_new) : 1.f;
+          const PowerOfTwo alpha = power_of_two(m_new > m ? m - m_new : 0.f);
           m = m_new;
-          l *= alpha;
+          l *= alpha.far * alpha.near;
           // a row whose logits so far are all -inf: 2^(-inf - 0) = 0, not NaN
           const float ref = m == -INFINITY ? 0.f : m;
           s0 = exp_sum(r0, scale_log2, ref);
           s1 = exp_sum(r1, scale_log2, ref);
           if constexpr (kKeepsSums) {
-            carry *= alpha;
+            carry = carry * alpha.far * alpha.near;
             // (columns of the other group are left alone; its threads rescale theirs)
             asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
             const int per_span = 128 / bs;
@@ -335,9 +348,10 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
                   uint32_t r;
                   asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(r) : "r"(t_stat + c) : "memory");
                   tmem_wait_ld();
-                  tmem_st1(t_stat + c, __uint_as_float(r) * alpha);
+                  tmem_st1(t_stat + c, __uint_as_float(r) * alpha.far * alpha.near);
                 } else {
-                  sm.more[c - tmem_sums(kMode)][rit] *= alpha;
+                  float& sum = sm.more[c - tmem_sums(kMode)][rit];
+                  sum = sum * alpha.far * alpha.near;
                 }
               }
           }
@@ -361,7 +375,7 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
         if constexpr (kMode == kPooled) {
           // 128 blocks are bs spans of 128 keys: bs / 2 spans, bs tiles of each group
           if ((j + 1) % bs == 0) {
-            fold(jb0, min(kChunk, nb - jb0), 1.f, 1.f);
+            fold(jb0, min(kChunk, nb - jb0), {1.f, 1.f}, {1.f, 1.f});
             jb0 += kChunk;
           }
         }
@@ -369,20 +383,20 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
     }
     if (*reinterpret_cast<volatile int*>(&sm.abort_flag) != 0) ok = false;
     // the two groups' references and denominators of a row meet
-    float w0 = 1.f, w1 = 1.f;
+    PowerOfTwo w0 = {1.f, 1.f}, w1 = {1.f, 1.f};
     if constexpr (kMode != kPooled) {
       sm.ml[g][rit] = make_float2(m, l);
       named_barrier_sync(1, 2 * kTileM);
       const float2 a = sm.ml[0][rit], b = sm.ml[1][rit];
       const float top = fmaxf(a.x, b.x);
-      const float f0 = fast_exp2(a.x - top), f1 = fast_exp2(b.x - top);
-      const float denom = a.y * f0 + b.y * f1;
+      const PowerOfTwo f0 = power_of_two(a.x - top), f1 = power_of_two(b.x - top);
+      const float denom = a.y * f0.far * f0.near + b.y * f1.far * f1.near;
       if constexpr (kMode == kRowStats) {
         if (ok && g == 0 && row_valid)
           p.lse_out[static_cast<int64_t>(bh) * p.seq_len + row] = (top + log2f(denom)) * 0.69314718055994531f;
       }
-      w0 = row_valid ? f0 / denom : 0.f;
-      w1 = row_valid ? f1 / denom : 0.f;
+      w0 = {f0.far, row_valid ? f0.near / denom : 0.f};
+      w1 = {f1.far, row_valid ? f1.near / denom : 0.f};
     }
     if constexpr (kMode != kRowStats) {
       if (nb > jb0) fold(jb0, min(kChunk, nb - jb0), w0, w1);

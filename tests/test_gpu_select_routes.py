@@ -71,3 +71,31 @@ def test_logits_that_outgrow_the_rows_reference(bs, L):
     _, _, _, scores = gpu_select(q, k, bs, 0.3, 0)
     ref = orc.pooled_scores(to_f64(q), to_f64(k), bs)
     np.testing.assert_allclose(scores.cpu().numpy(), ref, rtol=16 * SCORE_RTOL, atol=1e-7)
+
+
+@pytest.mark.parametrize("bs,spans,levels", [
+    # one group's reference lies far below the other's, its sums above its reference
+    (128, 16, {0: -140, 1: 0, 2: -100, 3: -80, 14: -90}), (32, 16, {0: -140, 1: 0, 2: -100, 3: -80, 14: -90}),
+    (64, 190, {0: -140, 1: 0, 2: -100, 3: -80, 188: -90}), (128, 400, {0: -140, 1: 0, 2: -100, 3: -80, 398: -90}),
+    # a group's reference moves by more than fp32's exponents reach below one
+    (128, 16, {0: -140, 2: -100, 4: 0, 6: -110}), (32, 16, {0: -140, 2: -100, 4: 0, 6: -110}),
+    (64, 190, {1: -140, 3: -100, 181: 0, 189: -110}), (128, 400, {0: -140, 386: -100, 396: 0, 398: -110})])
+def test_probabilities_down_to_the_end_of_fp32(bs, spans, levels):
+    """Rows whose logits (base 2) lie at a few levels, one per 128 keys: block scores down to 2^-120 keep their value and
+    their rank (everything below the levels is 2^-200, which fp32 does not hold)."""
+    L, per = spans * 128, 128 // bs
+    x = torch.full((spans,), -200.0)
+    for span, level in levels.items():
+        x[span] = level
+    q, k = torch.zeros(1, 1, L, 128, device=DEV), torch.zeros(1, 1, L, 128, device=DEV)
+    q[..., 0], k[..., 0] = 8.0, x.repeat_interleave(128).to(DEV)   # scaled logits: 1.02 times the levels
+    kept = (len(levels) - 1) * per
+    _, _, col_idx, scores = gpu_select(q.bfloat16(), k.bfloat16(), bs, kept / (spans * per), 0)
+    want = torch.tensor(sorted(s for s in levels if levels[s] != -140)).repeat_interleave(per) * per
+    want += torch.arange(per).repeat(len(levels) - 1)
+    assert torch.equal(col_idx.cpu().view(-1, kept), want.to(torch.int32).expand(spans * per, kept))
+    p = torch.softmax(x.double().repeat_interleave(per) * 8.0 / 128 ** 0.5, -1).numpy() / bs
+    p[p < 2.0 ** -120] = 0.0
+    # fp32 logits of up to 143 are known to 2^-17 (as above)
+    np.testing.assert_allclose(scores[0, 0].cpu().numpy(), np.broadcast_to(p, (spans * per,) * 2), rtol=16 * SCORE_RTOL,
+                               atol=2.0 ** -120)
