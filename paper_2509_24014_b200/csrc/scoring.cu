@@ -21,8 +21,8 @@
 // Pipeline per CTA (320 threads, two CTAs per SM but for kOnePassWide / Most): warp 8 streams 64-key K tiles by TMA into a ring of four, warp 9
 // issues S = Q K^T (one commit per tile: "S ready" for the softmax warps, "slot free" for the producer), warps 0-3 and
 // 4-7 are two groups with one thread per query row each. The groups take turns at 128 keys (two tiles), so that a key
-// block belongs to one of them; each has one S buffer, its own row references and its own denominators, which meet at
-// the end. A thread copies its row of S into registers, hands the buffer back at once, exponentiates and sums. Four
+// block belongs to one of them; each has one S buffer and its own reference and denominator of every row, which meet at the
+// end. A thread copies its row of S into registers, hands the buffer back at once, exponentiates and sums. Four
 // such warps per scheduler cover each other's waits: with two (one group per CTA, two S buffers) the first case below
 // took 2.53 ms, with the next tile's copy pipelined into the current one's exponentials as well 2.70 ms.
 // Sums run in a fixed order, so results are bitwise reproducible. When the keys of its block-row(s) fit in shared
@@ -55,9 +55,11 @@ __host__ __device__ constexpr int tmem_sums(int mode) { return tmem_cols(mode) -
 __host__ __device__ constexpr int smem_sums(int mode) { return mode == kOnePassMost ? 128 : 0; }   // ... in shared memory
 __host__ __device__ constexpr int block_sums(int mode) { return tmem_sums(mode) + smem_sums(mode); }
 
-// A row's reference, one in each group, is the maximum of the group's first 64-key tile and stays until the sum of a later
-// tile outgrows this: only fp32 sums are taken here (no bf16 probabilities), so 2^60 is as safe as 1. Sums may thus stand
-// up to 2^66 above their reference, which is why they are brought to another one in two steps (PowerOfTwo).
+// A row's reference is the maximum of both groups' first 64-key tiles, and stays until the sum of a later tile outgrows
+// this: only fp32 sums are taken here (no bf16 probabilities), so 2^60 is as safe as 1. Sums may thus stand up to 2^66
+// above their reference, which is why they are brought to another one in two steps (PowerOfTwo). Both groups start from
+// the same reference because a sum's rounding depends on it: equal key blocks then have bitwise equal scores whichever
+// group sums them, and rank by index as they should. (A group that has outgrown it goes on with one of its own.)
 constexpr float kOutgrown = 1152921504606846976.f;   // 2^60
 
 // 2^e as a product of two factors, each well inside the fp32 range: a sum of 2^60 brought down by 2^-150 is 2^-90, while
@@ -76,7 +78,10 @@ struct ScoreSmem {
   alignas(1024) __nv_bfloat16 k[kSlots][2][kTileN * 64];   // each slot: two 64-wide halves of head_dim
   uint32_t keys[kMaxKeys];          // ordered keys of this CTA's block-row(s)
   float quarter[4][block_sums(kMode)];   // block sums over each 32-row quarter of the tile
-  int hist[4][256];                 // one histogram per ranking warp
+  union {
+    int hist[4][256];               // one histogram per ranking warp
+    float first_max[2][kTileM];     // before that: the maximum of each row over each group's first tile
+  };
   uint64_t q_full, k_full[kSlots];
   uint64_t done[kSlots];            // the MMAs that read the slot have completed: S of that tile is ready
   uint64_t s_free[2];               // every warp of the group has copied its rows of the S buffer into registers
@@ -302,6 +307,26 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
     bool ok = true;
     int jb0 = 0;   // key block of column 0
     const int my_tiles = g == 0 ? tiles0 : tiles1;
+    if constexpr (kKeepsSums) {
+      // the common reference: the maximum over the first tile of either group (which the loop below copies once more)
+      float mx = -INFINITY;
+      if (my_tiles > 0) {
+        ok = mbar_wait(&sm.done[index_of(g, 0)], 0, &sm.abort_flag, p.status, 61);
+        ok = __all_sync(0xffffffffu, ok);
+        tc_fence_after();
+        uint32_t r0[32], r1[32];
+        tmem_ld32(tmem + g * kTileN + lane_base, r0);
+        tmem_ld32(tmem + g * kTileN + lane_base + 32, r1);
+        tmem_wait_ld();
+        const int valid_cols = p.seq_len - tile_of(g, 0) * kTileN;
+        if (valid_cols < kTileN) mask_columns_from(r0, r1, valid_cols);
+#pragma unroll
+        for (int c = 0; c < 32; ++c) mx = fmaxf(mx, fmaxf(__uint_as_float(r0[c]), __uint_as_float(r1[c])));
+      }
+      sm.first_max[g][rit] = mx;
+      named_barrier_sync(1, 2 * kTileM);
+      m = fmaxf(mx, sm.first_max[g ^ 1][rit]) * scale_log2;
+    }
     for (int j = 0; j < my_tiles; ++j) {
       const int i = index_of(g, j);
       const int t = tile_of(g, j);
@@ -323,7 +348,7 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
       float s0 = exp_sum(r0, scale_log2, m);
       float s1 = exp_sum(r1, scale_log2, m);
       if constexpr (kMode != kPooled) {
-        const bool outgrown = !(s0 + s1 <= kOutgrown);   // the row's first tile (m = -inf), far larger logits, or NaN
+        const bool outgrown = !(s0 + s1 <= kOutgrown);   // no reference yet (m = -inf), far larger logits, or NaN
         if (__any_sync(0xffffffffu, outgrown)) {
           // take the tile's own maximum as the reference and bring everything summed so far to it
           float mx = -INFINITY;

@@ -77,6 +77,8 @@ def test_logits_that_outgrow_the_rows_reference(bs, L):
     # one group's reference lies far below the other's, its sums above its reference
     (128, 16, {0: -140, 1: 0, 2: -100, 3: -80, 14: -90}), (32, 16, {0: -140, 1: 0, 2: -100, 3: -80, 14: -90}),
     (64, 190, {0: -140, 1: 0, 2: -100, 3: -80, 188: -90}), (128, 400, {0: -140, 1: 0, 2: -100, 3: -80, 398: -90}),
+    (128, 16, {0: -140, 1: -140, 2: -100, 3: 0, 5: -80, 14: -90}), (32, 16, {0: -140, 1: -140, 2: 0, 5: -80, 7: -90}),
+    (64, 190, {0: -140, 1: -140, 3: 0, 188: -90}), (128, 400, {0: -140, 1: -140, 2: -100, 3: -80, 397: 0, 398: -90}),
     # a group's reference moves by more than fp32's exponents reach below one
     (128, 16, {0: -140, 2: -100, 4: 0, 6: -110}), (32, 16, {0: -140, 2: -100, 4: 0, 6: -110}),
     (64, 190, {1: -140, 3: -100, 181: 0, 189: -110}), (128, 400, {0: -140, 386: -100, 396: 0, 398: -110})])
@@ -89,13 +91,25 @@ def test_probabilities_down_to_the_end_of_fp32(bs, spans, levels):
         x[span] = level
     q, k = torch.zeros(1, 1, L, 128, device=DEV), torch.zeros(1, 1, L, 128, device=DEV)
     q[..., 0], k[..., 0] = 8.0, x.repeat_interleave(128).to(DEV)   # scaled logits: 1.02 times the levels
-    kept = (len(levels) - 1) * per
+    spans_kept = sorted(s for s in levels if levels[s] != -140)
+    kept = len(spans_kept) * per
     _, _, col_idx, scores = gpu_select(q.bfloat16(), k.bfloat16(), bs, kept / (spans * per), 0)
-    want = torch.tensor(sorted(s for s in levels if levels[s] != -140)).repeat_interleave(per) * per
-    want += torch.arange(per).repeat(len(levels) - 1)
+    want = torch.tensor(spans_kept).repeat_interleave(per) * per + torch.arange(per).repeat(len(spans_kept))
     assert torch.equal(col_idx.cpu().view(-1, kept), want.to(torch.int32).expand(spans * per, kept))
     p = torch.softmax(x.double().repeat_interleave(per) * 8.0 / 128 ** 0.5, -1).numpy() / bs
     p[p < 2.0 ** -120] = 0.0
     # fp32 logits of up to 143 are known to 2^-17 (as above)
     np.testing.assert_allclose(scores[0, 0].cpu().numpy(), np.broadcast_to(p, (spans * per,) * 2), rtol=16 * SCORE_RTOL,
                                atol=2.0 ** -120)
+
+
+@pytest.mark.parametrize("bs,nb,period", [(128, 32, 3), (64, 63, 3), (32, 64, 5), (128, 160, 3), (64, 400, 7), (32, 500, 9)])
+def test_equal_key_blocks_rank_by_index(bs, nb, period):
+    """Key blocks that hold the same keys have bitwise equal scores, wherever they lie."""
+    g = torch.Generator(device=DEV).manual_seed(74)
+    q = (torch.randn(1, 2, nb * bs, 128, generator=g, device=DEV) * 2).bfloat16()
+    k = torch.randn(1, 2, period * bs, 128, generator=g, device=DEV).bfloat16().repeat(1, 1, -(-nb // period), 1)[:, :, :nb * bs]
+    _, _, col_idx, scores = gpu_select(q, k.contiguous(), bs, 0.2, 0)
+    assert torch.equal(scores, scores[..., torch.arange(nb, device=DEV) % period])
+    _, ci = orc.select_blocks(scores.cpu().numpy(), bs, 0, 0.2)
+    np.testing.assert_array_equal(col_idx.cpu().numpy(), ci)
