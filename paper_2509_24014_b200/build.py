@@ -23,7 +23,8 @@ ARCH_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a"]
 COMMON_FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC"]
 # Flags of single files. The CTA-pair dense kernel is built with denormals flushed to zero: its softmax handles
 # probabilities, for which a flushed 1e-38 is as good as the number, and the kernel measured 2-4 % faster that way
-# (8k-64k); the other kernels measured the same or slower with it and keep IEEE denormals.
+# (8k-64k); what is multiplied into the outputs keeps them (mul_keep_denormals). The other kernels measured the same or
+# slower with it and keep IEEE denormals.
 PER_FILE_FLAGS = {"attention_dense_pair.cu": ["-ftz=true"], "attention_dense_pair_split.cu": ["-ftz=true"]}
 
 

@@ -167,6 +167,14 @@ __device__ __forceinline__ bool packed_softmax_tile(uint32_t tS, bool keep0, boo
   return true;
 }
 
+// a * b with denormal results kept, whatever the file's -ftz flag says: accumulators and outputs hold multiples of V, which
+// may be as small as its type allows (probabilities and their sums need no such care).
+__device__ __forceinline__ float mul_keep_denormals(float a, float b) {
+  float y;
+  asm("mul.rn.f32 %0, %1, %2;" : "=f"(y) : "f"(a), "f"(b));
+  return y;
+}
+
 // Multiplies this thread's row of a 128-column fp32 accumulator in tensor memory by alpha.
 // The accumulator must be quiescent (every MMA that writes it has completed).
 __device__ __forceinline__ void rescale_accumulator_row(uint32_t t_acc_row, float alpha) {
@@ -176,7 +184,7 @@ __device__ __forceinline__ void rescale_accumulator_row(uint32_t t_acc_row, floa
     tmem_ld32(t_acc_row + c * 32, o);
     tmem_wait_ld();
 #pragma unroll
-    for (int j = 0; j < 32; ++j) o[j] = __float_as_uint(__uint_as_float(o[j]) * alpha);
+    for (int j = 0; j < 32; ++j) o[j] = __float_as_uint(mul_keep_denormals(__uint_as_float(o[j]), alpha));
     tmem_st32(t_acc_row + c * 32, o);
   }
 }
@@ -301,10 +309,14 @@ __device__ __forceinline__ void stage_output_row(uint32_t t_acc_row, bool have_a
 #pragma unroll
     for (int g = 0; g < 4; ++g) {
       uint4 out;
-      out.x = pack_bf16x2(__uint_as_float(r[8 * g + 0]) * inv_l, __uint_as_float(r[8 * g + 1]) * inv_l);
-      out.y = pack_bf16x2(__uint_as_float(r[8 * g + 2]) * inv_l, __uint_as_float(r[8 * g + 3]) * inv_l);
-      out.z = pack_bf16x2(__uint_as_float(r[8 * g + 4]) * inv_l, __uint_as_float(r[8 * g + 5]) * inv_l);
-      out.w = pack_bf16x2(__uint_as_float(r[8 * g + 6]) * inv_l, __uint_as_float(r[8 * g + 7]) * inv_l);
+      out.x = pack_bf16x2(mul_keep_denormals(__uint_as_float(r[8 * g + 0]), inv_l),
+                          mul_keep_denormals(__uint_as_float(r[8 * g + 1]), inv_l));
+      out.y = pack_bf16x2(mul_keep_denormals(__uint_as_float(r[8 * g + 2]), inv_l),
+                          mul_keep_denormals(__uint_as_float(r[8 * g + 3]), inv_l));
+      out.z = pack_bf16x2(mul_keep_denormals(__uint_as_float(r[8 * g + 4]), inv_l),
+                          mul_keep_denormals(__uint_as_float(r[8 * g + 5]), inv_l));
+      out.w = pack_bf16x2(mul_keep_denormals(__uint_as_float(r[8 * g + 6]), inv_l),
+                          mul_keep_denormals(__uint_as_float(r[8 * g + 7]), inv_l));
       *reinterpret_cast<uint4*>(half + (((4 * (c & 1) + g) ^ sw) << 4)) = out;
     }
   }

@@ -21,3 +21,16 @@ def test_same_bits_as_the_single_cta_kernel(Hq, Hkv, L, bs):
     o_plain, lse_plain = gpu_full(q, k, v)
     assert torch.equal(o, o_plain) and torch.equal(lse, lse_plain)
     assert torch.allclose(scores.double().sum(-1), torch.full_like(scores[..., 0], 1.0 / bs).double(), rtol=2e-5)
+
+
+@pytest.mark.parametrize("Hq,L,bs", [(2, 640, 128), (38, 512, 64), (1, 4096, 32)])
+def test_outputs_below_the_normal_range(Hq, L, bs):
+    """V around the end of bf16's exponents, with logits that rise along the keys so that accumulators are rescaled."""
+    q, k, v = syn.make_qkv(syn.AttnConfig("tiny", 1, Hq, Hq, L, 128, bs, 0.3, 0, seed=96, plant_norm=3.0), "cuda")
+    k = (k * torch.linspace(0.0, 12.0, L, device="cuda")[:, None]).bfloat16()
+    v = (v.abs().double() * 1e-38).bfloat16()
+    o = gpu_switch_step(q, k, v, bs, 0.3, 0)[0]
+    o_plain, _ = gpu_full(q, k, v)
+    ref = torch.softmax(q.double() @ k.double().transpose(-1, -2) / 128 ** 0.5, -1) @ v.double()
+    for out in (o, o_plain):   # P in bf16 (2^-9), O in bf16: 2^-9, or half a step of 2^-133
+        assert ((out.double() - ref).abs() <= ref * 2.0 ** -7 + 2.0 ** -134).all()
