@@ -379,6 +379,9 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
                   sum = sum * alpha.far * alpha.near;
                 }
               }
+            // the loop also writes the columns that this tile is about to fill, unread: those stores come first. (Leaving
+            // those columns out instead takes 1 % longer: 32 x 4096, block 32, 206.4 against 210.2 us.)
+            asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
           }
         }
         l += s0 + s1;

@@ -113,3 +113,21 @@ def test_equal_key_blocks_rank_by_index(bs, nb, period):
     assert torch.equal(scores, scores[..., torch.arange(nb, device=DEV) % period])
     _, ci = orc.select_blocks(scores.cpu().numpy(), bs, 0, 0.2)
     np.testing.assert_array_equal(col_idx.cpu().numpy(), ci)
+
+
+@pytest.mark.parametrize("bs,tiles", [(128, 24), (64, 24), (32, 24), (128, 300), (64, 300), (64, 500), (32, 250)])
+@pytest.mark.parametrize("rises", [(1, 5, -4), (2, 7, -1), (3, -8, -5), (4, -6, -3)])
+def test_references_that_move_at_any_tile_of_a_block(bs, tiles, rises):
+    """Probabilities of 2^-200 but for three tiles of 64 keys, each 2^62 above the one before it: whatever half of a
+    block or of a pair of tiles that happens in, what was summed before is kept and what is not summed yet not touched."""
+    L, nb = tiles * 64, tiles * 64 // bs
+    x = torch.full((tiles,), -200.0)
+    for level, tile in zip((-122, -61, 0), rises):
+        x[tile] = level
+    q, k = torch.zeros(1, 1, L, 128, device=DEV), torch.zeros(1, 1, L, 128, device=DEV)
+    q[..., 0], k[..., 0] = 8.0, x.repeat_interleave(64).to(DEV)
+    _, _, _, scores = gpu_select(q.bfloat16(), k.bfloat16(), bs, 0.3, 0)
+    p = torch.softmax(x.double().repeat_interleave(64) * 8.0 / 128 ** 0.5, -1).view(nb, bs).mean(-1)
+    p[p < 2.0 ** -120] = 0.0
+    np.testing.assert_allclose(scores[0, 0].cpu().numpy(), np.broadcast_to(p.numpy(), (nb, nb)), rtol=16 * SCORE_RTOL,
+                               atol=2.0 ** -120)
