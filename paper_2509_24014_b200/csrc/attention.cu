@@ -211,12 +211,14 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
   auto build_union = [&](const Item& it, int buf) -> int {
     const int words = (p.num_blocks + 31) >> 5;
     for (int i = lane; i < kGroups * Smem::kWords; i += 32) (&sm.member[0][0])[i] = 0u;
-    int bound[kGroups];   // bound[g] = first CSR entry after query block g's list
+    // (entries are unsigned: a list may end at 2^31 - 1, and the walk steps up to 287 beyond)
+    uint32_t bound[kGroups];   // bound[g] = first CSR entry after query block g's list
 #pragma unroll
-    for (int g = 0; g < kGroups; ++g) bound[g] = __ldcg(p.row_ptr + it.r0 + min(g + 1, it.groups_here));
+    for (int g = 0; g < kGroups; ++g)
+      bound[g] = static_cast<uint32_t>(__ldcg(p.row_ptr + it.r0 + min(g + 1, it.groups_here)));
     __syncwarp();
-    const int list_end = it.list_begin + it.list_len;
-    for (int e0 = it.list_begin + lane; e0 < list_end; e0 += 8 * 32) {
+    const uint32_t list_end = static_cast<uint32_t>(it.list_begin) + static_cast<uint32_t>(it.list_len);
+    for (uint32_t e0 = static_cast<uint32_t>(it.list_begin) + lane; e0 < list_end; e0 += 8 * 32) {
       int id[8];   // eight loads in flight per lane
 #pragma unroll
       for (int u = 0; u < 8; ++u) id[u] = e0 + 32 * u < list_end ? __ldcg(p.col_idx + e0 + 32 * u) : -1;

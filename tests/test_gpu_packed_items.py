@@ -39,3 +39,22 @@ def test_ctas_that_take_over_further_tiles(bs, L, Hq, Hkv):
     scale = max(1.0, float(np.abs(ref).max()))
     check_outputs(o.float() / scale, ref / scale, f"block {bs}")
     assert (o[0, 5] == 0).all()
+
+
+@pytest.mark.parametrize("bs,kept", [(32, (1, 5, 20, 13)), (32, (7, 0, 2, 31)), (64, (3, 16)), (128, (8,))])
+def test_lists_that_end_at_the_last_index_of_32_bits(bs, kept):
+    """The lists of one query tile as the last entries of a col_idx of 2^31 - 1."""
+    L = 32 * bs
+    nb, rows, last = 32, 128 // bs, 2 ** 31 - 1
+    g = torch.Generator(device=DEV).manual_seed(82)
+    q, k, v = (torch.randn(1, 1, L, 128, generator=g, device=DEV).bfloat16() for _ in range(3))
+    ids = torch.cat([torch.randperm(nb, generator=g, device=DEV)[:n].sort().values for n in kept]).to(torch.int32)
+    ends = torch.zeros(nb + 1, dtype=torch.int64, device=DEV)
+    ends[nb - rows + 1:] = torch.tensor(kept, device=DEV).cumsum(0)     # only the last query tile keeps anything
+    row_ptr = ends.to(torch.int32)
+    want = gpu_sparse(q, k, v, sd.pattern_from_csr(row_ptr, ids, bs, nb, 1, 1))
+    col_idx = torch.empty(last, dtype=torch.int32, device=DEV)
+    col_idx[last - ids.numel():] = ids
+    row_ptr_last = (ends + (last - ids.numel())).to(torch.int32)
+    got = gpu_sparse(q, k, v, sd.pattern_from_csr(row_ptr_last, col_idx, bs, nb, 1, 1))
+    assert torch.equal(got, want) and bool((want[0, 0, -128:] != 0).any())
