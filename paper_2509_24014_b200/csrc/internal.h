@@ -35,8 +35,9 @@ inline cudaError_t ensure_dynamic_smem(Kernel kernel, int bytes, SmemLimit& lim)
 }
 
 // Launches a kernel that begins with wait_for_previous_kernel(). If the grid fits on the device at once
-// (resident_ctas; 0: not known, or not wanted), its CTAs may be started before the kernel before it in the stream has ended, which takes
-// 1.7 us off a call of 15 (2 heads x 1024 tokens, dense). Larger grids gain nothing from it and are launched as usual.
+// (resident_ctas; 0: not known, or not wanted), its CTAs may be started before the kernel before it in the stream has
+// ended, which takes 1.7 us off a call of 15 (2 heads x 1024 tokens, dense). Larger grids gain nothing from it and are
+// launched as usual. An error is returned and not left as the thread's last one, which the program around would find.
 template <class... Params, class... Args>
 inline cudaError_t launch_overlapped(void (*kernel)(Params...), long long ctas, int resident_ctas, int threads, size_t smem,
                                      cudaStream_t stream, const Args&... args) {
@@ -50,7 +51,9 @@ inline cudaError_t launch_overlapped(void (*kernel)(Params...), long long ctas, 
   attr.val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = &attr;
   cfg.numAttrs = ctas <= resident_ctas ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, kernel, args...);
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, args...);
+  if (e != cudaSuccess) (void)cudaGetLastError();
+  return e;
 }
 
 // Parameters shared by the dense and the block-sparse attention kernels.
