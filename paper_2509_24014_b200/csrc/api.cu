@@ -621,13 +621,14 @@ sparsed_status sparsed_select_pattern(const sparsed_shape* shape, const sparsed_
   // With few enough blocks per row the pooled-scoring kernel ranks each block-row in its own
   // tail; A' then goes to memory only if the caller asked for it.
   const bool fused = score_ranks_in_kernel(nb, params->block_size);
-  // Up to 512 key blocks per row it also needs no log-sum-exp pass before it (one exponential per logit instead of
-  // two). The workspace asked for is that of the longest route either way.
+  // Up to 512 key blocks per row it also needs no log-sum-exp pass before it (one exponential per logit instead of two).
   const bool one_pass = lse_or_null == nullptr && score_in_one_pass(nb);
   const size_t bh = static_cast<size_t>(shape->batch) * shape->heads_q;
   const size_t score_bytes = round_up(bh * nb * nb * 4, 256);
   const size_t lse_bytes = round_up(bh * static_cast<size_t>(shape->seq_len) * 4, 256);
-  const bool need_score_ws = (nb > 1024 || params->block_size == 32) && scores_out_or_null == nullptr;
+  // Workspace: room for A' wherever the ranking has a kernel of its own, and, as callers have always been asked for it
+  // there, with 32-key blocks and beyond 1024 blocks per row; room for the LSE unless the caller has it.
+  const bool need_score_ws = (!fused || nb > 1024 || params->block_size == 32) && scores_out_or_null == nullptr;
   const size_t required = SPARSED_STATUS_BYTES + (need_score_ws ? score_bytes : 0) + (lse_or_null ? 0 : lse_bytes);
   if ((st = check_ws(ws, ws_bytes, required)) != SPARSED_OK) return st;
   if ((st = check_arch()) != SPARSED_OK) return st;

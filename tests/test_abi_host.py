@@ -129,3 +129,22 @@ def test_missing_library_fails_loudly(monkeypatch, tmp_path):
     monkeypatch.setattr(binding._build, "LIB_PATH", str(tmp_path / "nope.so"))
     with pytest.raises(RuntimeError, match="no CPU fallback"):
         binding.load_library()
+
+
+@pytest.mark.parametrize("bs,nb,room_for_scores", [
+    (128, 8, False), (128, 1024, False), (128, 1025, True), (128, 2048, True), (128, 2049, True), (64, 1024, False),
+    (64, 1025, True), (32, 4, True), (32, 512, True), (32, 513, True)])
+@pytest.mark.parametrize("with_lse", [False, True])
+@pytest.mark.parametrize("with_scores", [False, True])
+def test_workspace_that_a_selection_asks_for(lib, bs, nb, room_for_scores, with_lse, with_scores):
+    """The smallest workspace sparsed_select_pattern takes; nothing is launched (a workspace that is large enough is refused
+    here for its alignment)."""
+    shape = sd.Shape(1, 1, 1, nb * bs, 128)
+    params = sd.make_params(bs, 0.1, 0)
+    pat = sd.Pattern(1024, 2048, 1 << 30, 0, 0, 0, 0, 0)
+    need = 256 + (-(-nb * nb * 4 // 256) * 256 if room_for_scores and not with_scores else 0)
+    need += 0 if with_lse else -(-nb * bs * 4 // 256) * 256
+    for nbytes, status in ((need - 1, 4), (need, 3)):
+        got = lib.sparsed_select_pattern(ctypes.byref(shape), ctypes.byref(params), 4096, 8192, 4096 if with_lse else None,
+                                         ctypes.byref(pat), 4096 if with_scores else None, 4096 + 4, nbytes, None)
+        assert got == status
