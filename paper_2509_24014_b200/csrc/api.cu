@@ -7,6 +7,7 @@
 #include <mutex>
 
 #include "../../include/sparsed.h"
+#include "dense_choice.h"
 #include "internal.h"
 
 namespace {
@@ -353,21 +354,9 @@ sparsed_status sparsed_workspace_init(void* ws, size_t ws_bytes, void* cuda_stre
   return e == cudaSuccess ? SPARSED_OK : cuda_fail(e);
 }
 
-// Which dense kernel runs. The pass that also records row statistics has one kernel, whose MMAs span CTA
-// pairs (attention_dense_pair.cu). For the plain pass both kernels give the same bits. Per query row the pair kernel takes
-// 3-4 % less from 4096 tokens on (it fetches each K/V tile once for 512 rows instead of once for 128, and sustained
-// launches are bound by power: 32 heads x 8192 951 -> 920 us, 8 x 32 x 4096 1956 -> 1883), below that a cluster's set-up
-// and tear-down weigh more (32 x 1900: 64.4 against 65.6). A wave of either is the same number of rows, but the last one
-// may be emptier: 8 heads x 14000 are 3.03 waves of clusters (740 us) and 2.97 of single CTAs (687). So the waves
-// are counted: a last one that is at most half full as 0.65 where its half-empty SMs run faster (two CTAs per SM, or split
-// clusters), else as 0.5 and half its share (the SMs that are busy have the power of the others). The environment variable SPARSED_DENSE_KERNEL (read once) sends every plain pass to one of them, `pair` or
-// `single`, for A/B measurements and tests.
-static double waves(long long units, long long slots, bool half_wave) {
-  const long long last = units % slots;
-  const double whole = static_cast<double>(units / slots);
-  if (last == 0) return whole;
-  return whole + (half_wave && 2 * last <= slots ? 0.65 : 0.5 + 0.5 * static_cast<double>(last) / static_cast<double>(slots));
-}
+// Which dense kernel runs. The pass that also records row statistics has one kernel, the CTA-pair one. The environment
+// variable SPARSED_DENSE_KERNEL (read once) sends every plain pass to one of them, `pair` or `single`, for A/B measurements
+// and tests.
 static bool dense_pair_kernel(bool with_stats, const sparsed_shape* shape, int max_ctas) {
   static const int forced = [] {
     const char* v = std::getenv("SPARSED_DENSE_KERNEL");
@@ -377,11 +366,7 @@ static bool dense_pair_kernel(bool with_stats, const sparsed_shape* shape, int m
   }();
   if (with_stats) return true;
   if (forced >= 0) return forced == 1;
-  if (shape->seq_len < 4096 || max_ctas < 4) return false;
-  const long long bh = static_cast<long long>(shape->batch) * shape->heads_q;
-  const long long tiles = (shape->seq_len + 127) / 128;
-  const long long clusters = bh * ((tiles + 3) / 4), pairs = max_ctas / 4;
-  return 0.965 * waves(clusters, pairs, clusters < 2 * pairs) < waves(bh * tiles, max_ctas, true);
+  return dense_pair_pays(static_cast<long long>(shape->batch) * shape->heads_q, shape->seq_len, max_ctas);
 }
 
 static sparsed_status attn_full_impl(const sparsed_shape* shape, const void* q, const void* k, const void* v, void* o,

@@ -25,6 +25,7 @@
 // tear-down barrier, and so does its peer once its own waits run out.
 #include <type_traits>
 
+#include "dense_choice.h"
 #include "internal.h"
 #include "sm100_pair_primitives.cuh"
 #include "softmax_pipeline.cuh"
@@ -402,19 +403,14 @@ cudaError_t launch_attn_dense_pair_split(const CUtensorMap& tq, const CUtensorMa
 }
 #else
 // Tensor maps: Q and O boxes 64 x 128 rows, K box 64 x 32 rows, V box 64 x 64 rows. p.num_q_tiles = ceil(seq_len / 128).
-//
-// A cluster with one stream takes 0.65-0.8 of the time of one with two. So a last wave that would leave half of the SM
-// pairs idle or more is launched as clusters of one stream each: 2 heads x 4096 tokens 63.5 -> 47.1 us, 8 x 2048
-// 36.9 -> 28.7, 2 x 1024 22.6 -> 18.4, 16 x 3072 (1.3 waves) 95.0 -> 84.4 (statistics recorded). From two full waves on the
-// launch runs into the power limit, which an emptier last wave only relieves (32 x 4096, 3.46 waves: no gain).
 cudaError_t launch_attn_dense_pair(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv,
                                    const CUtensorMap& to, const AttnParams& p, cudaStream_t stream) {
   const long long bh = p.num_q_tiles > 0 ? p.num_items / p.num_q_tiles : 0;
   const long long clusters = bh * ((p.num_q_tiles + 3) / 4);
   if (clusters <= 0) return cudaSuccess;
   const long long pairs = p.max_ctas / 4;   // SM pairs of the device (max_ctas: two CTAs per SM)
-  const long long last = pairs > 0 ? clusters % pairs : 0;
-  if (last == 0 || 2 * last > pairs || clusters >= 2 * pairs) return launch_any(tq, tk, tv, to, p, clusters, stream);
+  if (!dense_pair_splits(clusters, pairs)) return launch_any(tq, tk, tv, to, p, clusters, stream);
+  const long long last = clusters % pairs;
   AttnParams split = p;
   split.max_ctas = static_cast<int>(clusters - last);
   return launch_attn_dense_pair_split(tq, tk, tv, to, split, clusters + last, stream);
