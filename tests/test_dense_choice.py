@@ -1,5 +1,5 @@
-"""Which of the two dense kernels a plain pass goes to, on a device of 148 SMs (296 resident CTAs of the single-CTA kernel,
-74 SM pairs): the rule's own arithmetic, compiled for the host."""
+"""Which of the two dense kernels a plain pass goes to, on a device of 148 SMs (296 resident CTAs of the single-CTA
+kernel, 74 SM pairs): the rule's own arithmetic, compiled for the host."""
 import os
 import subprocess
 
@@ -7,8 +7,8 @@ import pytest
 
 from paper_2509_24014_b200 import build
 
-# heads of all batch entries, tokens, whether the CTA-pair kernel runs. Where it does not although it is the faster one under
-# sustained load, launches with rests between them lose by it.
+# heads of all batch entries, tokens, whether the CTA-pair kernel runs. Where it does not although it is the faster one
+# under sustained load, launches with rests between them lose by it.
 TABLE = [
     (1, 1024, 0), (256, 4095, 0),                                  # below 4096 tokens
     (1, 4096, 1), (4, 4096, 1), (1, 8192, 1), (1, 16384, 1),       # every cluster split

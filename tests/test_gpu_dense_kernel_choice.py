@@ -1,8 +1,8 @@
 """Both dense kernels behind sparsed_attn_full.
 
-sparsed_attn_full_stats always runs the kernel whose MMAs span CTA pairs; sparsed_attn_full runs it from 16384
-tokens on and the single-CTA kernel below that, unless SPARSED_DENSE_KERNEL=pair|single (read once per process)
-names one. The oracle parity tests of the dense pass are re-run in child processes with each setting, so that the
+sparsed_attn_full_stats always runs the kernel whose MMAs span CTA pairs; sparsed_attn_full runs it from 4096 tokens
+on where that pays (tests/test_dense_choice.py) and the single-CTA kernel elsewhere, unless
+SPARSED_DENSE_KERNEL=pair|single (read once per process) names one. The oracle parity tests of the dense pass are re-run in child processes with each setting, so that the
 pair kernel is also checked on what the statistics path never gives it (lengths that are no multiple of 32, strided
 layouts, a softmax scale, the rescaling path) and the single-CTA kernel on the long workloads."""
 import os

@@ -1,5 +1,5 @@
-"""A launch that the runtime refuses (more threads than a block may have) is reported once, by the launch helper's return
-value, and does not stay behind as the calling thread's last error, which the host program's next check would find."""
+"""A launch that the runtime refuses (more threads than a block may have) is reported once, by the launch helper's
+return value, and does not stay behind as the calling thread's last error, which the host program's next check would find."""
 import subprocess
 
 import pytest

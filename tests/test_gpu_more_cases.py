@@ -35,13 +35,13 @@ def test_custom_scale_and_batch_two_through_all_entry_points():
     kp, kg = sd.sparsed_kept_per_row(params, L)
     a_ref = orc.pooled_scores(qd, kd, 128, scale=scale32)
     results = []
-    for path in ("stats", "two_pass", "two_pass_own_lse"):
+    for path in ("stats", "given_lse", "one_pass"):
         pat, rp_t, ci_t = sd.new_pattern(B, Hq, nb, kp + kg, DEV)
         scores = torch.empty(B, Hq, nb, nb, dtype=torch.float32, device=DEV)
         if path == "stats":
             sd.sparsed_select_from_stats(q, k, params, lse, stats, pat, ws, scores_out=scores)
         else:
-            sd.sparsed_select_pattern(q, k, params, pat, ws, lse=lse if path == "two_pass" else None,
+            sd.sparsed_select_pattern(q, k, params, pat, ws, lse=lse if path == "given_lse" else None,
                                       scores_out=scores, softmax_scale=scale)
         torch.cuda.synchronize()
         np.testing.assert_allclose(scores.cpu().numpy(), a_ref, rtol=SCORE_RTOL, atol=SCORE_ATOL)
@@ -155,7 +155,7 @@ def test_token_major_layout_through_every_entry_point():
     kp, kg = sd.sparsed_kept_per_row(params, L)
     a_ref = orc.pooled_scores(qd, kd, bs)
     lists = []
-    for path in ("stats", "two_pass"):
+    for path in ("stats", "one_pass"):
         pat, rp_t, ci_t = sd.new_pattern(B, Hq, nb, kp + kg, DEV)
         scores = torch.empty(B, Hq, nb, nb, dtype=torch.float32, device=DEV)
         if path == "stats":

@@ -80,8 +80,8 @@ def gpu_switch_step_from_stats(q, k, v, block_size, keep_ratio, prefill_len):
 
 def check_sampled(cfg, q, k, v, heads, n_blocks, seed, what, via_stats=False):
     """Full, select and sparse on the GPU at full size; the oracle on sampled row blocks.
-    via_stats: select from the full pass's row statistics (the benchmarked path) instead of the
-    two-pass scorer."""
+    via_stats: select from the full pass's row statistics (the benchmarked path) instead of a Q K^T pass of
+    the scorer's own with the full pass's LSE."""
     bs, nb, pb = cfg.block_size, cfg.num_blocks, cfg.prefill_len // cfg.block_size
     group = cfg.heads_q // cfg.heads_kv
     if via_stats:
@@ -152,7 +152,7 @@ def test_config2_exhaustive():
     print({kk: float(np.mean(vv)) for kk, vv in by_kind.items()}, "rows that had to match exactly")
 
 
-@pytest.mark.parametrize("via_stats", [False, True], ids=["two_pass", "from_stats"])
+@pytest.mark.parametrize("via_stats", [False, True], ids=["given_lse", "from_stats"])
 def test_config3_gqa_sampled(via_stats):
     cfg = syn.CONFIGS["c3"]
     q, k, v = syn.make_qkv(cfg, DEV)
@@ -160,10 +160,10 @@ def test_config3_gqa_sampled(via_stats):
     assert n_rows == 28 * 4 and worst <= 2e-2
 
 
-@pytest.mark.parametrize("via_stats", [False, True], ids=["two_pass", "from_stats"])
+@pytest.mark.parametrize("via_stats", [False, True], ids=["given_lse", "from_stats"])
 def test_config4_pattern_reuse_at_64k(via_stats):
     """Pattern selected at the switch step's tensors, reused on a later step's noisy tensors; once
-    through the two-pass scorer and once through the row statistics of the full pass (1024 key tiles
+    through the scorer's own Q K^T pass with the LSE and once through the row statistics of the full pass (1024 key tiles
     per row: the path the benchmark times)."""
     cfg = syn.CONFIGS["c4"]
     s = sd.sparsed_switch_step(cfg.total_steps, cfg.skip)
@@ -190,7 +190,7 @@ def test_config4_pattern_reuse_at_64k(via_stats):
             check_outputs(o_sp[0, h, ib * bs:(ib + 1) * bs], ref, f"c4 final step h{h} ib{ib}")
 
 
-@pytest.mark.parametrize("via_stats", [False, True], ids=["two_pass", "from_stats"])
+@pytest.mark.parametrize("via_stats", [False, True], ids=["given_lse", "from_stats"])
 def test_config5_schedule_layers_sampled(via_stats):
     """Four layers of projected Q/K/V at 32k with a 16k prompt; the schedule helper drives the mode.
     The sampled query blocks include the two that straddle the prompt boundary."""

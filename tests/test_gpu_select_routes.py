@@ -1,5 +1,6 @@
-"""Selection from Q and K: the one-pass routes (up to 128 and up to 512 key blocks per row), the two-pass route beyond
-them, and the route with the caller's LSE, at the sizes where one ends and the next begins and on ragged query and key tiles."""
+"""Selection from Q and K: the one-pass routes (up to 128, 384 and 512 key blocks per row), the two-pass route beyond them
+and the route with the caller's LSE, each with rows ranked in the scoring kernel and by the kernel of its own, at the sizes
+where one ends and the next begins and on ragged query and key tiles."""
 import numpy as np
 import pytest
 import torch
@@ -29,8 +30,11 @@ def check(q, k, bs, rho, p, lse=None):
 @pytest.mark.parametrize("bs,nb,Hq,Hkv,batch,p_blocks", [
     (32, 1, 1, 1, 1, 0), (32, 3, 2, 1, 2, 1), (32, 127, 1, 1, 1, 60), (32, 128, 2, 2, 1, 0), (32, 129, 1, 1, 1, 7),
     (64, 1, 2, 2, 1, 0), (64, 5, 4, 2, 1, 2), (64, 128, 1, 1, 1, 31), (64, 129, 1, 1, 1, 0),
-    (128, 1, 1, 1, 1, 0), (128, 3, 3, 1, 2, 1), (32, 383, 1, 1, 1, 100), (32, 385, 1, 1, 1, 9), (32, 511, 1, 1, 1, 0), (32, 512, 1, 1, 1, 77),
-    (64, 200, 2, 1, 1, 64), (32, 513, 1, 1, 1, 200)])
+    (128, 1, 1, 1, 1, 0), (128, 3, 3, 1, 2, 1), (32, 383, 1, 1, 1, 100), (32, 385, 1, 1, 1, 9), (32, 511, 1, 1, 1, 0),
+    (32, 512, 1, 1, 1, 77), (64, 200, 2, 1, 1, 64), (32, 513, 1, 1, 1, 200),
+    # with the LSE one group folds its sums inside its loop and the other after it: 64 n - 1 key tiles, the last ones of
+    # group 0 alone
+    (32, 125, 1, 1, 1, 0), (32, 126, 2, 1, 1, 31), (64, 127, 1, 1, 1, 0), (32, 254, 1, 1, 1, 0), (64, 255, 1, 1, 1, 128)])
 def test_every_route_at_its_ends(bs, nb, Hq, Hkv, batch, p_blocks):
     cfg = syn.AttnConfig("routes", batch, Hq, Hkv, nb * bs, 128, bs, 0.3, p_blocks * bs, seed=71, plant_norm=6.0)
     q, k, v = syn.make_qkv(cfg, DEV)
@@ -38,6 +42,24 @@ def test_every_route_at_its_ends(bs, nb, Hq, Hkv, batch, p_blocks):
     own = check(q, k, bs, 0.3, p_blocks * bs)
     given = check(q, k, bs, 0.3, p_blocks * bs, lse=lse)
     np.testing.assert_allclose(own, given, rtol=2 * SCORE_RTOL, atol=2 * SCORE_ATOL)
+
+
+@pytest.mark.parametrize("bs,nb,p_blocks", [(64, 513, 100), (64, 1024, 0), (128, 1025, 1000)])
+def test_long_rows_ranked_in_the_scoring_kernel_sampled(bs, nb, p_blocks):
+    """More than 512 key blocks per row: a log-sum-exp pass and a pooling pass that ranks its rows itself, or the latter
+    alone with the caller's LSE."""
+    cfg = syn.AttnConfig("long rows", 1, 1, 1, nb * bs, 128, bs, 0.05, p_blocks * bs, seed=75, plant_norm=6.0)
+    q, k, v = syn.make_qkv(cfg, DEV)
+    _, lse = gpu_full(q, k, v)
+    qd, kd = to_f64(q[0, 0]), to_f64(k[0, 0])
+    for given in (None, lse):
+        _, row_ptr, col_idx, scores = gpu_select(q, k, bs, 0.05, p_blocks * bs, lse=given)
+        a = scores.cpu().numpy()
+        for ib in (0, p_blocks, nb // 2, nb - 1):
+            np.testing.assert_allclose(a[0, 0, ib], orc.head_pooled_row(qd, kd, ib, bs), rtol=SCORE_RTOL, atol=SCORE_ATOL)
+        rp, ci = orc.select_blocks(a, bs, p_blocks * bs, 0.05)
+        np.testing.assert_array_equal(row_ptr.cpu().numpy(), rp)
+        np.testing.assert_array_equal(col_idx.cpu().numpy(), ci)
 
 
 def test_more_than_128_blocks_of_128_keys_sampled():
@@ -99,17 +121,18 @@ def test_probabilities_down_to_the_end_of_fp32(bs, spans, levels):
     p = torch.softmax(x.double().repeat_interleave(per) * 8.0 / 128 ** 0.5, -1).numpy() / bs
     p[p < 2.0 ** -120] = 0.0
     # fp32 logits of up to 143 are known to 2^-17 (as above)
-    np.testing.assert_allclose(scores[0, 0].cpu().numpy(), np.broadcast_to(p, (spans * per,) * 2), rtol=16 * SCORE_RTOL,
-                               atol=2.0 ** -120)
+    np.testing.assert_allclose(scores[0, 0].cpu().numpy(), np.broadcast_to(p, (spans * per,) * 2),
+                               rtol=16 * SCORE_RTOL, atol=2.0 ** -120)
 
 
-@pytest.mark.parametrize("bs,nb,period", [(128, 32, 3), (64, 63, 3), (32, 64, 5), (128, 160, 3), (64, 400, 7), (32, 500, 9)])
+@pytest.mark.parametrize("bs,nb,period", [(128, 32, 3), (64, 63, 3), (32, 64, 5), (128, 160, 3), (64, 400, 7),
+                                          (32, 500, 9)])
 def test_equal_key_blocks_rank_by_index(bs, nb, period):
     """Key blocks that hold the same keys have bitwise equal scores, wherever they lie."""
     g = torch.Generator(device=DEV).manual_seed(74)
     q = (torch.randn(1, 2, nb * bs, 128, generator=g, device=DEV) * 2).bfloat16()
-    k = torch.randn(1, 2, period * bs, 128, generator=g, device=DEV).bfloat16().repeat(1, 1, -(-nb // period), 1)[:, :, :nb * bs]
-    _, _, col_idx, scores = gpu_select(q, k.contiguous(), bs, 0.2, 0)
+    k = torch.randn(1, 2, period * bs, 128, generator=g, device=DEV).bfloat16().repeat(1, 1, -(-nb // period), 1)
+    _, _, col_idx, scores = gpu_select(q, k[:, :, :nb * bs].contiguous(), bs, 0.2, 0)
     assert torch.equal(scores, scores[..., torch.arange(nb, device=DEV) % period])
     _, ci = orc.select_blocks(scores.cpu().numpy(), bs, 0, 0.2)
     np.testing.assert_array_equal(col_idx.cpu().numpy(), ci)

@@ -1,6 +1,6 @@
 """The switch step without a second Q K^T pass: sparsed_attn_full_stats + sparsed_select_from_stats
 against the oracle (scores within tolerance, selection logic bit-exact on the scores it produced,
-full-attention output unchanged) and against the two-pass sparsed_select_pattern."""
+full-attention output unchanged) and against sparsed_select_pattern, which makes a Q K^T pass of its own."""
 import numpy as np
 import pytest
 import torch
@@ -56,7 +56,7 @@ def test_switch_step_from_stats_matches_oracle(name, L, Hq, Hkv, bs, rho, p):
         for ib in range(nb):
             r = h * nb + ib
             check_row_list(ci[rp[r]:rp[r + 1]], a_ref[0, h, ib], pb, rho)
-    # the two-pass path agrees within the score tolerance
+    # the scorer's own pass, with the LSE, agrees within the score tolerance
     _, _, _, scores2 = gpu_select(q, k, bs, rho, p, lse=lse)
     np.testing.assert_allclose(a_gpu, scores2.cpu().numpy(), rtol=2 * SCORE_RTOL, atol=2 * SCORE_ATOL)
 
