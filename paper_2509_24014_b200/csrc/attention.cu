@@ -29,8 +29,9 @@
 //   * 64- and 32-key blocks: the 128 query rows are two / four consecutive query blocks with lists
 //     of their own. The CTA walks the UNION of those lists (built in shared memory by the producer warp, one
 //     item ahead, from one bitmap per query block) and every warp skips, per 32-column half of a tile, the key
-//     blocks its own query block did not keep: no copy out of tensor memory and no exponentials, P = 0. All 128 rows of every MMA belong to real queries, and neighbouring query blocks
-//     share the K/V tiles they have in common.
+//     blocks its own query block did not keep: no copy out of tensor memory and no exponentials, P = 0. All 128
+//     rows of every MMA belong to real queries, and neighbouring query blocks share the K/V tiles they have in
+//     common.
 #include "internal.h"
 #include "softmax_pipeline.cuh"
 
@@ -88,8 +89,9 @@ constexpr int kIdBits = 11;
 static_assert((1 << kIdBits) == kMaxPackedBlocks, "ids of union entries");
 
 // kDense: walk every key tile of the sequence (kBlock must be 128 then; no block lists are read).
-// kOverlap: launched with launch_overlapped. (Of the unpacked walks there are both kinds: with the wait at its start the
-// compiler arranges the main loop differently, and long launches take 1.4 % longer, dense, or 0.4 %, 128-key blocks.)
+// kOverlap: begins with wait_for_previous_kernel, so that small grids may be launched overlapped. (Of the dense walk there
+// are both kinds: with the wait at its start the compiler arranges the main loop differently, and long launches take
+// 1.4 % longer. 128-key blocks take the same either way: 8k 229.6 against 230.5 us, 16k 551.7 against 551.0.)
 template <int kBlock, bool kDense, bool kOverlap>
 __global__ void __launch_bounds__(kThreads, 2)
 attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
@@ -124,9 +126,10 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
   //   128-key blocks: blockIdx.x, blockIdx.x + gridDim.x, ...; as many CTAs as fit on the device. A selected
   //     pattern's lists are equally long, so that is balanced.
   //   64- and 32-key blocks: unions differ in length by up to 1 : 4, so the grid has one CTA per item and a CTA that
-  //     runs takes over CTAs that have not been launched yet (cluster launch control), late in the
-  //     item before. Against equal shares: 1450 -> 1390 us for 8 x 32 heads x 4096 tokens, block 32, half kept; 8.64 -> 8.06 ms for 32 x 65536,
-  //     block 64. (With 128-key blocks it was 1 % slower than equal shares.)
+  //     runs takes over CTAs that have not been launched yet (cluster launch control), late in the item before. Block
+  //     32, 8 x 32 heads x 4096 tokens, half kept: 1524 us with one item per CTA, 1450 with equal shares, 1439 this way;
+  //     block 64, 32 x 65536: 8.64 ms with equal shares, 8.06 this way. (With 128-key blocks it was 1 % slower than equal
+  //     shares.)
   struct Item {
     int q_tile, bh, head, batch, kv_head, q_row0, groups_here, r0;
     int list_begin, list_len;   // CSR entries of the item's query blocks; dense: key tiles of the sequence
@@ -716,7 +719,9 @@ cudaError_t launch(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorM
   if (ctas <= 0) return cudaSuccess;
   // 128-key blocks: at most as many CTAs as are resident at once, each with its share of the items
   if (kBlock == 128 && !kDense && p.max_ctas > 0 && ctas > p.max_ctas) ctas = p.max_ctas;
-  return launch_overlapped(kernel, ctas, kOverlap ? p.max_ctas : 0, kThreads, smem, stream, tq, tk, tv, to, p);
+  // (128-key blocks: as many CTAs as fit may still stand for more items)
+  const bool overlap = kOverlap && (kBlock < 128 || p.num_items <= p.max_ctas);
+  return launch_overlapped(kernel, ctas, overlap ? p.max_ctas : 0, kThreads, smem, stream, tq, tk, tv, to, p);
 }
 
 }  // namespace
@@ -727,9 +732,7 @@ int attn_sparse_max_blocks(int block_size) { return block_size < kTileM ? kMaxPa
 // p.num_q_tiles = ceil(seq_len / 128), p.num_blocks = seq_len / block_size.
 cudaError_t launch_attn_sparse(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv,
                                const CUtensorMap& to, const AttnParams& p, int block_size, cudaStream_t stream) {
-  if (block_size == 128)
-    return p.num_items <= p.max_ctas ? launch<128, false, true>(tq, tk, tv, to, p, stream)
-                                     : launch<128, false, false>(tq, tk, tv, to, p, stream);
+  if (block_size == 128) return launch<128, false, true>(tq, tk, tv, to, p, stream);
   if (block_size == 64) return launch<64, false, true>(tq, tk, tv, to, p, stream);
   return launch<32, false, true>(tq, tk, tv, to, p, stream);
 }
