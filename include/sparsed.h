@@ -108,7 +108,8 @@ sparsed_status sparsed_attn_full(const sparsed_shape *shape, const void *q, cons
  * query block at a time without materialising the l x l matrix; for each head and query
  * block the top-rho% key blocks are chosen separately among prefill and generation blocks,
  * ranked by A' (fp32), ties to the lower block index, and written as ascending CSR lists.
- * lse_or_null: the LSE written by sparsed_attn_full for the same Q,K (saves a pass), or NULL.
+ * lse_or_null: the LSE written by sparsed_attn_full for the same Q,K (saves a pass beyond 512 key
+ * blocks per row), or NULL.
  * scores_out_or_null: device fp32 [batch, heads_q, nb, nb] receiving A', or NULL (then the
  * workspace holds it). `out`: host struct; its row_ptr/col_idx/col_capacity are inputs, the
  * other fields are filled in. Requires seq_len % block_size == 0 and
@@ -148,9 +149,11 @@ sparsed_status sparsed_select_from_scores(const sparsed_select_params *params, c
  * Same rules and errors as sparsed_attn_full / sparsed_select_pattern; the selection needs
  * seq_len / block_size <= 2048 (UNSUPPORTED beyond). Both buffers are caller-owned device memory.
  * sparsed_attn_full_stats runs on a kernel whose MMAs span pairs of CTAs (launched as clusters of two);
- * sparsed_attn_full runs on it from 16384 tokens on and on a single-CTA kernel below that. The environment
- * variable SPARSED_DENSE_KERNEL=pair|single, read at the first call, sends sparsed_attn_full to one of
- * them at every length, for measurements.
+ * sparsed_attn_full runs on it where that is the faster one (from 4096 tokens on, by the number of heads
+ * and tokens) and on a single-CTA kernel elsewhere. Both give the same bits (but an LSE within
+ * 1.2e-38 of zero is zero from the CTA-pair kernel). The environment variable
+ * SPARSED_DENSE_KERNEL=pair|single, read at the first call, sends sparsed_attn_full to one of them at
+ * every length, for measurements.
  */
 sparsed_status sparsed_tile_stats_bytes(const sparsed_shape *shape, int32_t block_size,
                                         size_t *out_bytes); /* host only */
@@ -231,9 +234,9 @@ sparsed_status sparsed_attention_step(const sparsed_shape *shape, const sparsed_
  * sparsed_attention_step with one of the method's components switched off: the rows of the paper's
  * component ablation (Table 2) as modes of the same call, for timing and for comparison.
  *   SPARSED_VARIANT_NO_REUSE     "- Sparse Reusing": every sparse step first selects its own pattern from
- *                                that step's Q and K (sparsed_select_pattern with no LSE: a row-statistics
- *                                pass, pooled scoring, ranking) and then attends on it; `pattern` is
- *                                overwritten at every sparse step. Such steps need
+ *                                that step's Q and K (sparsed_select_pattern with no LSE: pooled scoring,
+ *                                in one pass up to 512 key blocks per row, and ranking) and then attends
+ *                                on it; `pattern` is overwritten at every sparse step. Such steps need
  *                                sparsed_workspace_bytes(SPARSED_OP_SELECT_PATTERN, ...) bytes of workspace.
  *   SPARSED_VARIANT_NO_ISOLATION "- Isolated Selection": prefill_len is ignored, one top-rho% over all key
  *                                blocks (Eq. 5 without the split of Eq. 6).

@@ -354,9 +354,9 @@ sparsed_status sparsed_workspace_init(void* ws, size_t ws_bytes, void* cuda_stre
   return e == cudaSuccess ? SPARSED_OK : cuda_fail(e);
 }
 
-// Which dense kernel runs. The pass that also records row statistics has one kernel, the CTA-pair one. The environment
-// variable SPARSED_DENSE_KERNEL (read once) sends every plain pass to one of them, `pair` or `single`, for A/B measurements
-// and tests.
+// Which dense kernel runs. The pass that also records row statistics has one kernel, the CTA-pair one. The
+// environment variable SPARSED_DENSE_KERNEL (read once) sends every plain pass to one of them, `pair` or `single`,
+// for A/B measurements and tests.
 static bool dense_pair_kernel(bool with_stats, const sparsed_shape* shape, int max_ctas) {
   static const int forced = [] {
     const char* v = std::getenv("SPARSED_DENSE_KERNEL");
@@ -702,8 +702,8 @@ sparsed_status sparsed_attention_step_variant(const sparsed_shape* shape, const 
   const int32_t mode = sparsed_schedule_mode(step_1based, total_steps, skip);
   if (mode < 0) return SPARSED_ERR_INVALID_ARG;
   if (mode == SPARSED_MODE_SPARSE && (variant & SPARSED_VARIANT_NO_REUSE)) {
-    // "without Sparse Reusing": this step's own Q and K give this step's pattern (row statistics
-    // pass + pooled scoring + ranking), then the block-sparse attention runs on it
+    // "without Sparse Reusing": this step's own Q and K give this step's pattern (pooled scoring and
+    // ranking), then the block-sparse attention runs on it
     if (mode_out_or_null != nullptr) *mode_out_or_null = mode;
     sparsed_status st = sparsed_select_pattern(shape, &p2, q, k, nullptr, pattern, nullptr, ws, ws_bytes, cuda_stream);
     if (st != SPARSED_OK) return st;

@@ -30,9 +30,10 @@
 #include "sm100_pair_primitives.cuh"
 #include "softmax_pipeline.cuh"
 
-// This file is compiled twice: as it is, and (attention_dense_pair_split.cu) with SPARSED_SPLIT_CLUSTERS for grids whose last
-// clusters own one stream each. Not as a template parameter: any change in the text of the kernel, even one that folds
-// away, makes the compiler schedule the softmax warps' loop differently, by -4 to +1 % of the long launches' time.
+// This file is compiled twice: as it is, and (attention_dense_pair_split.cu) with SPARSED_SPLIT_CLUSTERS for grids
+// whose last clusters own one stream each. Not as a template parameter: as one, or with one more field in the
+// kernel's parameter struct (hence p.max_ctas, which holds the number of two-stream clusters in a split launch), the
+// compiler schedules the softmax warps' loop differently, and the long launches take 1-4 % longer.
 namespace sparsed {
 namespace {
 
@@ -71,7 +72,7 @@ constexpr uint32_t kQHalfStep = (kTileM * 64 * 2) >> 4;                  // 16 K
 constexpr uint32_t kKHalfStep = (32 * 64 * 2) >> 4;                      // 4 KB per head_dim half of a K half-tile
 constexpr uint32_t kSlotStep = (kTileN * 64 * 2) >> 4;                   // 8 KB per ring slot
 
-// kStatKeys: record one row statistic per 32 / 64 / 128 keys (none if p.tile_lse is null).
+// kStatKeys: record one row statistic per 32 / 64 / 128 keys (none is stored if p.tile_lse is null).
 template <int kStatKeys>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 attn_dense_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
@@ -276,13 +277,11 @@ attn_dense_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
     bool ok = true;
     RowState st{-INFINITY, 0.f};
     RowStatWriter<kStatKeys> stats;
-    if constexpr (kStatKeys > 0) {
-      const int groups = (p.seq_len + kStatKeys - 1) / kStatKeys;
-      float* first = nullptr;
-      if (p.tile_lse != nullptr && q_row0 + row_in_tile < p.seq_len)
-        first = p.tile_lse + (static_cast<int64_t>(bh) * p.num_q_tiles + q_tile) * groups * kTileM + row_in_tile;
-      stats.init(first, groups);
-    }
+    const int groups = (p.seq_len + kStatKeys - 1) / kStatKeys;
+    float* first = nullptr;
+    if (p.tile_lse != nullptr && q_row0 + row_in_tile < p.seq_len)
+      first = p.tile_lse + (static_cast<int64_t>(bh) * p.num_q_tiles + q_tile) * groups * kTileM + row_in_tile;
+    stats.init(first, groups);
     // One 64-key tile of the softmax; kOdd (a compile-time tag) is used by the walk that records one statistic per
     // 128 keys, which runs its tiles in pairs.
     auto tile_body = [&](int t, auto odd_tag) -> bool {
@@ -308,7 +307,7 @@ attn_dense_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
       }
       if (__any_sync(0xffffffffu, exact)) {
         const float alpha = softmax_group_exact(r0, r1, scale_log2, st, pk, sums);
-        if constexpr (kStatKeys > 0) stats.rescale(alpha);
+        stats.rescale(alpha);
         if (t > 0) {
           // O must be quiescent: wait until P_{t-1} V_{t-1} (which read ring load 2t-1) has drained
           const int gp = 2 * (t - 1) + 1;
@@ -319,14 +318,14 @@ attn_dense_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
         }
       }
       st.l += sums.x + sums.y;
-      if constexpr (kStatKeys > 0) stats.begin(sums, kOdd);
+      stats.begin(sums, kOdd);
       tmem_st32(tS, pk);  // P_t over the first 32 columns of S_t
       tmem_wait_st();
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive_cluster(buf ? p_full_leader1 : p_full_leader0);
       // the statistic is stored after P has been handed over: off the S -> P -> P V chain
-      if constexpr (kStatKeys > 0) stats.finish(st.m, kOdd);
+      stats.finish(st.m, kOdd);
       return true;
     };
     {
@@ -402,7 +401,8 @@ cudaError_t launch_attn_dense_pair_split(const CUtensorMap& tq, const CUtensorMa
   return launch_any(tq, tk, tv, to, p, clusters, stream);
 }
 #else
-// Tensor maps: Q and O boxes 64 x 128 rows, K box 64 x 32 rows, V box 64 x 64 rows. p.num_q_tiles = ceil(seq_len / 128).
+// Tensor maps: Q and O boxes 64 x 128 rows, K box 64 x 32 rows, V box 64 x 64 rows. p.num_q_tiles =
+// ceil(seq_len / 128).
 cudaError_t launch_attn_dense_pair(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv,
                                    const CUtensorMap& to, const AttnParams& p, cudaStream_t stream) {
   const long long bh = p.num_q_tiles > 0 ? p.num_items / p.num_q_tiles : 0;

@@ -3,19 +3,19 @@
 
 namespace sparsed {
 
-// Whether the last wave of `clusters` clusters over `pairs` SM pairs runs as clusters of one stream each. Such a cluster
-// takes 0.65-0.8 of the time of one with two. So a last wave that would leave half of the SM pairs idle or more is
-// launched that way: 2 heads x 4096 tokens 63.5 -> 47.1 us, 8 x 2048 36.9 -> 28.7, 2 x 1024 22.6 -> 18.4, 16 x 3072 (1.3
-// waves) 95.0 -> 84.4 (statistics recorded). From two full waves on the launch runs into the power limit, which an
-// emptier last wave only relieves (32 x 4096, 3.46 waves: no gain).
+// Whether the last wave of `clusters` clusters over `pairs` SM pairs runs as clusters of one stream each. Such a
+// cluster takes 0.65-0.8 of the time of one with two. So a last wave that would leave half of the SM pairs idle or
+// more is launched that way: 2 heads x 4096 tokens 63.5 -> 47.1 us, 8 x 2048 36.9 -> 28.7, 2 x 1024 22.6 -> 18.4,
+// 16 x 3072 (1.3 waves) 95.0 -> 84.4 (statistics recorded). From two full waves on the launch runs into the power
+// limit, which an emptier last wave only relieves (32 x 4096, 3.46 waves: no gain).
 inline bool dense_pair_splits(long long clusters, long long pairs) {
   const long long last = pairs > 0 ? clusters % pairs : 0;
   return last != 0 && 2 * last <= pairs && clusters < 2 * pairs;
 }
 
-// Time of `units` equal pieces of work on `slots`, in full waves. The last wave counts as 0.65 if it is at most half full and
-// its half-empty SMs run faster (two CTAs per SM, or split clusters), else as 0.5 and half its share (the SMs that are
-// busy have the power of the others).
+// Time of `units` equal pieces of work on `slots`, in full waves. The last wave counts as 0.65 if it is at most half
+// full and its half-empty SMs run faster (two CTAs per SM, or split clusters), else as 0.5 and half its share (the
+// SMs that are busy have the power of the others).
 inline double dense_waves(long long units, long long slots, bool half_wave) {
   const long long last = units % slots;
   const double whole = static_cast<double>(units / slots);
@@ -28,17 +28,18 @@ inline double dense_waves(long long units, long long slots, bool half_wave) {
 // entries; the single-CTA kernel (attention.cu) takes the others. Both give the same bits. max_ctas: CTAs of the latter
 // that fit on the device at once, two per SM.
 //
-// Per query row the pair kernel takes 3-7 % less under sustained load, which is bound by power (it fetches each K/V tile
-// once for 512 rows instead of once for 128): 32 heads x 8192 956 -> 928 us, 8 x 32 x 4096 1990 -> 1915, 32 x 16384
-// 3720 -> 3495. Launches too short to reach the power limit, or with rests between them, gain nothing from that, and the
-// longer set-up and tear-down of a cluster costs them 2-8 % (20 launches after a rest: 8 heads x 4096 60.0 against
-// 64.3 us, 20 heads 172 against 179). So the pair kernel runs where it was no slower either way:
+// Per query row the pair kernel takes 3-7 % less under sustained load, which is bound by power (it fetches each K/V
+// tile once for 512 rows instead of once for 128): 32 heads x 8192 956 -> 928 us, 8 x 32 x 4096 1990 -> 1915, 32 x
+// 16384 3720 -> 3495. Launches too short to reach the power limit, or with rests between them, gain nothing from
+// that, and the longer set-up and tear-down of a cluster costs them 2-8 % (20 launches after a rest: 8 heads x 4096
+// 60.0 against 64.3 us, 20 heads 172 against 179). So the pair kernel runs where it was no slower either way:
 //   * where the last wave, or the only one, runs as clusters of one stream each: its SMs would be half empty in both
 //     kernels (1 x 4096 48.3 -> 48.1 us, 6 x 8192 217 -> 198, 3 x 16384 417 -> 374);
-//   * from 2^29 logits on (32 heads x 4096, 8 x 8192), which take 200 us. Of those with fewer 12 heads x 6144 lose 1 % after
-//     a rest, and 5 heads x 4096 9 % even under sustained load: 40 clusters leave 68 SMs empty, 160 CTAs none.
-// A wave of either is the same number of rows, but the last one may be emptier: 8 heads x 14000 are 3.03 waves of clusters
-// (740 us) and 2.97 of single CTAs (690). So the waves are counted as well.
+//   * from 2^29 logits on (32 heads x 4096, 8 x 8192), which take 200 us. With fewer, 12 heads x 6144 lose 1 % after
+//     a rest, and 5 heads x 4096 9 % even under sustained load: 40 clusters leave 68 SMs empty, 160 CTAs
+//     none.
+// A wave of either is the same number of rows, but the last one may be emptier: 8 heads x 14000 are 3.03 waves of
+// clusters (740 us) and 2.97 of single CTAs (690). So the waves are counted as well.
 inline bool dense_pair_pays(long long bh, int seq_len, int max_ctas) {
   if (seq_len < 4096 || max_ctas < 4) return false;
   const long long tiles = (static_cast<long long>(seq_len) + 127) / 128;

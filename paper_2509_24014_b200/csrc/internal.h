@@ -62,7 +62,8 @@ struct AttnParams {
                            // write O through its tensor map)
   int64_t o_stride_b, o_stride_h, o_stride_t;
   float* lse;              // fp32 [B,Hq,L] or null
-  float* tile_lse;         // fp32 [B*Hq, ceil(L/128), ceil(L/stat_keys), 128] or null: base-2 log-sum-exp of each row over each group of stat_keys keys
+  float* tile_lse;         // fp32 [B*Hq, ceil(L/128), ceil(L/stat_keys), 128] or null: base-2 log-sum-exp of each row
+                           // over each group of stat_keys keys
   int stat_keys;           // 32, 64 or 128
   unsigned long long* slow_path_events;  // counts warp-level rescales of the output accumulator, or null
   int seq_len;

@@ -18,15 +18,15 @@
 //   * kRowStats log-sum-exp of every row: the first of the two passes that rows with more than 512 key blocks
 //               take.
 //
-// Pipeline per CTA (320 threads, two CTAs per SM but for kOnePassWide / Most): warp 8 streams 64-key K tiles by TMA into a ring of four, warp 9
-// issues S = Q K^T (one commit per tile: "S ready" for the softmax warps, "slot free" for the producer), warps 0-3 and
-// 4-7 are two groups with one thread per query row each. The groups take turns at 128 keys (two tiles), so that a key
-// block belongs to one of them; each has one S buffer and its own reference and denominator of every row, which meet at the
-// end. A thread copies its row of S into registers, hands the buffer back at once, exponentiates and sums. Four
-// such warps per scheduler cover each other's waits: with two (one group per CTA, two S buffers) the first case below
-// took 2.53 ms, with the next tile's copy pipelined into the current one's exponentials as well 2.70 ms.
-// Sums run in a fixed order, so results are bitwise reproducible. When the keys of its block-row(s) fit in shared
-// memory the CTA ranks them itself (warp_select_row) and writes the CSR lists.
+// Pipeline per CTA (320 threads, two CTAs per SM but for kOnePassWide / Most): warp 8 streams 64-key K tiles by TMA
+// into a ring of four, warp 9 issues S = Q K^T (one commit per tile: "S ready" for the softmax warps, "slot free" for
+// the producer), warps 0-3 and 4-7 are two groups with one thread per query row each. The groups take turns at 128
+// keys (two tiles), so that a key block belongs to one of them; each has one S buffer and its own reference and
+// denominator of every row, which meet at the end. A thread copies its row of S into registers, hands the buffer back
+// at once, exponentiates and sums. Four such warps per scheduler cover each other's waits: with two (one group per
+// CTA, two S buffers) the first case below took 2.53 ms, with the next tile's copy pipelined into the current one's
+// exponentials as well 2.70 ms. Sums run in a fixed order, so results are bitwise reproducible. When the keys of its
+// block-row(s) fit in shared memory the CTA ranks them itself (warp_select_row) and writes the CSR lists.
 //
 // Measured on B200, from Q and K alone (two passes over the logits before, with two CTAs of four softmax warps):
 //   28 heads x 16384 tokens, block 128   6.21 -> 2.50 ms (kOnePass; exponential unit busy 82 % of the time)
@@ -51,8 +51,9 @@ constexpr int kMaxKeys = 2048;  // ranking keys held in shared memory: (block-ro
 enum ScoreMode { kOnePass, kOnePassWide, kOnePassMost, kPooled, kRowStats };
 __host__ __device__ constexpr bool one_per_sm(int mode) { return mode == kOnePassWide || mode == kOnePassMost; }
 __host__ __device__ constexpr int tmem_cols(int mode) { return one_per_sm(mode) ? 512 : 256; }
-__host__ __device__ constexpr int tmem_sums(int mode) { return tmem_cols(mode) - kColStat; }     // block sums held per row in tensor memory
-__host__ __device__ constexpr int smem_sums(int mode) { return mode == kOnePassMost ? 128 : 0; }   // ... in shared memory
+// block sums held per row: in tensor memory, in shared memory, in all
+__host__ __device__ constexpr int tmem_sums(int mode) { return tmem_cols(mode) - kColStat; }
+__host__ __device__ constexpr int smem_sums(int mode) { return mode == kOnePassMost ? 128 : 0; }
 __host__ __device__ constexpr int block_sums(int mode) { return tmem_sums(mode) + smem_sums(mode); }
 
 // A row's reference is the maximum of both groups' first 64-key tiles, and stays until the sum of a later tile outgrows

@@ -54,7 +54,8 @@ __device__ __forceinline__ float2 softmax_group_fast(const uint32_t (&r0)[32], c
 }
 
 // The same over one half of a group: 32 columns, P into 16 registers, returns their sum.
-__device__ __forceinline__ float softmax_half_fast(const uint32_t (&r)[32], float scale_log2, float m, uint32_t (&pk)[16]) {
+__device__ __forceinline__ float softmax_half_fast(const uint32_t (&r)[32], float scale_log2, float m,
+                                                   uint32_t (&pk)[16]) {
   const float2 sc = make_float2(scale_log2, scale_log2);
   const float2 nm = make_float2(-m, -m);
   float2 acc0 = make_float2(0.f, 0.f), acc1 = make_float2(0.f, 0.f);
@@ -194,7 +195,7 @@ __device__ __forceinline__ void rescale_accumulator_row(uint32_t t_acc_row, floa
 // [key group][row in tile] so that a query tile's statistics are one contiguous run. The
 // attention kernels feed it 64 keys at a time (the two 32-column sums of a softmax group,
 // relative to the reference maximum in use at that moment).
-template <int kStatKeys>   // 0 = no statistics, else 32, 64 or 128 keys per statistic
+template <int kStatKeys>   // 32, 64 or 128 keys per statistic
 struct RowStatWriter {
   float* next;       // where this row's next statistic goes (statistics of one row are 128 floats apart)
   int left;          // statistics still to be written for this row (0 for rows beyond the sequence end)
@@ -226,7 +227,7 @@ struct RowStatWriter {
     } else if constexpr (kStatKeys == 32) {
       lg0 = fast_log2(sums.x);
       lg1 = fast_log2(sums.y);
-    } else if constexpr (kStatKeys == 128) {
+    } else {
       carry += sums.x + sums.y;
       if (second_half) {
         lg0 = fast_log2(carry);
@@ -246,7 +247,7 @@ struct RowStatWriter {
       if (left > 1) __stcs(next + 128, m + lg1);
       next += 256;
       left -= 2;
-    } else if constexpr (kStatKeys == 128) {
+    } else {
       if (second_half) {
         if (left > 0) __stcs(next, m + lg0);
         next += 128;
