@@ -29,10 +29,16 @@
 // block-row(s) fit in shared memory the CTA ranks them itself (warp_select_row) and writes the CSR lists.
 //
 // Measured on B200, from Q and K alone (two passes over the logits before, with two CTAs of four softmax warps):
-//   28 heads x 16384 tokens, block 128   6.21 -> 2.50 ms (kOnePass; exponential unit busy 82 % of the time)
-//   32 heads x 8192 tokens, block 128    1.79 -> 0.73 ms (kOnePass)
-//   28 heads x 16384 tokens, block 64    6.26 -> 3.53 ms (kOnePassWide; in two passes 5.0)
-//   8 heads x 65536 tokens, block 128    27.5 -> 15.9 ms (kOnePassMost; in two passes 22.3)
+//   28 heads x 16384 tokens, block 128   6.19 -> 2.45 ms (kOnePass; exponential unit busy 71 % of the time on average over
+//                                        the SMs and 82 % on the busiest, at 4 heads: 1.73 waves)
+//   32 heads x 8192 tokens, block 128    1.78 -> 0.73 ms (kOnePass)
+//   28 heads x 16384 tokens, block 64    6.21 -> 3.55 ms (kOnePassWide; in two passes 5.0)
+//   8 heads x 65536 tokens, block 128    27.4 -> 15.7 ms (kOnePassMost; in two passes 22.3)
+//   8 heads x 65536 tokens, block 64     27.5 -> 21.5 ms (kRowStats, kPooled)
+// and with the caller's LSE (kPooled, one pass before as well):
+//   28 heads x 16384 tokens, block 128   2.42 -> 2.35 ms
+//   8 heads x 65536 tokens, block 128    10.8 -> 11.0 ms
+//   32 heads x 4096 tokens, block 32     0.191 -> 0.194 ms
 #include "internal.h"
 #include "softmax_pipeline.cuh"
 #include "topk_device.cuh"
