@@ -29,16 +29,16 @@
 // block-row(s) fit in shared memory the CTA ranks them itself (warp_select_row) and writes the CSR lists.
 //
 // Measured on B200, from Q and K alone (two passes over the logits before, with two CTAs of four softmax warps):
-//   28 heads x 16384 tokens, block 128   6.19 -> 2.45 ms (kOnePass; exponential unit busy 71 % of the time on average over
+//   28 heads x 16384 tokens, block 128   6.21 -> 2.43 ms (kOnePass; exponential unit busy 71 % of the time on average over
 //                                        the SMs and 82 % on the busiest, at 4 heads: 1.73 waves)
-//   32 heads x 8192 tokens, block 128    1.78 -> 0.73 ms (kOnePass)
-//   28 heads x 16384 tokens, block 64    6.21 -> 3.55 ms (kOnePassWide; in two passes 5.0)
-//   8 heads x 65536 tokens, block 128    27.4 -> 15.7 ms (kOnePassMost; in two passes 22.3)
-//   8 heads x 65536 tokens, block 64     27.5 -> 21.5 ms (kRowStats, kPooled)
+//   32 heads x 8192 tokens, block 128    1.79 -> 0.72 ms (kOnePass)
+//   28 heads x 16384 tokens, block 64    6.24 -> 3.29 ms (kOnePassWide; in two passes 5.0)
+//   8 heads x 65536 tokens, block 128    27.4 -> 14.0 ms (kOnePassMost; in two passes 22.3)
+//   8 heads x 65536 tokens, block 64     27.6 -> 21.9 ms (kRowStats, kPooled)
 // and with the caller's LSE (kPooled, one pass before as well):
-//   28 heads x 16384 tokens, block 128   2.42 -> 2.35 ms
-//   8 heads x 65536 tokens, block 128    10.8 -> 11.0 ms
-//   32 heads x 4096 tokens, block 32     0.191 -> 0.194 ms
+//   28 heads x 16384 tokens, block 128   2.48 -> 2.38 ms
+//   8 heads x 65536 tokens, block 128    11.2 -> 10.9 ms
+//   32 heads x 4096 tokens, block 32     0.193 -> 0.196 ms
 #include "internal.h"
 #include "softmax_pipeline.cuh"
 #include "topk_device.cuh"
@@ -242,6 +242,7 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
     const int row = q_row0 + rit;
     const bool row_valid = row < p.seq_len;
     const int bs = p.block_size;
+    const int bs_shift = 31 - __clz(bs);   // (a division per tile took 3-12 % of the kernel's time)
     const int nb = kMode == kRowStats ? 0 : p.seq_len / bs;
     const int rows_here = kTileM / bs;                       // block-rows of A' in this tile: 1, 2 or 4
     const bool rank_here = kMode != kRowStats && p.row_ptr != nullptr;
@@ -394,7 +395,7 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
         l += s0 + s1;
       }
       if constexpr (kMode != kRowStats) {
-        const int col = (t * kTileN) / bs - jb0;   // first block of the tile
+        const int col = ((t * kTileN) >> bs_shift) - jb0;   // first block of the tile
         if (bs == 128) {
           if ((t & 1) == 0) {
             carry = s0 + s1;
@@ -409,7 +410,7 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
         }
         if constexpr (kMode == kPooled) {
           // 128 blocks are bs spans of 128 keys: bs / 2 spans, bs tiles of each group
-          if ((j + 1) % bs == 0) {
+          if (((j + 1) & (bs - 1)) == 0) {
             fold(jb0, min(kChunk, nb - jb0), {1.f, 1.f}, {1.f, 1.f});
             jb0 += kChunk;
           }
