@@ -29,8 +29,8 @@
 // block-row(s) fit in shared memory the CTA ranks them itself (warp_select_row) and writes the CSR lists.
 //
 // Measured on B200, from Q and K alone (two passes over the logits before, with two CTAs of four softmax warps):
-//   28 heads x 16384 tokens, block 128   6.21 -> 2.43 ms (kOnePass; exponential unit busy 71 % of the time on average over
-//                                        the SMs and 82 % on the busiest, at 4 heads: 1.73 waves)
+//   28 heads x 16384 tokens, block 128   6.21 -> 2.43 ms (kOnePass; exponential unit busy 73 % of the time on average over
+//                                        the SMs and 84 % on the busiest, at 4 heads: 1.73 waves)
 //   32 heads x 8192 tokens, block 128    1.79 -> 0.72 ms (kOnePass)
 //   28 heads x 16384 tokens, block 64    6.24 -> 3.29 ms (kOnePassWide; in two passes 5.0)
 //   8 heads x 65536 tokens, block 128    27.4 -> 14.0 ms (kOnePassMost; in two passes 22.3)
