@@ -355,18 +355,22 @@ sparsed_status sparsed_workspace_init(void* ws, size_t ws_bytes, void* cuda_stre
 }
 
 // Which dense kernel runs. The pass that also records row statistics has one kernel, the CTA-pair one. The
-// environment variable SPARSED_DENSE_KERNEL (read once) sends every plain pass to one of them, `pair` or `single`,
-// for A/B measurements and tests.
-static bool dense_pair_kernel(bool with_stats, const sparsed_shape* shape, int max_ctas) {
+// environment variable SPARSED_DENSE_KERNEL (read once) sends every plain pass to one of them, `pair`, `single` or
+// `lone`, for A/B measurements and tests.
+enum DenseKernel { kSingle, kPair, kLone };
+static DenseKernel dense_kernel(bool with_stats, const sparsed_shape* shape, int max_ctas) {
   static const int forced = [] {
     const char* v = std::getenv("SPARSED_DENSE_KERNEL");
-    if (v != nullptr && std::strcmp(v, "pair") == 0) return 1;
-    if (v != nullptr && std::strcmp(v, "single") == 0) return 0;
+    if (v != nullptr && std::strcmp(v, "pair") == 0) return static_cast<int>(kPair);
+    if (v != nullptr && std::strcmp(v, "single") == 0) return static_cast<int>(kSingle);
+    if (v != nullptr && std::strcmp(v, "lone") == 0) return static_cast<int>(kLone);
     return -1;
   }();
-  if (with_stats) return true;
-  if (forced >= 0) return forced == 1;
-  return dense_pair_pays(static_cast<long long>(shape->batch) * shape->heads_q, shape->seq_len, max_ctas);
+  if (with_stats) return kPair;
+  if (forced >= 0) return static_cast<DenseKernel>(forced);
+  const long long bh = static_cast<long long>(shape->batch) * shape->heads_q;
+  if (lone_ctas_pay(bh * ((static_cast<long long>(shape->seq_len) + 127) / 128), shape->seq_len, max_ctas)) return kLone;
+  return dense_pair_pays(bh, shape->seq_len, max_ctas) ? kPair : kSingle;
 }
 
 static sparsed_status attn_full_impl(const sparsed_shape* shape, const void* q, const void* k, const void* v, void* o,
@@ -381,11 +385,11 @@ static sparsed_status attn_full_impl(const sparsed_shape* shape, const void* q, 
   if ((st = check_ws(ws, ws_bytes, SPARSED_STATUS_BYTES)) != SPARSED_OK) return st;
   if ((st = check_arch()) != SPARSED_OK) return st;
   const int max_ctas = attn_max_ctas();
-  const bool pair = dense_pair_kernel(tile_lse_or_null != nullptr, shape, max_ctas);
+  const DenseKernel kernel = dense_kernel(tile_lse_or_null != nullptr, shape, max_ctas);
   CUtensorMap tq, tk, tv, to;
   if ((st = make_tensor_map(&tq, q, shape->batch, shape->heads_q, shape->seq_len, rs.q, 128)) != SPARSED_OK) return st;
   if ((st = make_tensor_map(&to, o, shape->batch, shape->heads_q, shape->seq_len, rs.o, 128)) != SPARSED_OK) return st;
-  if ((st = make_tensor_map(&tk, k, shape->batch, shape->heads_kv, shape->seq_len, rs.k, pair ? 32 : 64)) != SPARSED_OK) return st;
+  if ((st = make_tensor_map(&tk, k, shape->batch, shape->heads_kv, shape->seq_len, rs.k, kernel == kPair ? 32 : 64)) != SPARSED_OK) return st;
   if ((st = make_tensor_map(&tv, v, shape->batch, shape->heads_kv, shape->seq_len, rs.v, 64)) != SPARSED_OK) return st;
   AttnParams p;
   p.o = o;
@@ -408,8 +412,10 @@ static sparsed_status attn_full_impl(const sparsed_shape* shape, const void* q, 
   p.col_idx = nullptr;
   p.col_capacity = 0;
   p.status = static_cast<DeviceStatus*>(ws);
-  cudaError_t e = pair ? launch_attn_dense_pair(tq, tk, tv, to, p, static_cast<cudaStream_t>(cuda_stream))
-                      : launch_attn_dense(tq, tk, tv, to, p, static_cast<cudaStream_t>(cuda_stream));
+  const cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
+  cudaError_t e = kernel == kPair   ? launch_attn_dense_pair(tq, tk, tv, to, p, stream)
+                  : kernel == kLone ? launch_attn_dense_lone(tq, tk, tv, p, stream)
+                                    : launch_attn_dense(tq, tk, tv, to, p, stream);
   return e == cudaSuccess ? SPARSED_OK : cuda_fail(e);
 }
 
@@ -567,7 +573,12 @@ sparsed_status sparsed_attn_sparse(const sparsed_shape* shape, const sparsed_pat
   p.col_idx = pattern->col_idx;
   p.col_capacity = pattern->col_capacity;
   p.status = static_cast<DeviceStatus*>(ws);
-  cudaError_t e = launch_attn_sparse(tq, tk, tv, to, p, bs, static_cast<cudaStream_t>(cuda_stream));
+  const cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
+  // (the lists' average length; 0 if the caller's pattern does not say how many entries it has)
+  const long long rows = static_cast<long long>(shape->batch) * shape->heads_q * pattern->num_blocks;
+  const long long keys = pattern->nnz > 0 ? pattern->nnz / rows * bs : 0;
+  cudaError_t e = lone_ctas_pay(p.num_items, keys, p.max_ctas) ? launch_attn_sparse_lone(tq, tk, tv, p, bs, stream)
+                                                               : launch_attn_sparse(tq, tk, tv, to, p, bs, stream);
   return e == cudaSuccess ? SPARSED_OK : cuda_fail(e);
 }
 

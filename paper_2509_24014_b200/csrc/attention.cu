@@ -1,6 +1,7 @@
 // Attention for head_dim 128, bf16 in / bf16 out, fp32 softmax, on sm_100a, from one kernel:
 // dense bidirectional attention (Eq. 1 times V; the full-attention branch of Algorithm 1) and
-// block-sparse attention over CSR block lists (Eq. 3 / Eq. 4 times V; the "Sparse Reusing" branch).
+// block-sparse attention over CSR block lists (Eq. 3 / Eq. 4 times V; the "Sparse Reusing" branch). Grids of up to one
+// query tile per SM go to attention_lone.cu, large dense ones to attention_dense_pair.cu (dense_choice.h).
 //
 // One CTA owns 128 consecutive query rows of one (batch, head) and streams 64-key tiles through a
 // warp-specialised pipeline:
@@ -34,19 +35,17 @@
 //     common.
 #include "internal.h"
 #include "softmax_pipeline.cuh"
+#include "work_items.cuh"
 
 namespace sparsed {
 namespace {
 
 constexpr int kHeadDim = 128;
-constexpr int kTileM = 128;   // UMMA M; rows of tensor memory
-constexpr int kTileN = 64;    // keys per pipeline step
 constexpr int kSoftmaxThreads = 128;
 constexpr int kThreads = 192;
 constexpr int kTmemCols = 256;
 constexpr int kColS = 0;      // two S buffers of 64 fp32 columns; P (bf16 pairs) reuses the first 32
 constexpr int kColO = 128;    // O accumulator (fp32, 128 columns)
-constexpr int kMaxPackedBlocks = 2048;   // key blocks per row the union walk can hold (64- and 32-key blocks)
 
 // Debug builds (-DSPARSED_TIMELINE) record clock64 stamps of one CTA's pipeline roles after the
 // workspace status block: 3 regions of 2048 int64 (softmax thread 0, UMMA thread, TMA thread).
@@ -64,7 +63,6 @@ struct AttnSmem {
   static constexpr bool kPacked = kBlock < kTileM;
   static constexpr int kSlots = kPacked ? 4 : 5;
   static constexpr int kGroups = kTileM / kBlock;                       // query blocks per CTA
-  static constexpr int kWords = kPacked ? kMaxPackedBlocks / 32 : 1;    // bitmap words per query block
   alignas(1024) __nv_bfloat16 q[2][kTileM * 64];           // two 64-wide halves of head_dim
   alignas(1024) __nv_bfloat16 kv[kSlots][2][kTileN * 64];  // each slot: two 64-wide halves of head_dim
   uint64_t q_full, kv_full[kSlots];
@@ -83,10 +81,8 @@ struct AttnSmem {
   // ... and the union itself, ascending, one entry per key block: its id and, from bit kIdBits on, one bit per query block
   // that keeps it. One per item buffer: the next item's union is built while this one's is walked.
   alignas(16) uint16_t list[2][kPacked ? kMaxPackedBlocks + 2 : 2];
-  uint32_t member[kGroups][kWords];  // producer only: bit j of query block g = "g keeps key block j"
+  uint32_t member[kGroups][kMemberWords<kBlock>];  // producer only: bit j of query block g = "g keeps key block j"
 };
-constexpr int kIdBits = 11;
-static_assert((1 << kIdBits) == kMaxPackedBlocks, "ids of union entries");
 
 // kDense: walk every key tile of the sequence (kBlock must be 128 then; no block lists are read).
 // kOverlap: begins with wait_for_previous_kernel, so that small grids may be launched overlapped. (Of the dense walk there
@@ -130,39 +126,9 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
   //     32, 8 x 32 heads x 4096 tokens, half kept: 1524 us with one item per CTA, 1450 with equal shares, 1439 this way;
   //     block 64, 32 x 65536: 8.64 ms with equal shares, 8.06 this way. (With 128-key blocks it was 1 % slower than equal
   //     shares.)
-  struct Item {
-    int q_tile, bh, head, batch, kv_head, q_row0, groups_here, r0;
-    int list_begin, list_len;   // CSR entries of the item's query blocks; dense: key tiles of the sequence
-  };
+  using Item = WorkItem;
   const int n_items = p.num_items;
-  // with_list: read the item's row_ptr entries too
-  auto describe = [&](int item, bool with_list) -> Item {
-    Item it;
-    it.q_tile = item % p.num_q_tiles;
-    it.bh = item / p.num_q_tiles;
-    it.head = it.bh % p.heads_q;
-    it.batch = it.bh / p.heads_q;
-    it.kv_head = it.head / p.group;
-    it.q_row0 = it.q_tile * kTileM;
-    const int qb0 = it.q_tile * kGroups;                                   // first query block of the item
-    it.groups_here = kDense ? 1 : min(kGroups, p.num_blocks - qb0);        // the last tile of a head may hold fewer
-    it.r0 = it.bh * p.num_blocks + qb0;                                    // CSR row of query block qb0
-    it.list_begin = 0;
-    it.list_len = (p.seq_len + kTileN - 1) / kTileN;
-    if (!kDense && with_list) {
-      // adjacent rows are adjacent in col_idx, so the item's lists are one run of entries
-      it.list_begin = __ldcg(p.row_ptr + it.r0);
-      it.list_len = __ldcg(p.row_ptr + it.r0 + it.groups_here) - it.list_begin;
-      if (it.list_begin < 0 || it.list_len < 0 ||
-          static_cast<int64_t>(it.list_begin) + it.list_len > p.col_capacity) {
-        // row_ptr points outside col_idx: not followed; the rows get zeros and the status word says why
-        if (atomicCAS(&p.status->code, 0, 3) == 0) p.status->where = 2;
-        it.list_begin = 0;
-        it.list_len = 0;
-      }
-    }
-    return it;
-  };
+  auto describe = [&](int item, bool with_list) -> Item { return describe_item<kGroups, kDense>(p, item, with_list); };
   // tiles of an item in the unpacked walks (the packed walk counts its union instead)
   auto unpacked_tiles = [&](const Item& it) -> int { return kDense ? it.list_len : it.list_len * kTilesPerBlock; };
 
@@ -208,46 +174,9 @@ attn_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CU
     const int e = t / kTilesPerBlock;
     return __shfl_sync(0xffffffffu, list_ids, e & 31) * kBlock + (t % kTilesPerBlock) * kTileN;
   };
-  // Packed walks, producer warp: one bitmap per query block of the item, then their union into list buffer `buf`;
-  // returns its length. The last tile of an odd union of 32-key blocks is filled up with its own last block, which no
-  // query block keeps there.
+  // packed walks, producer warp: the union of the item's lists into list buffer `buf`; returns its length
   auto build_union = [&](const Item& it, int buf) -> int {
-    const int words = (p.num_blocks + 31) >> 5;
-    for (int i = lane; i < kGroups * Smem::kWords; i += 32) (&sm.member[0][0])[i] = 0u;
-    // (entries are unsigned: a list may end at 2^31 - 1, and the walk steps up to 287 beyond)
-    uint32_t bound[kGroups];   // bound[g] = first CSR entry after query block g's list
-#pragma unroll
-    for (int g = 0; g < kGroups; ++g)
-      bound[g] = static_cast<uint32_t>(__ldcg(p.row_ptr + it.r0 + min(g + 1, it.groups_here)));
-    __syncwarp();
-    const uint32_t list_end = static_cast<uint32_t>(it.list_begin) + static_cast<uint32_t>(it.list_len);
-    for (uint32_t e0 = static_cast<uint32_t>(it.list_begin) + lane; e0 < list_end; e0 += 8 * 32) {
-      int id[8];   // eight loads in flight per lane
-#pragma unroll
-      for (int u = 0; u < 8; ++u) id[u] = e0 + 32 * u < list_end ? __ldcg(p.col_idx + e0 + 32 * u) : -1;
-#pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        int g = 0;
-#pragma unroll
-        for (int j = 0; j + 1 < kGroups; ++j) g += (e0 + 32 * u >= bound[j]) ? 1 : 0;
-        if (id[u] >= 0 && id[u] < p.num_blocks) atomicOr(&sm.member[g][id[u] >> 5], 1u << (id[u] & 31));
-      }
-    }
-    __syncwarp();
-    uint16_t* list = sm.list[buf];
-    int n = 0;
-    for (int w = 0; w < words; ++w) {   // lane = bit of the word
-      uint32_t mask = 0u;
-#pragma unroll
-      for (int g = 0; g < kGroups; ++g) mask |= ((sm.member[g][w] >> lane) & 1u) << g;
-      const uint32_t any = __ballot_sync(0xffffffffu, mask != 0u);
-      if (mask != 0u)
-        list[n + __popc(any & ((1u << lane) - 1u))] = static_cast<uint16_t>((w * 32 + lane) | (mask << kIdBits));
-      n += __popc(any);
-    }
-    __syncwarp();
-    if (kBlocksPerTile > 1 && (n & 1) != 0 && lane == 0) list[n] = list[n - 1] & ((1u << kIdBits) - 1u);
-    return n;
+    return build_list_union<kGroups, kBlocksPerTile>(p, it, lane, sm.member, sm.list[buf]);
   };
   // the CTA's next item (-1: none), `entries` key blocks long, to the other roles
   auto publish = [&](int buf, int item, int entries) {

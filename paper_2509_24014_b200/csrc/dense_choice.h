@@ -34,7 +34,8 @@ inline double dense_waves(long long units, long long slots, bool half_wave) {
 // that, and the longer set-up and tear-down of a cluster costs them 2-8 % (20 launches after a rest: 8 heads x 4096
 // 60.0 against 64.3 us, 20 heads 172 against 179). So the pair kernel runs where it was no slower either way:
 //   * where the last wave, or the only one, runs as clusters of one stream each: its SMs would be half empty in both
-//     kernels (1 x 4096 48.3 -> 48.1 us, 6 x 8192 217 -> 198, 3 x 16384 417 -> 374);
+//     kernels (6 x 8192 217 -> 198 us, 3 x 16384 417 -> 374; an only wave that is split is up to one query tile per SM, and
+//     goes to a third kernel first, see below);
 //   * from 2^29 logits on (32 heads x 4096, 8 x 8192), which take 200 us. With fewer, 12 heads x 6144 lose 1 % after
 //     a rest, and 5 heads x 4096 9 % even under sustained load: 40 clusters leave 68 SMs empty, 160 CTAs
 //     none.
@@ -48,6 +49,17 @@ inline bool dense_pair_pays(long long bh, int seq_len, int max_ctas) {
   const double logits = static_cast<double>(bh) * seq_len * seq_len;
   if (!split && logits < static_cast<double>(1 << 29)) return false;
   return 0.965 * dense_waves(clusters, pairs, split) < dense_waves(bh * tiles, max_ctas, true);
+}
+
+// Whether attention on `items` query tiles, dense or over block lists, with `keys` keys to a row (on average) goes to the
+// kernel whose CTAs have an SM each (attention_lone.cu), before the choice above is asked. It gives the same bits as the
+// others. Up to one item per SM it was the fastest from five tiles of 64 keys on: dense, against the single-CTA kernel, 2
+// heads x 320 7.70 -> 6.79 us, 2 x 1024 14.9 -> 12.1, 8 x 2304 (144 items) 29.7 -> 23.4, and against split clusters 2 x
+// 4096 44.0 -> 35.8, 2 x 9400 102 -> 77.5; sparse 2 x 8192 block 128 at 4 blocks a row 10.5 -> 9.5, block 64 at 26 34.5 ->
+// 26.1. Its set-up is longer: 2 x 100 5.1 -> 5.9. Beyond one item per SM its items come one after the other, set-up and all:
+// 32 x 1900 58 -> 77.
+inline bool lone_ctas_pay(long long items, long long keys, int max_ctas) {
+  return items <= max_ctas / 2 && keys >= 256;
 }
 
 }  // namespace sparsed

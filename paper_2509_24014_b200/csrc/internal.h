@@ -156,6 +156,11 @@ cudaError_t launch_attn_dense_pair_split(const CUtensorMap& tq, const CUtensorMa
 int attn_sparse_max_blocks(int block_size);   // most key blocks per row the sparse kernel handles
 cudaError_t launch_attn_sparse(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv,
                                const CUtensorMap& to, const AttnParams& p, int block_size, cudaStream_t stream);
+// Both in CTAs that have an SM each, for grids of no more query tiles than the device has SMs (attention_lone.cu)
+cudaError_t launch_attn_sparse_lone(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv,
+                                    const AttnParams& p, int block_size, cudaStream_t stream);
+cudaError_t launch_attn_dense_lone(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv,
+                                   const AttnParams& p, cudaStream_t stream);
 bool score_ranks_in_kernel(int nb, int block_size);   // the pooled-scoring kernel ranks rows of nb key blocks itself
 bool score_in_one_pass(int nb);                       // ... and needs no log-sum-exp of the rows
 // (K tensor map of both: boxes of 64 x 64 rows)

@@ -286,27 +286,23 @@ __device__ __forceinline__ void store_output_row(uint32_t t_acc_row, bool have_a
   }
 }
 
-// O / l -> bf16, this thread's row, from tensor memory into a shared-memory tile from which a TMA store
-// writes the whole 128-row tile out. (Storing each row from its own thread instead - 32 different cache lines
-// per warp instruction - was measured at about 6000 clocks per 128-row tile.)
-// tile: 128 rows x 128 columns of bf16 as two 64-column halves of 128 rows x 128 bytes (16 KB each, 1024-byte
-// aligned), 128-byte swizzle as the tensor maps use it: the 16-byte chunk c of row r sits at chunk c ^ (r & 7).
-// t_acc_row: the row's tensor-memory address; have_acc = false writes zeros (empty key list).
-__device__ __forceinline__ void stage_output_row(uint32_t t_acc_row, bool have_acc, float inv_l, __nv_bfloat16* tile,
-                                                 int row) {
-  uint8_t* base = reinterpret_cast<uint8_t*>(tile) + row * 128;
+// O / l -> bf16, 64 columns of this thread's row, from tensor memory into a shared-memory tile of 128 rows x 64 columns of
+// bf16 (128 bytes a row; 1024-byte aligned), 128-byte swizzle as the tensor maps use it: the 16-byte chunk c of row r sits
+// at chunk c ^ (r & 7). t_acc: the columns' tensor-memory address in this row; have_acc = false writes zeros.
+__device__ __forceinline__ void stage_output_half(uint32_t t_acc, bool have_acc, float inv_l, __nv_bfloat16* half_tile,
+                                                  int row) {
+  uint8_t* base = reinterpret_cast<uint8_t*>(half_tile) + row * 128;
   const int sw = row & 7;
 #pragma unroll
-  for (int c = 0; c < 4; ++c) {   // 32 columns each: chunks 4 (c & 1) .. +3 of half c >> 1
+  for (int c = 0; c < 2; ++c) {   // 32 columns each: chunks 4c .. 4c + 3
     uint32_t r[32];
     if (have_acc) {
-      tmem_ld32(t_acc_row + c * 32, r);
+      tmem_ld32(t_acc + c * 32, r);
       tmem_wait_ld();
     } else {
 #pragma unroll
       for (int j = 0; j < 32; ++j) r[j] = 0u;
     }
-    uint8_t* half = base + (c >> 1) * (128 * 128);
 #pragma unroll
     for (int g = 0; g < 4; ++g) {
       uint4 out;
@@ -318,9 +314,18 @@ __device__ __forceinline__ void stage_output_row(uint32_t t_acc_row, bool have_a
                           mul_keep_denormals(__uint_as_float(r[8 * g + 5]), inv_l));
       out.w = pack_bf16x2(mul_keep_denormals(__uint_as_float(r[8 * g + 6]), inv_l),
                           mul_keep_denormals(__uint_as_float(r[8 * g + 7]), inv_l));
-      *reinterpret_cast<uint4*>(half + (((4 * (c & 1) + g) ^ sw) << 4)) = out;
+      *reinterpret_cast<uint4*>(base + (((4 * c + g) ^ sw) << 4)) = out;
     }
   }
+}
+
+// The whole row (tile: two such half tiles, 16 KB each), from which a TMA store writes the 128-row tile out. (Storing each
+// row from its own thread instead - 32 different cache lines per warp instruction - was measured at about 6000 clocks per
+// 128-row tile.)
+__device__ __forceinline__ void stage_output_row(uint32_t t_acc_row, bool have_acc, float inv_l, __nv_bfloat16* tile,
+                                                 int row) {
+  stage_output_half(t_acc_row, have_acc, inv_l, tile, row);
+  stage_output_half(t_acc_row + 64, have_acc, inv_l, tile + 128 * 64, row);
   fence_proxy_async_smem();   // the TMA store reads these writes through the async proxy
 }
 
@@ -352,6 +357,20 @@ __device__ __forceinline__ void issue_qk64(uint32_t tmem_s, uint32_t q_lo, uint3
                           k_lo + (kk >> 2) * UmmaTile64::kHalfStep + (kk & 3) * 2, UmmaTile64::kHi,
                           UmmaTile64::kIdescQK);
     }
+    umma_commit(done);
+  }
+  __syncwarp();
+}
+
+// The same with Q (bf16 pairs, 64 columns) read from tensor memory.
+__device__ __forceinline__ void issue_qk64_ts(uint32_t tmem_s, uint32_t tmem_q, uint32_t k_lo, uint64_t* done) {
+  tc_fence_after();
+  if (elect_one_sync()) {
+    umma_ts_words(tmem_s, tmem_q, k_lo, UmmaTile64::kHi, UmmaTile64::kIdescQK, 0u);
+#pragma unroll
+    for (int kk = 1; kk < 8; ++kk)
+      umma_ts_words(tmem_s, tmem_q + kk * 8, k_lo + (kk >> 2) * UmmaTile64::kHalfStep + (kk & 3) * 2, UmmaTile64::kHi,
+                    UmmaTile64::kIdescQK, 1u);
     umma_commit(done);
   }
   __syncwarp();

@@ -1,0 +1,52 @@
+"""Grids of up to one query tile per SM run on a kernel of their own (one CTA to an SM, two groups of softmax warps): it
+must give bitwise what the other kernels give, from the fewest tiles of keys it takes on to rings that wrap around,
+whether references stay or move with every tile."""
+import pytest
+import torch
+
+import paper_2509_24014_b200 as sd
+from tests.parity_util import gpu_full, gpu_sparse
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda"
+
+
+def _inputs(H, Hkv, L, seed, rising):
+    g = torch.Generator(device=DEV).manual_seed(seed)
+    q = torch.randn(1, H, L, 128, generator=g, device=DEV).bfloat16()
+    k, v = (torch.randn(1, Hkv, L, 128, generator=g, device=DEV).bfloat16() for _ in range(2))
+    if rising:   # logits that keep outgrowing the reference
+        k = (k * torch.linspace(0.2, 14.0, L, device=DEV)[:, None]).bfloat16()
+    return q, k, v
+
+
+@pytest.mark.parametrize("rising", [False, True])
+@pytest.mark.parametrize("L", [256, 257, 300, 384, 449, 640, 700, 1473])   # 4 to 24 tiles, ragged by 1 to 63 keys
+def test_dense_equals_the_kernels_of_larger_grids(L, rising):
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    few = sms // ((L + 127) // 128)
+    q, k, v = _inputs(few + 2, few + 2, L, 71, rising)
+    o_all, lse_all = gpu_full(q, k, v)                                           # more query tiles than SMs
+    o, lse = gpu_full(*(t[:, :few].contiguous() for t in (q, k, v)))
+    assert torch.equal(o, o_all[:, :few]) and torch.equal(lse, lse_all[:, :few])
+
+
+@pytest.mark.parametrize("rising", [False, True])
+@pytest.mark.parametrize("bs,L", [(128, 1280), (64, 1344), (32, 1376), (32, 608), (128, 8192)])
+def test_sparse_equals_the_kernels_of_larger_grids(bs, L, rising):
+    """Lists of every length, empty ones among them (128-key blocks, 8192 tokens: more than the 32 ids fetched at once)."""
+    H, Hkv, nb = (2, 1, L // bs)
+    q, k, v = _inputs(H, Hkv, L, 72, rising)
+    g = torch.Generator(device=DEV).manual_seed(73)
+    keep = torch.rand(H, nb, nb, generator=g, device=DEV) < torch.rand(H, nb, 1, generator=g, device=DEV) * 1.3
+    keep &= torch.rand(H, nb, 1, generator=g, device=DEV) < 0.9
+    keep[:, 1] = False
+    keep[:, 2] = True
+    row_ptr = torch.zeros(H * nb + 1, dtype=torch.int32, device=DEV)
+    row_ptr[1:] = keep.sum(-1).flatten().cumsum(0)
+    col_idx = keep.flatten(0, 1).nonzero()[:, 1].to(torch.int32).contiguous()
+    pat = sd.pattern_from_csr(row_ptr, col_idx, bs, nb, 1, H)
+    assert pat.nnz == col_idx.numel() and pat.nnz * bs >= 256 * H * nb   # long enough for the kernel under test
+    o = gpu_sparse(q, k, v, pat)
+    pat.nnz = 0                                                          # not told how long the lists are: the others
+    assert torch.equal(o, gpu_sparse(q, k, v, pat))
