@@ -32,8 +32,8 @@
 //   28 heads x 16384 tokens, block 128   6.21 -> 2.43 ms (kOnePass; exponential unit busy 73 % of the time on average over
 //                                        the SMs and 84 % on the busiest, at 4 heads: 1.73 waves)
 //   32 heads x 8192 tokens, block 128    1.79 -> 0.72 ms (kOnePass)
-//   28 heads x 16384 tokens, block 64    6.24 -> 3.29 ms (kOnePassWide; in two passes 5.0)
-//   8 heads x 65536 tokens, block 128    27.4 -> 14.0 ms (kOnePassMost; in two passes 22.3)
+//   28 heads x 16384 tokens, block 64    6.24 -> 3.00 ms (kOnePassWide; in two passes 5.0)
+//   8 heads x 65536 tokens, block 128    27.4 -> 12.8 ms (kOnePassMost; in two passes 22.3)
 //   8 heads x 65536 tokens, block 64     27.6 -> 21.9 ms (kRowStats, kPooled)
 // and with the caller's LSE (kPooled, one pass before as well):
 //   28 heads x 16384 tokens, block 128   2.48 -> 2.38 ms
@@ -61,6 +61,12 @@ __host__ __device__ constexpr int tmem_cols(int mode) { return one_per_sm(mode) 
 __host__ __device__ constexpr int tmem_sums(int mode) { return tmem_cols(mode) - kColStat; }
 __host__ __device__ constexpr int smem_sums(int mode) { return mode == kOnePassMost ? 128 : 0; }
 __host__ __device__ constexpr int block_sums(int mode) { return tmem_sums(mode) + smem_sums(mode); }
+
+// Of 16 pairs of exponentials, how many are taken off the exponential unit (exp2_by_polynomial, 16 instructions a pair).
+// Only where one CTA per SM leaves issue slots: 28 x 16384 block 64 3292 -> 2996 us with two, 3078 with three, 2982 with
+// four; 8 x 65536 block 128 14040 -> 13266, 12800, 13108. With two CTAs per SM the launch is at its power limit instead
+// (28 x 16384 block 128 2458, 2460, 2443, 2493), or short of work (2 x 1024 13.9, 13.9, 14.8, 14.6).
+__host__ __device__ constexpr int poly_pairs(int mode) { return mode == kOnePassMost ? 3 : mode == kOnePassWide ? 2 : 0; }
 
 // A row's reference is the maximum of both groups' first 64-key tiles, and stays until the sum of a later tile outgrows
 // this: only fp32 sums are taken here (no bf16 probabilities), so 2^60 is as safe as 1. Sums may thus stand up to 2^66
@@ -118,7 +124,36 @@ __device__ __forceinline__ float warp_column_sums(float (&v)[32], int lane) {
   return v[0];
 }
 
-// Sum of 2^(scale * s - m) over 32 columns.
+__device__ __forceinline__ float2 twice(float c) { return make_float2(c, c); }
+
+// 2^x without the exponential unit: x = n + f with n whole and |f| <= 1/2, 2^f by the polynomial of degree 6 with the least
+// largest relative error there (1.9e-9, found by Lawson's reweighted least squares; 7.8e-8 with its fp32 roundings, where
+// ex2.approx has 2^-22), times 2^n put together from its bits. The clamps keep n in [-127, 128], whose bits are those of 0
+// and infinity, and hand NaN on.
+__device__ __forceinline__ float2 exp2_by_polynomial(float2 x) {
+  auto clamp = [](float v) -> float {
+    float y;
+    asm("max.NaN.f32 %0, %1, 0fC2FE0000;" : "=f"(y) : "f"(v));   // -127
+    asm("min.NaN.f32 %0, %1, 0f43000000;" : "=f"(y) : "f"(y));   // 128
+    return y;
+  };
+  x = make_float2(clamp(x.x), clamp(x.y));
+  const float2 t = __fadd2_rn(x, twice(12582912.f));   // 1.5 * 2^23 + n: n in the low bits
+  const float2 f = __fadd2_rn(x, __ffma2_rn(t, twice(-1.f), twice(12582912.f)));
+  float2 y = twice(0x1.41d332d89fe66p-13f);
+  y = __ffma2_rn(y, f, twice(0x1.5f456a8954f25p-10f));
+  y = __ffma2_rn(y, f, twice(0x1.3b2dbbc1d72d0p-7f));
+  y = __ffma2_rn(y, f, twice(0x1.c6aed4b954772p-5f));
+  y = __ffma2_rn(y, f, twice(0x1.ebfbdadcaf7c8p-3f));
+  y = __ffma2_rn(y, f, twice(0x1.62e430c7e91fcp-1f));
+  y = __ffma2_rn(y, f, twice(1.f));
+  return __fmul2_rn(y, make_float2(__uint_as_float(__float_as_uint(t.x) * 8388608u + 0x3f800000u),
+                                   __uint_as_float(__float_as_uint(t.y) * 8388608u + 0x3f800000u)));
+}
+
+// Sum of 2^(scale * s - m) over 32 columns, kPairs of its 16 pairs of exponentials by the polynomial. (The same columns of
+// every 32 keys, so that equal key blocks have equal sums.)
+template <int kPairs>
 __device__ __forceinline__ float exp_sum(const uint32_t (&r)[32], float scale_log2, float m) {
   const float2 sc = make_float2(scale_log2, scale_log2);
   const float2 nm = make_float2(-m, -m);
@@ -127,8 +162,9 @@ __device__ __forceinline__ float exp_sum(const uint32_t (&r)[32], float scale_lo
   for (int j = 0; j < 8; ++j) {
     const float2 x0 = __ffma2_rn(make_float2(__uint_as_float(r[4 * j]), __uint_as_float(r[4 * j + 1])), sc, nm);
     const float2 x1 = __ffma2_rn(make_float2(__uint_as_float(r[4 * j + 2]), __uint_as_float(r[4 * j + 3])), sc, nm);
+    const bool polynomial = (kPairs == 2 && j % 4 == 1) || (kPairs == 3 && (j == 1 || j == 4 || j == 6));   // spread evenly
     a0 = __fadd2_rn(a0, make_float2(fast_exp2(x0.x), fast_exp2(x0.y)));
-    a1 = __fadd2_rn(a1, make_float2(fast_exp2(x1.x), fast_exp2(x1.y)));
+    a1 = __fadd2_rn(a1, polynomial ? exp2_by_polynomial(x1) : make_float2(fast_exp2(x1.x), fast_exp2(x1.y)));
   }
   const float2 a = __fadd2_rn(a0, a1);
   return a.x + a.y;
@@ -353,8 +389,8 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
       if (lane == 0) mbar_arrive(&sm.s_free[g]);
       const int valid_cols = p.seq_len - t * kTileN;   // ragged tail of the sequence
       if (valid_cols < kTileN) mask_columns_from(r0, r1, valid_cols);
-      float s0 = exp_sum(r0, scale_log2, m);
-      float s1 = exp_sum(r1, scale_log2, m);
+      float s0 = exp_sum<poly_pairs(kMode)>(r0, scale_log2, m);
+      float s1 = exp_sum<poly_pairs(kMode)>(r1, scale_log2, m);
       if constexpr (kMode != kPooled) {
         const bool outgrown = !(s0 + s1 <= kOutgrown);   // no reference yet (m = -inf), far larger logits, or NaN
         if (__any_sync(0xffffffffu, outgrown)) {
@@ -368,8 +404,8 @@ score_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ C
           l *= alpha.far * alpha.near;
           // a row whose logits so far are all -inf: 2^(-inf - 0) = 0, not NaN
           const float ref = m == -INFINITY ? 0.f : m;
-          s0 = exp_sum(r0, scale_log2, ref);
-          s1 = exp_sum(r1, scale_log2, ref);
+          s0 = exp_sum<poly_pairs(kMode)>(r0, scale_log2, ref);
+          s1 = exp_sum<poly_pairs(kMode)>(r1, scale_log2, ref);
           if constexpr (kKeepsSums) {
             carry = carry * alpha.far * alpha.near;
             // (columns of the other group are left alone; its threads rescale theirs)

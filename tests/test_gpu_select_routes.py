@@ -154,3 +154,16 @@ def test_references_that_move_at_any_tile_of_a_block(bs, tiles, rises):
     p[p < 2.0 ** -120] = 0.0
     np.testing.assert_allclose(scores[0, 0].cpu().numpy(), np.broadcast_to(p.numpy(), (nb, nb)), rtol=16 * SCORE_RTOL,
                                atol=2.0 ** -120)
+
+
+@pytest.mark.parametrize("bs,nb", [(32, 64), (32, 200), (32, 500)])
+@pytest.mark.parametrize("key", [0, 6, 18, 26, 31])
+def test_a_key_of_nan_makes_every_score_nan(bs, nb, key):
+    """Whichever way a column's exponentials are taken (with 129 to 512 key blocks per row, columns 6, 18 and 26 of 32 are
+    among those that do without the exponential unit)."""
+    g = torch.Generator(device=DEV).manual_seed(76)
+    q, k = (torch.randn(1, 1, nb * bs, 128, generator=g, device=DEV).bfloat16() for _ in range(2))
+    k[0, 0, 7 * 32 + key] = float("nan")
+    _, _, col_idx, scores = gpu_select(q, k, bs, 0.2, 0)
+    assert torch.isnan(scores).all()
+    assert int(col_idx.min()) >= 0 and int(col_idx.max()) < nb
