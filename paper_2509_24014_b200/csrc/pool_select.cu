@@ -8,16 +8,20 @@
 // puts on key block g, so A'[ib][jb] is the sum of that mass over the rows of query block ib,
 // divided by block_size^2.
 //
-// One CTA owns one 128-row query tile of one (batch, head), i.e. one, two or four query blocks.
-// Statistics are read with 16-byte loads (four consecutive rows of one key block; the layout
-// [bh][128-row query tile][key block][row] makes a CTA's reads one contiguous run), eight in flight
-// per thread and six CTAs per SM (the best point of a sweep: 5.9 TB/s at 64k), exponentiated,
-// parked in shared memory in chunks of 32 key blocks, and summed per key block and 32-row quarter
-// in a fixed, bank-conflict-free order (bitwise reproducible); the next chunk's loads are issued
-// before the current chunk is summed. The quarters are then combined into the CTA's block-row(s)
-// of A', which are optionally written out, and one warp per block-row ranks it (warp_select_row)
-// and writes the CSR list. HBM-bound: 4 * 128 * ceil(L/128) * (L / block_size) bytes read per
-// (batch, head).
+// One CTA owns one 128-row query tile of one (batch, head), i.e. one, two or four query blocks. Its statistics are one
+// contiguous run (layout [bh][128-row query tile][key block][row]), read by four warps that go their own ways: a warp takes
+// eight key blocks at a time, lane l of it rows 4l .. 4l + 3 of each in one 16-byte load, and asks for the next eight as
+// soon as it has taken the exponentials of these. A lane's four rows are added up, then the eight lanes of a 32-row
+// quarter by a butterfly that leaves each lane with one key block of the eight (seven shuffles for all; a fixed tree, the
+// same for every key block: bitwise reproducible). The quarters are then combined into the CTA's block-row(s) of A',
+// which are optionally written out, and one warp per block-row ranks it (warp_select_row) and writes the CSR list.
+// HBM-bound: 4 * 128 * ceil(L/128) * (L / block_size) bytes read per (batch, head).
+//
+// Seven CTAs per SM are the most whose registers do not spill. 32 heads, block 128: 65536 tokens 776 -> 643 us (4.3 GB: 6.7
+// TB/s), 16384 (28 heads) 60 -> 52, 8192 27.7 -> 22; block 32, 4096 tokens 28 -> 23 - before, the exponentials went through
+// shared memory, 32 key blocks at a time with two barriers each, to be added up by one lane per key block, six CTAs per SM.
+// (With two batches of loads in flight, five CTAs: 8 heads x 65536 196 us against 187; six or eight CTAs 193, 189. What is
+// left at 8192 is one CTA's own chain, 6 us from its first load to its ranked row.)
 #include "internal.h"
 #include "topk_device.cuh"
 
@@ -25,55 +29,46 @@ namespace sparsed {
 namespace {
 
 constexpr int kRows = 128;
-#ifndef SPARSED_POOL_IN_FLIGHT
-#define SPARSED_POOL_IN_FLIGHT 8
-#endif
-#ifndef SPARSED_POOL_CTAS_PER_SM
-#define SPARSED_POOL_CTAS_PER_SM 6
-#endif
-constexpr int kInFlight = SPARSED_POOL_IN_FLIGHT;  // 16-byte loads each thread keeps in flight
-constexpr int kChunk = 4 * kInFlight;  // tiles per transposition chunk: one batch of loads per thread
-constexpr int kPitch = kRows + 4;   // floats per chunk row: keeps float4 stores aligned
+constexpr int kCtasPerSm = 7;
+constexpr int kBatch = 8;           // key blocks a warp takes at a time: 16-byte loads each thread has in flight
 constexpr int kMaxBlocks = 2048;    // key blocks per row: seq_len <= 2048 * block_size
 
-// Shared memory (dynamic, sized for the actual sequence): the transposition chunk, the per-block
-// mass of each 32-row quarter of the query tile, the ordered keys of this CTA's block-row(s), one
-// top-k histogram per block-row.
+// Floats between the quarters' sums of one key block: four quarters of eight key blocks then lie in 32 different banks.
+__host__ __device__ constexpr int quarter_pitch(int nb) { return (nb + 31) / 32 * 32 + 8; }
+
+// Shared memory (dynamic, sized for the actual sequence): the per-block mass of each 32-row quarter of the query tile, the
+// ordered keys of this CTA's block-row(s), one top-k histogram per block-row.
 struct PoolSmem {
-  float* chunk;                     // [key block in chunk][kPitch]
   float* quarter_sum;               // [32-row quarter][key block]
   uint32_t* keys;                   // [block-row of this CTA][key block]
   int* hist;                        // [block-row][256]
 };
 
 __host__ __device__ inline size_t pool_smem_bytes(int nb, int rows_here) {
-  return sizeof(float) * kChunk * kPitch + sizeof(float) * 4 * nb + sizeof(uint32_t) * rows_here * nb +
-         sizeof(int) * 256 * rows_here;
+  return sizeof(float) * 4 * quarter_pitch(nb) + sizeof(uint32_t) * rows_here * nb + sizeof(int) * 256 * rows_here;
 }
 
-__global__ void __launch_bounds__(kRows, SPARSED_POOL_CTAS_PER_SM) pool_select_kernel(const PoolParams p) {
+__global__ void __launch_bounds__(kRows, kCtasPerSm) pool_select_kernel(const PoolParams p) {
   extern __shared__ __align__(16) uint8_t pool_smem_raw[];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int L = p.seq_len;
   const int bs = p.block_size;
   const int nb = L / bs;                    // key blocks per row = statistics per row
   const int rows_here = kRows / bs;         // block-rows of A' this CTA produces: 1, 2 or 4
+  const int pitch = quarter_pitch(nb);
   PoolSmem sm;
   {
     float* f = reinterpret_cast<float*>(pool_smem_raw);
-    sm.chunk = f;
-    f += kChunk * kPitch;
     sm.quarter_sum = f;
-    f += 4 * nb;
+    f += 4 * pitch;
     sm.keys = reinterpret_cast<uint32_t*>(f);
     sm.hist = reinterpret_cast<int*>(sm.keys + rows_here * nb);
   }
   const int num_q_tiles = (L + kRows - 1) / kRows;
   const int q_tile = blockIdx.x % num_q_tiles;
   const int bh = blockIdx.x / num_q_tiles;
-  // Loading: lane l owns rows 4l..4l+3 of the query tile (one 16-byte load covers them), warp w
-  // takes key blocks w, w+4, ... of the chunk. seq_len is a multiple of 32 here, so a group of four
-  // rows is valid or invalid as a whole and 16-byte aligned.
+  // Lane l owns rows 4l..4l+3 of the query tile. seq_len is a multiple of 32 here, so a group of four rows is valid or
+  // invalid as a whole and 16-byte aligned.
   const int row4 = q_tile * kRows + lane * 4;
   const bool rows_valid = row4 < L;
   float4 lse2 = make_float4(INFINITY, INFINITY, INFINITY, INFINITY);
@@ -85,56 +80,43 @@ __global__ void __launch_bounds__(kRows, SPARSED_POOL_CTAS_PER_SM) pool_select_k
   // statistics layout [bh][query tile][key block][128 rows]: this CTA's share is one contiguous run
   const float* src = p.tile_lse + (static_cast<int64_t>(bh) * num_q_tiles + q_tile) * nb * kRows + lane * 4;
 
-  // One batch = this thread's kInFlight loads of a chunk (warp w takes key blocks w, w+4, ... of it).
-  // The next chunk's batch is issued before the current chunk is summed, so loads stay in flight
-  // through the shared-memory phase.
-  static_assert(kChunk == 4 * kInFlight, "one batch of loads per thread covers one chunk");
-  static_assert(kChunk == 32, "the summation assigns one key block of the chunk to each lane");
-  float4 v[kInFlight];
-  auto issue = [&](int c0) {
-    const int n_here = min(kChunk, nb - c0);
+  auto load = [&](float4 (&v)[kBatch], int jb0) {
 #pragma unroll
-    for (int u = 0; u < kInFlight; ++u) {
-      const int t = warp + 4 * u;
-      v[u] = (rows_valid && t < n_here)
-                 ? __ldcs(reinterpret_cast<const float4*>(src + static_cast<int64_t>(c0 + t) * kRows))
-                 : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
-    }
+    for (int u = 0; u < kBatch; ++u)
+      v[u] = (rows_valid && jb0 + u < nb) ? __ldcs(reinterpret_cast<const float4*>(src + static_cast<int64_t>(jb0 + u) * kRows))
+                                          : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
   };
-  issue(0);
-  for (int c0 = 0; c0 < nb; c0 += kChunk) {
-    const int n_here = min(kChunk, nb - c0);
+  constexpr int kStep = 4 * kBatch;   // of the four warps together
+  float4 v[kBatch];
+  load(v, warp * kBatch);
+  for (int jb0 = warp * kBatch; jb0 < nb; jb0 += kStep) {
+    // this lane's four rows' mass on the key blocks [jb0, jb0 + 8)
+    float m[kBatch];
 #pragma unroll
-    for (int u = 0; u < kInFlight; ++u) {
-      const int t = warp + 4 * u;
-      if (t < n_here) {
-        const float4 e = make_float4(fast_exp2(v[u].x - lse2.x), fast_exp2(v[u].y - lse2.y),
-                                     fast_exp2(v[u].z - lse2.z), fast_exp2(v[u].w - lse2.w));
-        *reinterpret_cast<float4*>(sm.chunk + t * kPitch + lane * 4) = e;
+    for (int u = 0; u < kBatch; ++u)
+      m[u] = (fast_exp2(v[u].x - lse2.x) + fast_exp2(v[u].y - lse2.y)) +
+             (fast_exp2(v[u].z - lse2.z) + fast_exp2(v[u].w - lse2.w));
+    load(v, jb0 + kStep);
+    // ... the quarter's: eight lanes', key block jb0 + (lane & 7) left in each
+#pragma unroll
+    for (int half = kBatch / 2; half > 0; half >>= 1) {
+      const bool upper = (lane & half) != 0;
+#pragma unroll
+      for (int u = 0; u < half; ++u) {
+        const float keep = upper ? m[u + half] : m[u];
+        const float give = upper ? m[u] : m[u + half];
+        m[u] = keep + __shfl_xor_sync(0xffffffffu, give, half);
       }
     }
-    __syncthreads();
-    if (c0 + kChunk < nb) issue(c0 + kChunk);
-    {
-      // Summing: warp w adds rows 32w..32w+31 (one quarter of the query tile), lane j key block j of
-      // the chunk. Each lane starts at its own rotation of the 32 rows so that a warp's reads hit 32
-      // different banks; the order is fixed per key block, so the result is reproducible.
-      const int j = lane;
-      if (j < n_here) {
-        const float* rowp = sm.chunk + j * kPitch + warp * 32;
-        float acc = 0.f;
-#pragma unroll 8
-        for (int r = 0; r < 32; ++r) acc += rowp[(r + 29 * j) & 31];
-        sm.quarter_sum[warp * nb + c0 + j] = acc;
-      }
-    }
-    __syncthreads();
+    const int jb = jb0 + (lane & 7);
+    if (jb < nb) sm.quarter_sum[(lane >> 3) * pitch + jb] = m[0];
   }
+  __syncthreads();
 
   const float inv_area = 1.f / (static_cast<float>(bs) * static_cast<float>(bs));
   for (int jb = tid; jb < nb; jb += kRows) {
-    const float q0 = sm.quarter_sum[jb], q1 = sm.quarter_sum[nb + jb], q2 = sm.quarter_sum[2 * nb + jb],
-                q3 = sm.quarter_sum[3 * nb + jb];
+    const float q0 = sm.quarter_sum[jb], q1 = sm.quarter_sum[pitch + jb], q2 = sm.quarter_sum[2 * pitch + jb],
+                q3 = sm.quarter_sum[3 * pitch + jb];
     float score[4];
     if (bs == 128) {
       score[0] = ((q0 + q1) + (q2 + q3)) * inv_area;
