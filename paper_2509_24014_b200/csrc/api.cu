@@ -354,9 +354,8 @@ sparsed_status sparsed_workspace_init(void* ws, size_t ws_bytes, void* cuda_stre
   return e == cudaSuccess ? SPARSED_OK : cuda_fail(e);
 }
 
-// Which dense kernel runs. The pass that also records row statistics has one kernel, the CTA-pair one. The
-// environment variable SPARSED_DENSE_KERNEL (read once) sends every plain pass to one of them, `pair`, `single` or
-// `lone`, for A/B measurements and tests.
+// Which dense kernel runs. The single-CTA one records no row statistics. The environment variable SPARSED_DENSE_KERNEL
+// (read once) sends every plain pass to one of them, `pair`, `single` or `lone`, for A/B measurements and tests.
 enum DenseKernel { kSingle, kPair, kLone };
 static DenseKernel dense_kernel(bool with_stats, const sparsed_shape* shape, int max_ctas) {
   static const int forced = [] {
@@ -366,10 +365,10 @@ static DenseKernel dense_kernel(bool with_stats, const sparsed_shape* shape, int
     if (v != nullptr && std::strcmp(v, "lone") == 0) return static_cast<int>(kLone);
     return -1;
   }();
-  if (with_stats) return kPair;
-  if (forced >= 0) return static_cast<DenseKernel>(forced);
+  if (!with_stats && forced >= 0) return static_cast<DenseKernel>(forced);
   const long long bh = static_cast<long long>(shape->batch) * shape->heads_q;
   if (lone_ctas_pay(bh * ((static_cast<long long>(shape->seq_len) + 127) / 128), shape->seq_len, max_ctas)) return kLone;
+  if (with_stats) return kPair;
   return dense_pair_pays(bh, shape->seq_len, max_ctas) ? kPair : kSingle;
 }
 

@@ -24,7 +24,7 @@
 // Where the keys come from:
 //   * dense: every 64-key tile of the sequence in order; the last one may be ragged (any seq_len).
 //     Optional output: the rows' LSE. (The dense pass that also records the row statistics of the switch
-//     step runs on a kernel of its own, attention_dense_pair.cu.)
+//     step runs on the kernels of attention_dense_pair.cu and, on small grids, attention_lone.cu.)
 //   * 128-key blocks: the 128 query rows are one query block; its CSR list is walked as it is,
 //     two tiles per block.
 //   * 64- and 32-key blocks: the 128 query rows are two / four consecutive query blocks with lists

@@ -1,4 +1,4 @@
-// Attention (dense, and block-sparse over CSR block lists) for grids of no more query tiles than the device has SMs: the
+// Attention (dense, with or without the row statistics of the switch step, and block-sparse over CSR block lists) for grids of no more query tiles than the device has SMs: the
 // work of attention.cu, bit for bit, by a CTA that has an SM to itself.
 //
 // What bounds such a grid is one CTA's chain of 64-key tiles. In attention.cu that is 1290 clocks a tile: one warp issues
@@ -64,6 +64,7 @@ struct LoneSmem {
   uint64_t p_full[kSBuffers];
   uint64_t turn[2][4];       // [group][32-row quarter]: the other group has passed the rows' state on
   float2 state[kTileM];      // reference maximum and sum of each row, after the last tile done with
+  float carry[kTileM];       // 128-key statistics: the sum over the group's first tile (group 0's) for group 1's
   uint32_t tmem_base;
   int abort_flag;
   int entries;               // packed walks: key blocks in the union, and the union (work_items.cuh)
@@ -71,7 +72,8 @@ struct LoneSmem {
   uint32_t member[kGroups][kMemberWords<kBlock>];
 };
 
-template <int kBlock, bool kDense>
+// kStatKeys: record one row statistic per 32 / 64 / 128 keys (RowStatWriter in softmax_pipeline.cuh), or none (0).
+template <int kBlock, bool kDense, int kStatKeys>
 __global__ void __launch_bounds__(kThreads, 1)
 attn_lone_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                  const __grid_constant__ CUtensorMap tm_v, const AttnParams p) {
@@ -256,6 +258,11 @@ attn_lone_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
       if (lane == 0) mbar_arrive(&sm.q_ready);
     }
     RowState st{-INFINITY, 0.f};
+    // this row's first statistic
+    [[maybe_unused]] float* stats = nullptr;
+    [[maybe_unused]] const int stat_groups = kStatKeys > 0 ? (p.seq_len + kStatKeys - 1) / kStatKeys : 0;
+    if (kStatKeys > 0 && it.q_row0 + row_in_tile < p.seq_len)
+      stats = p.tile_lse + (static_cast<int64_t>(it.bh) * p.num_q_tiles + it.q_tile) * stat_groups * kTileM + row_in_tile;
     // takes over the row's state after the other group's nth tile
     auto take_state = [&](int nth) -> bool {
       if (!wait(&sm.turn[g][quarter], nth & 1, 76)) return false;
@@ -280,6 +287,7 @@ attn_lone_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
       const int valid_cols = kDense ? p.seq_len - t * kTileN : kTileN;   // ragged tail of the sequence
       uint32_t pk[32];
       float2 sums = make_float2(0.f, 0.f);
+      [[maybe_unused]] float carry = 0.f;   // 128-key statistics: the tile before this one, in group 1
       bool tried = false;   // pk and sums hold the tile against st.m (where that is a number)
       auto load_logits = [&](uint32_t (&r0)[32], uint32_t (&r1)[32]) {
         tmem_ld32(tS, r0);
@@ -310,6 +318,7 @@ attn_lone_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
       if (t > 0) {
         const float m = st.m;
         if (!(ok = take_state((t - 1) >> 1))) break;   // after tile t - 1
+        if (kStatKeys == 128 && g == 1) carry = sm.carry[row_in_tile];
         if (kept && __any_sync(0xffffffffu, m != st.m)) fast();
       }
       if (kept) {
@@ -326,6 +335,7 @@ attn_lone_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
             for (int j = 0; j < 32; ++j) r1[j] = 0xff800000u;
           }
           const float alpha = softmax_group_exact(r0, r1, scale_log2, st, pk, sums);
+          if constexpr (kStatKeys == 128) carry *= alpha;
           if (t > 0) {
             // O must be quiescent: wait until P_{t-1} V_{t-1} has drained
             const TilePos last(t - 1);
@@ -341,6 +351,7 @@ attn_lone_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
         for (int j = 0; j < 32; ++j) pk[j] = 0u;
       }
       sm.state[row_in_tile] = make_float2(st.m, st.l);
+      if (kStatKeys == 128 && g == 0) sm.carry[row_in_tile] = sums.x + sums.y;
       __syncwarp();
       if (lane == 0) mbar_arrive(&sm.turn[g ^ 1][quarter]);
       tmem_st32(tS, pk);  // P_t over the first 32 columns of S_t
@@ -348,6 +359,15 @@ attn_lone_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(&sm.p_full[t % kSBuffers]);
+      if (kStatKeys > 0 && stats != nullptr) {
+        if constexpr (kStatKeys == 64) __stcs(stats + t * kTileM, st.m + fast_log2(sums.x + sums.y));
+        if constexpr (kStatKeys == 32) {
+          __stcs(stats + 2 * t * kTileM, st.m + fast_log2(sums.x));
+          if (2 * t + 1 < stat_groups) __stcs(stats + (2 * t + 1) * kTileM, st.m + fast_log2(sums.y));
+        }
+        // (the sequence is a whole number of 128-key groups here: each ends with a tile of group 1)
+        if (kStatKeys == 128 && g == 1) __stcs(stats + (t >> 1) * kTileM, st.m + fast_log2(carry + (sums.x + sums.y)));
+      }
     }
     // ---- epilogue: O / l -> bf16 -> shared memory -> global, 64 columns of head_dim per group ----------------------
     const int row = it.q_row0 + row_in_tile;
@@ -402,10 +422,10 @@ attn_lone_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant
   }
 }
 
-template <int kBlock, bool kDense>
+template <int kBlock, bool kDense, int kStatKeys>
 cudaError_t launch(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv, const AttnParams& p,
                    cudaStream_t stream) {
-  auto kernel = attn_lone_kernel<kBlock, kDense>;
+  auto kernel = attn_lone_kernel<kBlock, kDense, kStatKeys>;
   const int smem = static_cast<int>(sizeof(LoneSmem<kBlock>));
   static_assert(sizeof(LoneSmem<kBlock>) > 114 * 1024 && sizeof(LoneSmem<kBlock>) <= 227 * 1024, "one CTA per SM");
   static SmemLimit limit;  // per template instantiation
@@ -420,14 +440,17 @@ cudaError_t launch(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorM
 // Tensor maps of both as in attention.cu.
 cudaError_t launch_attn_sparse_lone(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv,
                                     const AttnParams& p, int block_size, cudaStream_t stream) {
-  if (block_size == 128) return launch<128, false>(tq, tk, tv, p, stream);
-  if (block_size == 64) return launch<64, false>(tq, tk, tv, p, stream);
-  return launch<32, false>(tq, tk, tv, p, stream);
+  if (block_size == 128) return launch<128, false, 0>(tq, tk, tv, p, stream);
+  if (block_size == 64) return launch<64, false, 0>(tq, tk, tv, p, stream);
+  return launch<32, false, 0>(tq, tk, tv, p, stream);
 }
 
 cudaError_t launch_attn_dense_lone(const CUtensorMap& tq, const CUtensorMap& tk, const CUtensorMap& tv,
                                    const AttnParams& p, cudaStream_t stream) {
-  return launch<128, true>(tq, tk, tv, p, stream);
+  if (p.tile_lse == nullptr) return launch<128, true, 0>(tq, tk, tv, p, stream);
+  if (p.stat_keys == 128) return launch<128, true, 128>(tq, tk, tv, p, stream);
+  if (p.stat_keys == 64) return launch<128, true, 64>(tq, tk, tv, p, stream);
+  return launch<128, true, 32>(tq, tk, tv, p, stream);
 }
 
 }  // namespace sparsed

@@ -5,8 +5,8 @@ namespace sparsed {
 
 // Whether the last wave of `clusters` clusters over `pairs` SM pairs runs as clusters of one stream each. Such a
 // cluster takes 0.65-0.8 of the time of one with two. So a last wave that would leave half of the SM pairs idle or
-// more is launched that way: 2 heads x 4096 tokens 63.5 -> 47.1 us, 8 x 2048 36.9 -> 28.7, 2 x 1024 22.6 -> 18.4,
-// 16 x 3072 (1.3 waves) 95.0 -> 84.4 (statistics recorded). From two full waves on the launch runs into the power
+// more is launched that way: 16 x 3072 (1.3 waves) 95.0 -> 84.4 us (statistics recorded); so is a grid of less than half
+// a wave, of which only the shortest sequences still come here (lone_ctas_pay below). From two full waves on the launch runs into the power
 // limit, which an emptier last wave only relieves (32 x 4096, 3.46 waves: no gain).
 inline bool dense_pair_splits(long long clusters, long long pairs) {
   const long long last = pairs > 0 ? clusters % pairs : 0;
@@ -51,12 +51,12 @@ inline bool dense_pair_pays(long long bh, int seq_len, int max_ctas) {
   return 0.965 * dense_waves(clusters, pairs, split) < dense_waves(bh * tiles, max_ctas, true);
 }
 
-// Whether attention on `items` query tiles, dense or over block lists, with `keys` keys to a row (on average) goes to the
+// Whether attention on `items` query tiles, dense (with or without row statistics) or over block lists, with `keys` keys to a row (on average) goes to the
 // kernel whose CTAs have an SM each (attention_lone.cu), before the choice above is asked. It gives the same bits as the
 // others. Up to one item per SM it was the fastest from five tiles of 64 keys on: dense, against the single-CTA kernel, 2
 // heads x 320 7.70 -> 6.79 us, 2 x 1024 14.9 -> 12.1, 8 x 2304 (144 items) 29.7 -> 23.4, and against split clusters 2 x
 // 4096 44.0 -> 35.8, 2 x 9400 102 -> 77.5; sparse 2 x 8192 block 128 at 4 blocks a row 10.5 -> 9.5, block 64 at 26 34.5 ->
-// 26.1. Its set-up is longer: 2 x 100 5.1 -> 5.9. Beyond one item per SM its items come one after the other, set-up and all:
+// 26.1; switch steps 2 x 1024 18.9 -> 15.8, 8 x 2048 32.8 -> 26.5, 2 x 8192 88.8 -> 78.4. Its set-up is longer: 2 x 100 5.1 -> 5.9. Beyond one item per SM its items come one after the other, set-up and all:
 // 32 x 1900 58 -> 77.
 inline bool lone_ctas_pay(long long items, long long keys, int max_ctas) {
   return items <= max_ctas / 2 && keys >= 256;

@@ -6,6 +6,7 @@ import torch
 
 import paper_2509_24014_b200 as sd
 from tests.parity_util import gpu_full, gpu_sparse
+from tests.test_gpu_switch_step_stats import gpu_switch_step
 
 pytestmark = pytest.mark.gpu
 DEV = "cuda"
@@ -50,3 +51,16 @@ def test_sparse_equals_the_kernels_of_larger_grids(bs, L, rising):
     o = gpu_sparse(q, k, v, pat)
     pat.nnz = 0                                                          # not told how long the lists are: the others
     assert torch.equal(o, gpu_sparse(q, k, v, pat))
+
+
+@pytest.mark.parametrize("rising", [False, True])
+@pytest.mark.parametrize("bs,L", [(32, 256), (32, 288), (32, 1376), (64, 320), (64, 1408), (128, 256), (128, 1408)])
+def test_row_statistics_equal_those_of_larger_grids(bs, L, rising):
+    """Block scores pooled from the statistics that the pass records (128-key ones span a tile of either group)."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    few = sms // ((L + 127) // 128)
+    q, k, v = _inputs(few + 2, few + 2, L, 74, rising)
+    all_heads = gpu_switch_step(q, k, v, bs, 0.3, 0)
+    some = gpu_switch_step(*(t[:, :few].contiguous() for t in (q, k, v)), bs, 0.3, 0)
+    for i in (0, 1, 5):   # O, LSE, scores
+        assert torch.equal(some[i], all_heads[i][:, :few])
