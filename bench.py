@@ -42,30 +42,30 @@ METRIC = "block-sparse attn TFLOP/s, % bf16 peak, speedup vs own dense kernel at
 # sha256 prefix of that file when the capture was taken). A figure whose kernel source has changed
 # since is reported as null with the reason, instead of going stale silently.
 _C2_ATTN = "ncu capture of one launch on the 8k workload (summary under profiles/)"
-_C2_POOL = "ncu --set full capture of one launch on the 8k workload (summary under profiles/)"
-_ATTN_SRC = ("paper_2509_24014_b200/csrc/attention.cu", "paper_2509_24014_b200/csrc/softmax_pipeline.cuh",
-             "paper_2509_24014_b200/csrc/sm100_primitives.cuh")
-_ATTN_SHA = "9958bd4e596d"
+_C2_POOL = "ncu capture of one launch on the 8k workload (summary under profiles/)"
+_ATTN_SRC = ("paper_2509_24014_b200/csrc/attention.cu", "paper_2509_24014_b200/csrc/work_items.cuh",
+             "paper_2509_24014_b200/csrc/softmax_pipeline.cuh", "paper_2509_24014_b200/csrc/sm100_primitives.cuh")
+_ATTN_SHA = "5bc5f2cb7baa"
 _PAIR_SRC = ("paper_2509_24014_b200/csrc/attention_dense_pair.cu", "paper_2509_24014_b200/csrc/sm100_pair_primitives.cuh",
              "paper_2509_24014_b200/csrc/softmax_pipeline.cuh", "paper_2509_24014_b200/csrc/sm100_primitives.cuh",
              "paper_2509_24014_b200/build.py")   # (its compile flags are set per file there)
-_PAIR_SHA = "51201f2226c8"
+_PAIR_SHA = "ca7aa076cc3b"
 _POOL_SRC = ("paper_2509_24014_b200/csrc/pool_select.cu", "paper_2509_24014_b200/csrc/topk_device.cuh")
-_POOL_SHA = "2a48dbebbbc2"
+_POOL_SHA = "11ccb7f1aa7d"
 NCU_DRAM_TRAFFIC = {
-    ("attn_dense_pair_kernel", "c2"): (201488896 + 99233280, _C2_ATTN, _PAIR_SRC, _PAIR_SHA),
-    ("attn_kernel<sparse>", "c2"): (156422400 + 40941824, _C2_ATTN, _ATTN_SRC, _ATTN_SHA),
-    ("pool_select_kernel", "c2"): (68194816 + 587776, _C2_POOL, _POOL_SRC, _POOL_SHA),
+    ("attn_dense_pair_kernel", "c2"): (201667584 + 103738368, _C2_ATTN, _PAIR_SRC, _PAIR_SHA),
+    ("attn_kernel<sparse>", "c2"): (156430592 + 43112448, _C2_ATTN, _ATTN_SRC, _ATTN_SHA),
+    ("pool_select_kernel", "c2"): (68195584 + 175616, _C2_POOL, _POOL_SRC, _POOL_SHA),
     # 64k workload: the 8k capture scaled by the algorithmic bytes of a launch (traffic was the algorithmic
     # traffic at 8k: every K/V re-read hits L2), instead of a multi-counter capture of a 7 GB workload.
     # dense + statistics: Q,K,V,O + LSE + statistics = 6450 MB at 64k against 336 MB at 8k
-    ("attn_dense_pair_kernel", "c4"): (int((201488896 + 99233280) * 6450.0 / 336.0), _C2_ATTN + ", scaled x19.2 by algorithmic bytes",
+    ("attn_dense_pair_kernel", "c4"): (int((201667584 + 103738368) * 6450.0 / 336.0), _C2_ATTN + ", scaled x19.2 by algorithmic bytes",
                                        _PAIR_SRC, _PAIR_SHA),
     # sparse: Q + O + touched K,V: 8x the rows and 8x the K/V of the 8k workload
-    ("attn_kernel<sparse>", "c4"): ((156422400 + 40941824) * 8, _C2_ATTN + ", scaled x8 by algorithmic bytes",
+    ("attn_kernel<sparse>", "c4"): ((156430592 + 43112448) * 8, _C2_ATTN + ", scaled x8 by algorithmic bytes",
                                     _ATTN_SRC, _ATTN_SHA),
     # pooling: the statistics stream, 64x the 8k one (rows x8, key blocks x8)
-    ("pool_select_kernel", "c4"): ((68194816 + 587776) * 64, _C2_POOL + ", scaled x64 by algorithmic bytes",
+    ("pool_select_kernel", "c4"): ((68195584 + 175616) * 64, _C2_POOL + ", scaled x64 by algorithmic bytes",
                                    _POOL_SRC, _POOL_SHA),
 }
 
