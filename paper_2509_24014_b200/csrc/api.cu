@@ -573,11 +573,8 @@ sparsed_status sparsed_attn_sparse(const sparsed_shape* shape, const sparsed_pat
   p.col_capacity = pattern->col_capacity;
   p.status = static_cast<DeviceStatus*>(ws);
   const cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
-  // (the lists' average length; 0 if the caller's pattern does not say how many entries it has)
-  const long long rows = static_cast<long long>(shape->batch) * shape->heads_q * pattern->num_blocks;
-  const long long keys = pattern->nnz > 0 ? pattern->nnz / rows * bs : 0;
-  cudaError_t e = lone_ctas_pay(p.num_items, keys, p.max_ctas) ? launch_attn_sparse_lone(tq, tk, tv, p, bs, stream)
-                                                               : launch_attn_sparse(tq, tk, tv, to, p, bs, stream);
+  cudaError_t e = sparse_lone_ctas_pay(p.num_items, p.max_ctas) ? launch_attn_sparse_lone(tq, tk, tv, p, bs, stream)
+                                                                : launch_attn_sparse(tq, tk, tv, to, p, bs, stream);
   return e == cudaSuccess ? SPARSED_OK : cuda_fail(e);
 }
 

@@ -51,15 +51,21 @@ inline bool dense_pair_pays(long long bh, int seq_len, int max_ctas) {
   return 0.965 * dense_waves(clusters, pairs, split) < dense_waves(bh * tiles, max_ctas, true);
 }
 
-// Whether attention on `items` query tiles, dense (with or without row statistics) or over block lists, with `keys` keys to a row (on average) goes to the
-// kernel whose CTAs have an SM each (attention_lone.cu), before the choice above is asked. It gives the same bits as the
-// others. Up to one item per SM it was the fastest from five tiles of 64 keys on: dense, against the single-CTA kernel, 2
-// heads x 320 7.70 -> 6.79 us, 2 x 1024 14.9 -> 12.1, 8 x 2304 (144 items) 29.7 -> 23.4, and against split clusters 2 x
-// 4096 44.0 -> 35.8, 2 x 9400 102 -> 77.5; sparse 2 x 8192 block 128 at 4 blocks a row 10.5 -> 9.5, block 64 at 26 34.5 ->
-// 26.1; switch steps 2 x 1024 18.9 -> 15.8, 8 x 2048 32.8 -> 26.5, 2 x 8192 88.8 -> 78.4. Its set-up is longer: 2 x 100 5.1 -> 5.9. Beyond one item per SM its items come one after the other, set-up and all:
-// 32 x 1900 58 -> 77.
+// Whether attention on `items` query tiles over `keys` keys to a row goes to the kernel whose CTAs have an SM each
+// (attention_lone.cu), before the choice above is asked. It gives the same bits as the others. Up to one item per SM it
+// was the fastest (us, 20 calls in a row): dense from four tiles of 64 keys on, against the single-CTA kernel 2 heads x
+// 256 6.95 -> 6.36, 2 x 320 7.61 -> 6.68, 2 x 1024 14.8 -> 11.9, 8 x 2304 (144 items) 29.1 -> 23.4, and against split
+// clusters 2 x 4096 44.0 -> 35.8, 2 x 9400 102 -> 77.5; switch steps 2 x 256 12.1 -> 10.7, 2 x 1024 18.9 -> 15.8, 8 x 2304
+// 43.1 -> 28.5, 2 x 8192 88.8 -> 78.4. With fewer keys its longer set-up shows: 2 x 100 5.1 -> 5.9. Beyond one item per SM
+// its items come one after the other, set-up and all: 32 x 1900 58 -> 77.
 inline bool lone_ctas_pay(long long items, long long keys, int max_ctas) {
   return items <= max_ctas / 2 && keys >= 256;
 }
+
+// The same for block-sparse attention, where the lists may be of any length: 2 heads x 1024 block 128, one block a row
+// 5.85 -> 5.56, six 12.3 -> 10.5; 16 x 512 block 32 (walked as the union of four rows' lists) one 7.72 -> 7.15, ten 11.9
+// -> 10.4; 2 x 4096 block 32, twelve 21.8 -> 16.3; no blocks at all, 8 x 1024 block 32, 4.2 -> 3.7; one whole row among
+// rows of one block, 2 x 8192 block 64, 91 -> 71.
+inline bool sparse_lone_ctas_pay(long long items, int max_ctas) { return items <= max_ctas / 2; }
 
 }  // namespace sparsed

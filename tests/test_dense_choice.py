@@ -20,29 +20,44 @@ TABLE = [
 ]
 
 
+# Block-sparse attention, query tiles and whether the kernel whose CTAs have an SM each runs: up to one tile per SM, and
+# however short the lists are.
+SPARSE_TABLE = [(1, 1), (16, 1), (64, 1), (148, 1), (149, 0), (4096, 0)]
+
+
 @pytest.fixture(scope="module")
-def pays(tmp_path_factory):
+def choice(tmp_path_factory):
     folder = tmp_path_factory.mktemp("dense_choice")
     src, exe = folder / "choice.cpp", folder / "choice"
-    src.write_text('#include <cstdio>\n#include <cstdlib>\n#include "dense_choice.h"\n'
+    src.write_text('#include <cstdio>\n#include <cstdlib>\n#include <cstring>\n#include "dense_choice.h"\n'
+                   "using namespace sparsed;\n"
                    "int main(int argc, char** argv) {\n"
-                   "  for (int i = 1; i + 2 < argc; i += 3)\n"
-                   "    std::printf(\"%d\\n\", sparsed::dense_pair_pays(std::atoll(argv[i]), std::atoi(argv[i + 1]),\n"
-                   "                                                   std::atoi(argv[i + 2])));\n}\n")
+                   "  for (int i = 2; i + 2 < argc; i += 3) {\n"
+                   "    const long long a = std::atoll(argv[i]), b = std::atoll(argv[i + 1]);\n"
+                   "    const int ctas = std::atoi(argv[i + 2]);\n"
+                   '    if (std::strcmp(argv[1], "pair") == 0) std::printf("%d\\n", dense_pair_pays(a, static_cast<int>(b), ctas));\n'
+                   '    if (std::strcmp(argv[1], "lone") == 0) std::printf("%d\\n", lone_ctas_pay(a, b, ctas));\n'
+                   '    if (std::strcmp(argv[1], "sparse") == 0) std::printf("%d\\n", sparse_lone_ctas_pay(a, ctas));\n'
+                   "  }\n}\n")
     subprocess.run([os.environ.get("CXX", "g++"), "-std=c++17", "-I", build.CSRC, str(src), "-o", str(exe)], check=True,
                    capture_output=True, timeout=120)
 
-    def ask(rows):
-        args = [str(x) for row in rows for x in row]
+    def ask(rule, rows):
+        args = [rule] + [str(x) for row in rows for x in row]
         return [int(x) for x in subprocess.run([str(exe), *args], check=True, capture_output=True, text=True).stdout.split()]
 
     return ask
 
 
-def test_choice(pays):
-    got = pays([(bh, tokens, 296) for bh, tokens, _ in TABLE])
+def test_choice(choice):
+    got = choice("pair", [(bh, tokens, 296) for bh, tokens, _ in TABLE])
     assert got == [want for _, _, want in TABLE]
 
 
-def test_no_pairs_without_a_known_device(pays):
-    assert pays([(bh, tokens, ctas) for bh, tokens, _ in TABLE for ctas in (0, 2)]) == [0] * (2 * len(TABLE))
+def test_sparse_choice(choice):
+    assert choice("sparse", [(items, 0, 296) for items, _ in SPARSE_TABLE]) == [want for _, want in SPARSE_TABLE]
+    assert choice("sparse", [(items, 0, 0) for items, _ in SPARSE_TABLE]) == [0] * len(SPARSE_TABLE)
+
+
+def test_no_pairs_without_a_known_device(choice):
+    assert choice("pair", [(bh, tokens, ctas) for bh, tokens, _ in TABLE for ctas in (0, 2)]) == [0] * (2 * len(TABLE))

@@ -33,9 +33,11 @@ def test_dense_equals_the_kernels_of_larger_grids(L, rising):
 
 
 @pytest.mark.parametrize("rising", [False, True])
+@pytest.mark.parametrize("most", ["one", "four", "all"])   # blocks of a list at most
 @pytest.mark.parametrize("bs,L", [(128, 1280), (64, 1344), (32, 1376), (32, 608), (128, 8192)])
-def test_sparse_equals_the_kernels_of_larger_grids(bs, L, rising):
-    """Lists of every length, empty ones among them (128-key blocks, 8192 tokens: more than the 32 ids fetched at once)."""
+def test_sparse_equals_the_kernels_of_larger_grids(bs, L, most, rising):
+    """Lists of every length, empty ones among them (128-key blocks, 8192 tokens: more than the 32 ids fetched at once),
+    and lists of a few blocks only. Copies of the same heads make up the larger grid."""
     H, Hkv, nb = (2, 1, L // bs)
     q, k, v = _inputs(H, Hkv, L, 72, rising)
     g = torch.Generator(device=DEV).manual_seed(73)
@@ -43,14 +45,20 @@ def test_sparse_equals_the_kernels_of_larger_grids(bs, L, rising):
     keep &= torch.rand(H, nb, 1, generator=g, device=DEV) < 0.9
     keep[:, 1] = False
     keep[:, 2] = True
-    row_ptr = torch.zeros(H * nb + 1, dtype=torch.int32, device=DEV)
-    row_ptr[1:] = keep.sum(-1).flatten().cumsum(0)
-    col_idx = keep.flatten(0, 1).nonzero()[:, 1].to(torch.int32).contiguous()
-    pat = sd.pattern_from_csr(row_ptr, col_idx, bs, nb, 1, H)
-    assert pat.nnz == col_idx.numel() and pat.nnz * bs >= 256 * H * nb   # long enough for the kernel under test
-    o = gpu_sparse(q, k, v, pat)
-    pat.nnz = 0                                                          # not told how long the lists are: the others
-    assert torch.equal(o, gpu_sparse(q, k, v, pat))
+    if most != "all":
+        keep &= keep.cumsum(-1) <= {"one": 1, "four": 4}[most]
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    copies = sms // (H * ((L + 127) // 128)) + 1
+
+    def attend(n):   # n copies of the heads
+        row_ptr = torch.zeros(n * H * nb + 1, dtype=torch.int32, device=DEV)
+        row_ptr[1:] = keep.repeat(n, 1, 1).sum(-1).flatten().cumsum(0)
+        col_idx = keep.repeat(n, 1, 1).flatten(0, 1).nonzero()[:, 1].to(torch.int32).contiguous()
+        return gpu_sparse(q.repeat(1, n, 1, 1), k.repeat(1, n, 1, 1), v.repeat(1, n, 1, 1),
+                          sd.pattern_from_csr(row_ptr, col_idx, bs, nb, 1, n * H))
+
+    o, o_many = attend(1), attend(copies)                                        # more query tiles than SMs
+    assert torch.equal(o_many, o.repeat(1, copies, 1, 1))
 
 
 @pytest.mark.parametrize("rising", [False, True])
