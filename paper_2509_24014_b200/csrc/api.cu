@@ -367,7 +367,8 @@ static DenseKernel dense_kernel(bool with_stats, const sparsed_shape* shape, int
   }();
   if (!with_stats && forced >= 0) return static_cast<DenseKernel>(forced);
   const long long bh = static_cast<long long>(shape->batch) * shape->heads_q;
-  if (lone_ctas_pay(bh * ((static_cast<long long>(shape->seq_len) + 127) / 128), shape->seq_len, max_ctas)) return kLone;
+  const long long items = bh * ((static_cast<long long>(shape->seq_len) + 127) / 128);
+  if (lone_ctas_pay(with_stats, items, shape->seq_len, max_ctas)) return kLone;
   if (with_stats) return kPair;
   return dense_pair_pays(bh, shape->seq_len, max_ctas) ? kPair : kSingle;
 }
@@ -573,8 +574,10 @@ sparsed_status sparsed_attn_sparse(const sparsed_shape* shape, const sparsed_pat
   p.col_capacity = pattern->col_capacity;
   p.status = static_cast<DeviceStatus*>(ws);
   const cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
-  cudaError_t e = sparse_lone_ctas_pay(p.num_items, p.max_ctas) ? launch_attn_sparse_lone(tq, tk, tv, p, bs, stream)
-                                                                : launch_attn_sparse(tq, tk, tv, to, p, bs, stream);
+  const long long rows = static_cast<long long>(shape->batch) * shape->heads_q * pattern->num_blocks;
+  const bool lone = sparse_lone_ctas_pay(p.num_items, pattern->nnz, rows, pattern->num_blocks, bs, p.max_ctas);
+  cudaError_t e = lone ? launch_attn_sparse_lone(tq, tk, tv, p, bs, stream)
+                       : launch_attn_sparse(tq, tk, tv, to, p, bs, stream);
   return e == cudaSuccess ? SPARSED_OK : cuda_fail(e);
 }
 

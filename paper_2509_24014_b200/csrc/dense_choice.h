@@ -58,14 +58,37 @@ inline bool dense_pair_pays(long long bh, int seq_len, int max_ctas) {
 // clusters 2 x 4096 44.0 -> 35.8, 2 x 9400 102 -> 77.5; switch steps 2 x 256 12.1 -> 10.7, 2 x 1024 18.9 -> 15.8, 8 x 2304
 // 43.1 -> 28.5, 2 x 8192 88.8 -> 78.4. With fewer keys its longer set-up shows: 2 x 100 5.1 -> 5.9. Beyond one item per SM
 // its items come one after the other, set-up and all: 32 x 1900 58 -> 77.
-inline bool lone_ctas_pay(long long items, long long keys, int max_ctas) {
-  return items <= max_ctas / 2 && keys >= 256;
+//
+// That is for a call alone. Calls side by side on several streams lose by it once all their items together are more than
+// the SMs, where two CTAs of the other kernels share one. A plain call's rule cannot see its neighbours; the line lies
+// where a pair of equal calls loses about as much as a call alone gains. Dense, alone | a pair (time over that of the
+// single-CTA kernel): 100 items x 256 keys 0.96 | 1.05, x 768 0.87 | 0.97; 128 x 512 0.90 | 1.14, 148 x 256 0.95 | 1.36,
+// x 512 0.87 | 1.30; 128 x 1024 0.84 | 1.09, 144 x 1024 0.82 | 1.17, x 2048 0.75 | 1.11, 128 x 4096 0.87 | 1.01. So beyond
+// two thirds of the SMs it takes 1024 keys. (Three calls of 64 items: x 1024 keys 0.87; four: 1.10.) Switch steps gain
+// either way, their other kernel takes two SMs to a cluster: 144 x 1024 0.85 | 0.82.
+inline bool lone_ctas_pay(bool with_stats, long long items, long long keys, int max_ctas) {
+  const long long sms = max_ctas / 2;
+  return items <= sms && keys >= (with_stats || 3 * items <= 2 * sms ? 256 : 1024);
 }
 
-// The same for block-sparse attention, where the lists may be of any length: 2 heads x 1024 block 128, one block a row
+// The same for block-sparse attention. Alone, the lists may be of any length: 2 heads x 1024 block 128, one block a row
 // 5.85 -> 5.56, six 12.3 -> 10.5; 16 x 512 block 32 (walked as the union of four rows' lists) one 7.72 -> 7.15, ten 11.9
 // -> 10.4; 2 x 4096 block 32, twelve 21.8 -> 16.3; no blocks at all, 8 x 1024 block 32, 4.2 -> 3.7; one whole row among
-// rows of one block, 2 x 8192 block 64, 91 -> 71.
-inline bool sparse_lone_ctas_pay(long long items, int max_ctas) { return items <= max_ctas / 2; }
+// rows of one block, 2 x 8192 block 64, 91 -> 71. Side by side (alone | a pair): block 128, 72 items x 128 keys 0.98 | 0.98,
+// 80 x 256 0.95 | 1.09, x 512 0.93 | 1.05, 128 x 1024 0.86 | 1.18, x 2048 0.82 | 1.13, 148 x 2048 0.81 | 1.25, x 3072 0.79 |
+// 1.17; block 64 and 32, whose unions are longer than the lists, 100 x 128 0.90 | 1.10, 128 x 256 0.88 | 1.18 and 0.84 |
+// 1.09, 144 x 512 0.82 | 1.14 and 0.83 | 1.12. keys: on average in the `rows` lists, as far as `nnz` (all entries) says;
+// 0 if it does not.
+inline bool sparse_lone_ctas_pay(long long items, long long nnz, long long rows, int num_blocks, int block_size,
+                                 int max_ctas) {
+  const long long sms = max_ctas / 2;
+  if (items > sms || rows < 1) return false;
+  if (nnz < 0) nnz = 0;
+  if (nnz > rows * num_blocks) nnz = rows * num_blocks;   // (room rather than entries)
+  const long long keys = nnz * block_size / rows;
+  const bool packed = block_size < 128;
+  if (2 * items <= sms) return true;
+  return keys >= (3 * items <= 2 * sms ? (packed ? 0 : 512) : (packed ? 512 : 2048));
+}
 
 }  // namespace sparsed

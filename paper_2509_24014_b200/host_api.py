@@ -41,8 +41,9 @@ class HostSparseAttention:
         for kv0 in range(0, Hkv, kv_heads_per_chunk):
             kv1 = min(Hkv, kv0 + kv_heads_per_chunk)
             h0, h1 = kv0 * self.group, kv1 * self.group
+            # (nnz: the chunk's share of the layer's entries, by which the call chooses its kernel)
             pat = sd.Pattern(row_ptr.data_ptr() + 4 * h0 * self.nb, col_idx.data_ptr(), col_idx.numel(),
-                             int(col_idx.numel()), block_size, self.nb, 1, h1 - h0)
+                             col_idx.numel() * (h1 - h0) // Hq, block_size, self.nb, 1, h1 - h0)
             self.chunks.append((kv0, kv1, h0, h1, pat))
 
     def run(self, q_host, k_host, v_host, o_host) -> None:

@@ -20,9 +20,21 @@ TABLE = [
 ]
 
 
-# Block-sparse attention, query tiles and whether the kernel whose CTAs have an SM each runs: up to one tile per SM, and
-# however short the lists are.
-SPARSE_TABLE = [(1, 1), (16, 1), (64, 1), (148, 1), (149, 0), (4096, 0)]
+# The kernel whose CTAs have an SM each, which is asked for first: whether row statistics are recorded, query tiles, keys.
+LONE_TABLE = [
+    (0, 1, 255, 0), (0, 1, 256, 1), (0, 16, 1024, 1), (0, 98, 256, 1),     # up to two thirds of the SMs
+    (0, 99, 256, 0), (0, 148, 1023, 0), (0, 99, 1024, 1), (0, 148, 1024, 1), (0, 128, 8192, 1),
+    (0, 149, 256, 0), (0, 149, 8192, 0), (0, 480, 1900, 0),                # more tiles than SMs
+    (1, 148, 255, 0), (1, 99, 256, 1), (1, 148, 256, 1), (1, 149, 8192, 0),
+]
+# The same for block-sparse attention: query tiles, average list in blocks (None: not known), block size.
+SPARSE_TABLE = [
+    (1, None, 128, 1), (74, None, 128, 1), (74, 0.1, 32, 1), (74, 1, 64, 1),   # up to half of the SMs: any lists
+    (75, None, 128, 0), (75, 3.9, 128, 0), (75, 4, 128, 1), (98, 4, 128, 1), (98, None, 64, 1), (98, 0.1, 32, 1),
+    (99, 4, 128, 0), (99, 15.9, 128, 0), (99, 16, 128, 1), (148, 16, 128, 1),  # beyond two thirds
+    (99, None, 64, 0), (148, 7.9, 64, 0), (148, 8, 64, 1), (148, 15.9, 32, 0), (148, 16, 32, 1),
+    (149, 64, 128, 0), (149, 64, 32, 0), (149, None, 64, 0),
+]
 
 
 @pytest.fixture(scope="module")
@@ -32,13 +44,14 @@ def choice(tmp_path_factory):
     src.write_text('#include <cstdio>\n#include <cstdlib>\n#include <cstring>\n#include "dense_choice.h"\n'
                    "using namespace sparsed;\n"
                    "int main(int argc, char** argv) {\n"
-                   "  for (int i = 2; i + 2 < argc; i += 3) {\n"
-                   "    const long long a = std::atoll(argv[i]), b = std::atoll(argv[i + 1]);\n"
-                   "    const int ctas = std::atoi(argv[i + 2]);\n"
-                   '    if (std::strcmp(argv[1], "pair") == 0) std::printf("%d\\n", dense_pair_pays(a, static_cast<int>(b), ctas));\n'
-                   '    if (std::strcmp(argv[1], "lone") == 0) std::printf("%d\\n", lone_ctas_pay(a, b, ctas));\n'
-                   '    if (std::strcmp(argv[1], "sparse") == 0) std::printf("%d\\n", sparse_lone_ctas_pay(a, ctas));\n'
-                   "  }\n}\n")
+                   "  auto arg = [&](int i) { return std::atoll(argv[i]); };\n"
+                   "  auto is = [&](const char* rule) { return std::strcmp(argv[1], rule) == 0; };\n"
+                   "  const int n = is(\"pair\") ? 3 : is(\"lone\") ? 4 : 6;\n"
+                   "  for (int i = 2; i + n <= argc; i += n)\n"
+                   '    std::printf("%d\\n", is("pair")   ? dense_pair_pays(arg(i), arg(i + 1), arg(i + 2))\n'
+                   '                        : is("lone") ? lone_ctas_pay(arg(i), arg(i + 1), arg(i + 2), arg(i + 3))\n'
+                   "                                     : sparse_lone_ctas_pay(arg(i), arg(i + 1), arg(i + 2), arg(i + 3),\n"
+                   "                                                            arg(i + 4), arg(i + 5)));\n}\n")
     subprocess.run([os.environ.get("CXX", "g++"), "-std=c++17", "-I", build.CSRC, str(src), "-o", str(exe)], check=True,
                    capture_output=True, timeout=120)
 
@@ -54,9 +67,22 @@ def test_choice(choice):
     assert got == [want for _, _, want in TABLE]
 
 
+def test_lone_choice(choice):
+    assert choice("lone", [(*row[:3], 296) for row in LONE_TABLE]) == [row[3] for row in LONE_TABLE]
+    assert choice("lone", [(*row[:3], 0) for row in LONE_TABLE]) == [0] * len(LONE_TABLE)
+
+
 def test_sparse_choice(choice):
-    assert choice("sparse", [(items, 0, 296) for items, _ in SPARSE_TABLE]) == [want for _, want in SPARSE_TABLE]
-    assert choice("sparse", [(items, 0, 0) for items, _ in SPARSE_TABLE]) == [0] * len(SPARSE_TABLE)
+    def ask(ctas):
+        rows = [(items, items * 128 // bs) for items, _, bs, _ in SPARSE_TABLE]   # one head: a list per query block
+        return choice("sparse", [(items, 0 if blocks is None else int(n * blocks + 0.5), n, n, bs, ctas)
+                                 for (items, n), (_, blocks, bs, _) in zip(rows, SPARSE_TABLE)])
+
+    assert ask(296) == [row[3] for row in SPARSE_TABLE]
+    assert ask(0) == [0] * len(SPARSE_TABLE)
+    # counts that cannot be: more entries than the rows have blocks (a buffer's room), a field nobody set
+    assert choice("sparse", [(148, 1 << 40, 148, 148, 128, 296), (148, 1 << 62, 148, 15, 128, 296),
+                             (148, -1, 148, 148, 128, 296), (148, -(1 << 63), 592, 592, 32, 296)]) == [1, 0, 0, 0]
 
 
 def test_no_pairs_without_a_known_device(choice):

@@ -20,6 +20,7 @@ def test_host_sparse_attention_matches_resident(Hq, Hkv, chunk):
     hq, hk, hv = (t.cpu().pin_memory() for t in (q, k, v))
     ho = torch.zeros(q.shape, dtype=torch.bfloat16).pin_memory()
     plan = HostSparseAttention(hq, hk, row_ptr, col_idx, 128, DEV, kv_heads_per_chunk=chunk, n_streams=2)
+    assert sum(pat_c.nnz for *_, pat_c in plan.chunks) == col_idx.numel()   # each chunk's own entries (lists are equally long)
     for _ in range(2):
         plan.run(hq, hk, hv, ho)
         torch.cuda.synchronize()

@@ -25,8 +25,9 @@ def _inputs(H, Hkv, L, seed, rising):
 @pytest.mark.parametrize("L", [256, 257, 300, 384, 449, 640, 700, 1473])   # 4 to 24 tiles, ragged by 1 to 63 keys
 def test_dense_equals_the_kernels_of_larger_grids(L, rising):
     sms = torch.cuda.get_device_properties(0).multi_processor_count
-    few = sms // ((L + 127) // 128)
-    q, k, v = _inputs(few + 2, few + 2, L, 71, rising)
+    tiles = (L + 127) // 128
+    few, many = 2 * sms // 3 // tiles, sms // tiles + 1
+    q, k, v = _inputs(many, many, L, 71, rising)
     o_all, lse_all = gpu_full(q, k, v)                                           # more query tiles than SMs
     o, lse = gpu_full(*(t[:, :few].contiguous() for t in (q, k, v)))
     assert torch.equal(o, o_all[:, :few]) and torch.equal(lse, lse_all[:, :few])
@@ -34,10 +35,10 @@ def test_dense_equals_the_kernels_of_larger_grids(L, rising):
 
 @pytest.mark.parametrize("rising", [False, True])
 @pytest.mark.parametrize("most", ["one", "four", "all"])   # blocks of a list at most
-@pytest.mark.parametrize("bs,L", [(128, 1280), (64, 1344), (32, 1376), (32, 608), (128, 8192)])
+@pytest.mark.parametrize("bs,L", [(128, 1280), (64, 1344), (32, 1376), (32, 608), (128, 4736), (128, 8192)])
 def test_sparse_equals_the_kernels_of_larger_grids(bs, L, most, rising):
-    """Lists of every length, empty ones among them (128-key blocks, 8192 tokens: more than the 32 ids fetched at once),
-    and lists of a few blocks only. Copies of the same heads make up the larger grid."""
+    """Lists of every length, empty ones among them (128-key blocks, 4736 and 8192 tokens: more than the 32 ids fetched at
+    once), and lists of a few blocks only. Copies of the same heads make up the larger grid."""
     H, Hkv, nb = (2, 1, L // bs)
     q, k, v = _inputs(H, Hkv, L, 72, rising)
     g = torch.Generator(device=DEV).manual_seed(73)
