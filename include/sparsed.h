@@ -87,7 +87,8 @@ typedef struct sparsed_pattern {
   int32_t *row_ptr;     /* device, batch*heads_q*num_blocks + 1 entries */
   int32_t *col_idx;     /* device, col_capacity entries */
   int64_t col_capacity; /* entries available in col_idx */
-  int64_t nnz;          /* set by the selection calls: entries used */
+  int64_t nnz;          /* set by the selection calls: entries used. sparsed_attn_sparse only chooses between
+                           kernels that give the same bits by it (0: not known) */
   int32_t block_size, num_blocks, batch, heads_q; /* set by the selection calls */
 } sparsed_pattern;
 
@@ -148,12 +149,13 @@ sparsed_status sparsed_select_from_scores(const sparsed_select_params *params, c
  *                               recorded with.
  * Same rules and errors as sparsed_attn_full / sparsed_select_pattern; the selection needs
  * seq_len / block_size <= 2048 (UNSUPPORTED beyond). Both buffers are caller-owned device memory.
- * sparsed_attn_full_stats runs on a kernel whose MMAs span pairs of CTAs (launched as clusters of two);
- * sparsed_attn_full runs on it where that is the faster one (from 4096 tokens on, by the number of heads
- * and tokens) and on a single-CTA kernel elsewhere. Both give the same bits (but an LSE within
- * 1.2e-38 of zero is zero from the CTA-pair kernel). The environment variable
- * SPARSED_DENSE_KERNEL=pair|single, read at the first call, sends sparsed_attn_full to one of them at
- * every length, for measurements.
+ * Three dense kernels do the work: one whose thread blocks have an SM each (up to one 128-row query tile
+ * per SM, from 256 keys on, longer where the tiles are many), one whose MMAs span pairs of CTAs (other
+ * passes that record statistics; plain ones from 4096 tokens on, by the number of heads and tokens), and
+ * a single-CTA kernel (the other plain passes). All give the same bits (but an LSE within 1.2e-38 of zero
+ * is zero from the CTA-pair kernel). The environment variable SPARSED_DENSE_KERNEL=lone|pair|single, read
+ * at the first call, sends every dense pass to one of them, for measurements and tests (a pass that
+ * records statistics is never sent to the single-CTA kernel).
  */
 sparsed_status sparsed_tile_stats_bytes(const sparsed_shape *shape, int32_t block_size,
                                         size_t *out_bytes); /* host only */

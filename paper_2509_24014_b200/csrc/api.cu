@@ -354,23 +354,20 @@ sparsed_status sparsed_workspace_init(void* ws, size_t ws_bytes, void* cuda_stre
   return e == cudaSuccess ? SPARSED_OK : cuda_fail(e);
 }
 
-// Which dense kernel runs. The single-CTA one records no row statistics. The environment variable SPARSED_DENSE_KERNEL
-// (read once) sends every plain pass to one of them, `pair`, `single` or `lone`, for A/B measurements and tests.
-enum DenseKernel { kSingle, kPair, kLone };
+// Which dense kernel runs. The environment variable SPARSED_DENSE_KERNEL (read once) sends every pass to one of them,
+// `pair`, `single` or `lone`, for A/B measurements and tests; a pass that records row statistics, which the single-CTA
+// kernel cannot do, is not sent there.
 static DenseKernel dense_kernel(bool with_stats, const sparsed_shape* shape, int max_ctas) {
   static const int forced = [] {
     const char* v = std::getenv("SPARSED_DENSE_KERNEL");
-    if (v != nullptr && std::strcmp(v, "pair") == 0) return static_cast<int>(kPair);
-    if (v != nullptr && std::strcmp(v, "single") == 0) return static_cast<int>(kSingle);
-    if (v != nullptr && std::strcmp(v, "lone") == 0) return static_cast<int>(kLone);
+    if (v != nullptr && std::strcmp(v, "pair") == 0) return static_cast<int>(DenseKernel::kPair);
+    if (v != nullptr && std::strcmp(v, "single") == 0) return static_cast<int>(DenseKernel::kSingle);
+    if (v != nullptr && std::strcmp(v, "lone") == 0) return static_cast<int>(DenseKernel::kLone);
     return -1;
   }();
-  if (!with_stats && forced >= 0) return static_cast<DenseKernel>(forced);
-  const long long bh = static_cast<long long>(shape->batch) * shape->heads_q;
-  const long long items = bh * ((static_cast<long long>(shape->seq_len) + 127) / 128);
-  if (lone_ctas_pay(with_stats, items, shape->seq_len, max_ctas)) return kLone;
-  if (with_stats) return kPair;
-  return dense_pair_pays(bh, shape->seq_len, max_ctas) ? kPair : kSingle;
+  if (forced >= 0 && !(with_stats && forced == static_cast<int>(DenseKernel::kSingle)))
+    return static_cast<DenseKernel>(forced);
+  return choose_dense_kernel(with_stats, static_cast<long long>(shape->batch) * shape->heads_q, shape->seq_len, max_ctas);
 }
 
 static sparsed_status attn_full_impl(const sparsed_shape* shape, const void* q, const void* k, const void* v, void* o,
@@ -389,7 +386,8 @@ static sparsed_status attn_full_impl(const sparsed_shape* shape, const void* q, 
   CUtensorMap tq, tk, tv, to;
   if ((st = make_tensor_map(&tq, q, shape->batch, shape->heads_q, shape->seq_len, rs.q, 128)) != SPARSED_OK) return st;
   if ((st = make_tensor_map(&to, o, shape->batch, shape->heads_q, shape->seq_len, rs.o, 128)) != SPARSED_OK) return st;
-  if ((st = make_tensor_map(&tk, k, shape->batch, shape->heads_kv, shape->seq_len, rs.k, kernel == kPair ? 32 : 64)) != SPARSED_OK) return st;
+  const int k_box = kernel == DenseKernel::kPair ? 32 : 64;
+  if ((st = make_tensor_map(&tk, k, shape->batch, shape->heads_kv, shape->seq_len, rs.k, k_box)) != SPARSED_OK) return st;
   if ((st = make_tensor_map(&tv, v, shape->batch, shape->heads_kv, shape->seq_len, rs.v, 64)) != SPARSED_OK) return st;
   AttnParams p;
   p.o = o;
@@ -413,9 +411,9 @@ static sparsed_status attn_full_impl(const sparsed_shape* shape, const void* q, 
   p.col_capacity = 0;
   p.status = static_cast<DeviceStatus*>(ws);
   const cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
-  cudaError_t e = kernel == kPair   ? launch_attn_dense_pair(tq, tk, tv, to, p, stream)
-                  : kernel == kLone ? launch_attn_dense_lone(tq, tk, tv, p, stream)
-                                    : launch_attn_dense(tq, tk, tv, to, p, stream);
+  cudaError_t e = kernel == DenseKernel::kPair   ? launch_attn_dense_pair(tq, tk, tv, to, p, stream)
+                  : kernel == DenseKernel::kLone ? launch_attn_dense_lone(tq, tk, tv, p, stream)
+                                                 : launch_attn_dense(tq, tk, tv, to, p, stream);
   return e == cudaSuccess ? SPARSED_OK : cuda_fail(e);
 }
 

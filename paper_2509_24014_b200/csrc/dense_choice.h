@@ -1,13 +1,14 @@
-// The rule by which plain dense attention goes to one of its two kernels. Host arithmetic only.
+// The rules by which an attention call goes to one of the kernels that can do it. Host arithmetic only.
 #pragma once
 
 namespace sparsed {
 
 // Whether the last wave of `clusters` clusters over `pairs` SM pairs runs as clusters of one stream each. Such a
 // cluster takes 0.65-0.8 of the time of one with two. So a last wave that would leave half of the SM pairs idle or
-// more is launched that way: 16 x 3072 (1.3 waves) 95.0 -> 84.4 us (statistics recorded); so is a grid of less than half
-// a wave, of which only the shortest sequences still come here (lone_ctas_pay below). From two full waves on the launch runs into the power
-// limit, which an emptier last wave only relieves (32 x 4096, 3.46 waves: no gain).
+// more is launched that way: 16 x 3072 (1.3 waves) 95.0 -> 84.4 us (statistics recorded). So is a grid of less than half
+// a wave, but only those of fewer than 256 keys come here (choose_dense_kernel). From two full waves on the launch runs
+// into the power limit, which an emptier last wave only relieves: 32 x 4096 (3.46 waves) at 1755 MHz where 37 x 4096 (4.0)
+// is at 1687, no gain.
 inline bool dense_pair_splits(long long clusters, long long pairs) {
   const long long last = pairs > 0 ? clusters % pairs : 0;
   return last != 0 && 2 * last <= pairs && clusters < 2 * pairs;
@@ -25,7 +26,7 @@ inline double dense_waves(long long units, long long slots, bool half_wave) {
 }
 
 // Whether the kernel whose MMAs span CTA pairs (attention_dense_pair.cu) takes a plain pass over bh heads of all batch
-// entries; the single-CTA kernel (attention.cu) takes the others. Both give the same bits. max_ctas: CTAs of the latter
+// entries that lone_ctas_pay has not taken; the single-CTA kernel (attention.cu) takes the others. Both give the same bits. max_ctas: CTAs of the latter
 // that fit on the device at once, two per SM.
 //
 // Per query row the pair kernel takes 3-7 % less under sustained load, which is bound by power (it fetches each K/V
@@ -33,9 +34,9 @@ inline double dense_waves(long long units, long long slots, bool half_wave) {
 // 16384 3720 -> 3495. Launches too short to reach the power limit, or with rests between them, gain nothing from
 // that, and the longer set-up and tear-down of a cluster costs them 2-8 % (20 launches after a rest: 8 heads x 4096
 // 60.0 against 64.3 us, 20 heads 172 against 179). So the pair kernel runs where it was no slower either way:
-//   * where the last wave, or the only one, runs as clusters of one stream each: its SMs would be half empty in both
-//     kernels (6 x 8192 217 -> 198 us, 3 x 16384 417 -> 374; an only wave that is split is up to one query tile per SM, and
-//     goes to a third kernel first, see below);
+//   * where the last wave runs as clusters of one stream each: its SMs would be half empty in both kernels (6 x 8192 217 ->
+//     198 us, 3 x 16384 417 -> 374; where that is the only wave there is at most one query tile per SM, and lone_ctas_pay
+//     has taken the call);
 //   * from 2^29 logits on (32 heads x 4096, 8 x 8192), which take 200 us. With fewer, 12 heads x 6144 lose 1 % after
 //     a rest, and 5 heads x 4096 9 % even under sustained load: 40 clusters leave 68 SMs empty, 160 CTAs
 //     none.
@@ -71,7 +72,16 @@ inline bool lone_ctas_pay(bool with_stats, long long items, long long keys, int 
   return items <= sms && keys >= (with_stats || 3 * items <= 2 * sms ? 256 : 1024);
 }
 
-// The same for block-sparse attention. Alone, the lists may be of any length: 2 heads x 1024 block 128, one block a row
+enum class DenseKernel { kSingle, kPair, kLone };
+
+// Dense attention over bh heads of all batch entries. The single-CTA kernel records no row statistics.
+inline DenseKernel choose_dense_kernel(bool with_stats, long long bh, int seq_len, int max_ctas) {
+  const long long items = bh * ((static_cast<long long>(seq_len) + 127) / 128);
+  if (lone_ctas_pay(with_stats, items, seq_len, max_ctas)) return DenseKernel::kLone;
+  return with_stats || dense_pair_pays(bh, seq_len, max_ctas) ? DenseKernel::kPair : DenseKernel::kSingle;
+}
+
+// lone_ctas_pay for block-sparse attention. Alone, the lists may be of any length: 2 heads x 1024 block 128, one block a row
 // 5.85 -> 5.56, six 12.3 -> 10.5; 16 x 512 block 32 (walked as the union of four rows' lists) one 7.72 -> 7.15, ten 11.9
 // -> 10.4; 2 x 4096 block 32, twelve 21.8 -> 16.3; no blocks at all, 8 x 1024 block 32, 4.2 -> 3.7; one whole row among
 // rows of one block, 2 x 8192 block 64, 91 -> 71. Side by side (alone | a pair): block 128, 72 items x 128 keys 0.98 | 0.98,

@@ -1,10 +1,10 @@
-"""Both dense kernels behind sparsed_attn_full.
+"""Every dense kernel behind sparsed_attn_full and sparsed_attn_full_stats.
 
-sparsed_attn_full_stats always runs the kernel whose MMAs span CTA pairs; sparsed_attn_full runs it from 4096 tokens
-on where that pays (tests/test_dense_choice.py) and the single-CTA kernel elsewhere, unless
-SPARSED_DENSE_KERNEL=pair|single (read once per process) names one. The oracle parity tests of the dense pass are re-run in child processes with each setting, so that the
-pair kernel is also checked on what the statistics path never gives it (lengths that are no multiple of 32, strided
-layouts, a softmax scale, the rescaling path) and the single-CTA kernel on the long workloads."""
+Which one runs goes by the number of query tiles and keys (tests/test_dense_choice.py), unless SPARSED_DENSE_KERNEL=
+pair|single|lone (read once per process) names one; the single-CTA kernel records no row statistics, so a pass that does is
+not sent there. The oracle parity tests of the dense pass are re-run in child processes with each setting, so that each
+kernel is also checked on what its own rule never or seldom gives it: lengths that are no multiple of 32, strided layouts, a
+softmax scale, the rescaling path, short and long workloads."""
 import os
 import subprocess
 import sys
@@ -17,7 +17,10 @@ ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 @pytest.mark.parametrize("kernel,files,keyword", [
     ("pair", ["tests/test_gpu_parity_small.py", "tests/test_gpu_more_cases.py"], "attn_full or entry_point"),
+    ("pair", ["tests/test_gpu_switch_step_stats.py"], "matches_oracle"),
+    ("single", ["tests/test_gpu_parity_small.py", "tests/test_gpu_more_cases.py"], "attn_full or entry_point"),
     ("single", ["tests/test_gpu_parity_configs.py"], "config3"),
+    ("lone", ["tests/test_gpu_parity_small.py", "tests/test_gpu_more_cases.py"], "attn_full or entry_point"),
 ])
 def test_dense_parity_suite_with_one_kernel_forced(kernel, files, keyword):
     env = dict(os.environ, SPARSED_DENSE_KERNEL=kernel)
