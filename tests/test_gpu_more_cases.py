@@ -181,6 +181,47 @@ def test_token_major_layout_through_every_entry_point():
     assert sd.sparsed_last_device_status(ws) == (0, 0)
 
 
+@pytest.mark.parametrize("B,Hq,Hkv,L,bs", [(2, 8, 4, 1280, 64), (2, 8, 2, 1312, 32), (2, 10, 5, 1152, 128)])
+def test_token_major_layout_and_scale_with_more_query_tiles_than_sms(B, Hq, Hkv, L, bs):
+    """The kernels of larger grids (plain dense, dense with statistics, sparse): token-major Q, K, V and O give the bits
+    that head-major ones do, with a softmax scale and two batch entries, and these agree with the oracle."""
+    assert B * Hq * ((L + 127) // 128) > torch.cuda.get_device_properties(0).multi_processor_count
+    scale, rho, nb, group = 0.11, 0.3, L // bs, Hq // Hkv
+    qkv = syn.make_qkv(syn.AttnConfig("tm2", B, Hq, Hkv, L, 128, bs, rho, 0, seed=124), DEV)
+    params = sd.make_params(bs, rho, 0)
+    kp, kg = sd.sparsed_kept_per_row(params, L)
+    ws = sd.new_workspace(256, DEV)
+    out = []
+    for token_major in (False, True):
+        q, k, v = (t.transpose(1, 2).contiguous().transpose(1, 2) for t in qkv) if token_major else qkv
+        assert q.is_contiguous() != token_major
+        o_plain, o_stats, o_sparse = (torch.full_like(q, float("nan")) for _ in range(3))   # (strides of q)
+        assert o_plain.stride() == q.stride()
+        lse = torch.empty(B, Hq, L, dtype=torch.float32, device=DEV)
+        stats = sd.new_tile_stats(q, bs)
+        pat, rp, ci = sd.new_pattern(B, Hq, nb, kp + kg, DEV)
+        sd.sparsed_attn_full(q, k, v, o_plain, None, ws, softmax_scale=scale)
+        sd.sparsed_attn_full_stats(q, k, v, o_stats, lse, stats, ws, bs, softmax_scale=scale)
+        sd.sparsed_select_from_stats(q, k, params, lse, stats, pat, ws)
+        sd.sparsed_attn_sparse(q, k, v, o_sparse, pat, ws, softmax_scale=scale)
+        torch.cuda.synchronize()
+        assert sd.sparsed_last_device_status(ws) == (0, 0)
+        assert torch.equal(o_plain, o_stats)
+        out.append((o_plain, lse, rp, ci, o_sparse))
+    for head_major, token_major in zip(*out):
+        assert torch.equal(head_major, token_major)
+    o_plain, lse, rp, ci, o_sparse = out[0]
+    b, h = 1, Hq - 1
+    qd, kd, vd = (to_f64(t[b:b + 1, i:i + 1]) for t, i in zip(qkv, (h, h // group, h // group)))
+    o_ref, lse_ref = orc.attn_full(qd, kd, vd, scale=float(np.float32(scale)))
+    check_outputs(o_plain[b:b + 1, h:h + 1], o_ref, "full")
+    np.testing.assert_allclose(to_f64(lse[b:b + 1, h:h + 1]), lse_ref, atol=3e-5, rtol=3e-6)
+    r = (b * Hq + h) * nb
+    rp_h = rp[r:r + nb + 1].cpu().numpy()
+    o_ref = orc.attn_sparse(qd, kd, vd, rp_h - rp_h[0], ci.cpu().numpy()[rp_h[0]:rp_h[-1]], bs, scale=float(np.float32(scale)))
+    check_outputs(o_sparse[b:b + 1, h:h + 1], o_ref, "sparse")
+
+
 def test_ctas_that_run_through_several_query_tiles_match_one_tile_per_cta():
     """Block-sparse launches with more query tiles than CTAs fit on the device let every CTA roll on into
     further tiles (ring slots, S buffers and barrier phases carry over). 768 query tiles with ragged
