@@ -127,7 +127,7 @@ __device__ __forceinline__ float warp_column_sums(float (&v)[32], int lane) {
 __device__ __forceinline__ float2 twice(float c) { return make_float2(c, c); }
 
 // 2^x without the exponential unit: x = n + f with n whole and |f| <= 1/2, 2^f by the polynomial of degree 6 with the least
-// largest relative error there (1.9e-9, found by Lawson's reweighted least squares; 7.8e-8 with its fp32 roundings, where
+// largest relative error there (1.9e-9, found by Lawson's reweighted least squares; 7.9e-8 with its fp32 roundings, where
 // ex2.approx has 2^-22), times 2^n put together from its bits. The clamps keep n in [-127, 128], whose bits are those of 0
 // and infinity, and hand NaN on.
 __device__ __forceinline__ float2 exp2_by_polynomial(float2 x) {
