@@ -45,11 +45,11 @@ _C2_ATTN = "ncu capture of one launch on the 8k workload (summary under profiles
 _C2_POOL = "ncu capture of one launch on the 8k workload (summary under profiles/)"
 _ATTN_SRC = ("paper_2509_24014_b200/csrc/attention.cu", "paper_2509_24014_b200/csrc/work_items.cuh",
              "paper_2509_24014_b200/csrc/softmax_pipeline.cuh", "paper_2509_24014_b200/csrc/sm100_primitives.cuh")
-_ATTN_SHA = "5bc5f2cb7baa"
+_ATTN_SHA = "e7ca22932b08"
 _PAIR_SRC = ("paper_2509_24014_b200/csrc/attention_dense_pair.cu", "paper_2509_24014_b200/csrc/sm100_pair_primitives.cuh",
              "paper_2509_24014_b200/csrc/softmax_pipeline.cuh", "paper_2509_24014_b200/csrc/sm100_primitives.cuh",
              "paper_2509_24014_b200/build.py")   # (its compile flags are set per file there)
-_PAIR_SHA = "ca7aa076cc3b"
+_PAIR_SHA = "6be259e89da8"
 _POOL_SRC = ("paper_2509_24014_b200/csrc/pool_select.cu", "paper_2509_24014_b200/csrc/topk_device.cuh")
 _POOL_SHA = "11ccb7f1aa7d"
 NCU_DRAM_TRAFFIC = {
@@ -595,7 +595,7 @@ def run_ours(args, cfg):
                 "traffic": traffic, "traffic_source": source,
                 "note": "event time of a single launch includes launch latency; L2 flushed before it"}
 
-    # the dense pass of the step records row statistics: that entry point runs the CTA-pair kernel
+    # the dense pass of the step records row statistics: from 149 query tiles on that entry point runs the CTA-pair kernel
     roof_dense = tensor_roofline("attn_dense_pair_kernel", dense_flops(cfg_work), full_ms)
     roof_sparse = tensor_roofline("attn_kernel<sparse>", sparse_flops(cfg_work, nnz), sparse_ms)
     launches_per_step = 3

@@ -15,8 +15,8 @@ PKG_DIR = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(PKG_DIR, "csrc")
 OBJ_DIR = os.path.join(PKG_DIR, "build")
 LIB_PATH = os.path.join(PKG_DIR, "libsparsed.so")
-SOURCES = ["api.cu", "attention.cu", "attention_lone.cu", "attention_dense_pair.cu", "attention_dense_pair_split.cu", "scoring.cu", "topk.cu",
-           "pool_select.cu", "patterns.cu", "pooled_qk.cu"]
+SOURCES = ["api.cu", "attention.cu", "attention_lone.cu", "attention_dense_pair.cu", "attention_dense_pair_split.cu",
+           "scoring.cu", "topk.cu", "pool_select.cu", "patterns.cu", "pooled_qk.cu"]
 HEADERS = ["internal.h", "dense_choice.h", "attention_dense_pair.cu", "sm100_primitives.cuh", "sm100_pair_primitives.cuh",
            "softmax_pipeline.cuh", "work_items.cuh", "topk_device.cuh", os.path.join("..", "..", "include", "sparsed.h")]
 ARCH_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a"]

@@ -1,7 +1,7 @@
-// Attention for head_dim 128, bf16 in / bf16 out, fp32 softmax, on sm_100a, from one kernel:
-// dense bidirectional attention (Eq. 1 times V; the full-attention branch of Algorithm 1) and
-// block-sparse attention over CSR block lists (Eq. 3 / Eq. 4 times V; the "Sparse Reusing" branch). Grids of up to one
-// query tile per SM go to attention_lone.cu, large dense ones to attention_dense_pair.cu (dense_choice.h).
+// Attention for head_dim 128, bf16 in / bf16 out, fp32 softmax, on sm_100a: dense bidirectional attention (Eq. 1 times V;
+// the full-attention branch of Algorithm 1) and block-sparse attention over CSR block lists (Eq. 3 / Eq. 4 times V; the
+// "Sparse Reusing" branch). Two more kernels do parts of the same work: attention_lone.cu most grids of up to one query
+// tile per SM, attention_dense_pair.cu large dense ones and dense ones with row statistics (dense_choice.h).
 //
 // One CTA owns 128 consecutive query rows of one (batch, head) and streams 64-key tiles through a
 // warp-specialised pipeline:

@@ -1,5 +1,6 @@
-// Attention (dense, with or without the row statistics of the switch step, and block-sparse over CSR block lists) for grids of no more query tiles than the device has SMs: the
-// work of attention.cu, bit for bit, by a CTA that has an SM to itself.
+// Attention (dense, with or without the row statistics of the switch step, and block-sparse over CSR block lists) for
+// grids of no more query tiles than the device has SMs: the work of attention.cu, bit for bit, by a CTA that has an SM to
+// itself.
 //
 // What bounds such a grid is one CTA's chain of 64-key tiles. In attention.cu that is 1290 clocks a tile: one warp issues
 // both kinds of MMAs, each batch with a commit and a poll of its own, and one group of softmax warps waits for its logits,
@@ -12,10 +13,12 @@
 //   warps 4-7, 8-11: two groups of softmax warps, one thread per row each; group g takes tiles g, g + 2, ...; a warp and
 //                    the one of the other group with the same 32 rows pass the rows' state (reference maximum, sum) on
 //                    from tile to tile through shared memory
-// and a tile takes 960 clocks, 0.49 us: 2 heads x 4096 tokens 44.0 -> 35.8 us, 2 x 1024 14.7 -> 12.1. What bounds it now is
-// the SM's link to L2: 32 KB of K and V a tile are 66 GB/s, and bulk copies alone get 71.2 GB/s into an SM, however many
-// SMs take part. (One issuer for both: 46.9 and 14.9 us. Q from shared memory and one loading warp: 37.7 and 13.2. The
-// next tile's logits copied while a tile is finished, or each tile's columns split between two warps, 16 in all: no gain.)
+// and a tile takes 960 clocks, 0.49 us: 2 heads x 4096 tokens 44.0 -> 35.8 us, 2 x 1024 14.8 -> 11.9. What bounds it now is
+// the chain of a tile's steps, none of them alone: copies with work left out took, instead of 36.0 us (2 x 4096), 35.9 with
+// K and V loaded for the first five tiles only, 34.0 without exponentials, 35.0 without either. (32 KB of K and V a tile are
+// 66 GB/s; bulk copies alone get 71.2 GB/s into an SM, however many SMs take part.)
+// (One issuer for both: 46.9 and 14.9 us. Q from shared memory and one loading warp: 37.7 and 13.2. The next tile's logits
+// copied while a tile is finished, or each tile's columns split between two warps, 16 in all: no gain.)
 // A tile is exponentiated against the reference its group knows, before the tile before it is known to have kept it; if
 // it has not (rare, softmax_pipeline.cuh), the tile is done again from S, which is still in tensor memory. P is handed
 // over only after that. So rows see the same maxima, and sums and products are added in the same order, as with one group.

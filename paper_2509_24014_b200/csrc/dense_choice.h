@@ -6,9 +6,9 @@ namespace sparsed {
 // Whether the last wave of `clusters` clusters over `pairs` SM pairs runs as clusters of one stream each. Such a
 // cluster takes 0.65-0.8 of the time of one with two. So a last wave that would leave half of the SM pairs idle or
 // more is launched that way: 16 x 3072 (1.3 waves) 95.0 -> 84.4 us (statistics recorded). So is a grid of less than half
-// a wave, but only those of fewer than 256 keys come here (choose_dense_kernel). From two full waves on the launch runs
-// into the power limit, which an emptier last wave only relieves: 32 x 4096 (3.46 waves) at 1755 MHz where 37 x 4096 (4.0)
-// is at 1687, no gain.
+// a wave, but only those of fewer than 256 keys come here (choose_dense_kernel). From two full waves on it gained nothing
+// (32 x 4096, 3.46 waves): there the launch is at the power limit, and an emptier last wave raises the clock (1755 MHz
+// against 1687 at 37 x 4096, 4.0 waves), which leaves 5 % of its cost (979 against 1029 TFLOP/s).
 inline bool dense_pair_splits(long long clusters, long long pairs) {
   const long long last = pairs > 0 ? clusters % pairs : 0;
   return last != 0 && 2 * last <= pairs && clusters < 2 * pairs;

@@ -58,8 +58,8 @@ inline cudaError_t launch_overlapped(void (*kernel)(Params...), long long ctas, 
 
 // Parameters shared by the dense and the block-sparse attention kernels.
 struct AttnParams {
-  void* o;                 // bf16 [B,Hq,L,D]; used by the plain dense kernel, which stores rows itself (the others
-                           // write O through its tensor map)
+  void* o;                 // bf16 [B,Hq,L,D]; used by the kernels that store rows themselves: plain dense (attention.cu)
+                           // and the one for small grids (attention_lone.cu). The others write O through its tensor map
   int64_t o_stride_b, o_stride_h, o_stride_t;
   float* lse;              // fp32 [B,Hq,L] or null
   float* tile_lse;         // fp32 [B*Hq, ceil(L/128), ceil(L/stat_keys), 128] or null: base-2 log-sum-exp of each row

@@ -29,8 +29,11 @@
 // block-row(s) fit in shared memory the CTA ranks them itself (warp_select_row) and writes the CSR lists.
 //
 // Measured on B200, from Q and K alone (two passes over the logits before, with two CTAs of four softmax warps):
-//   28 heads x 16384 tokens, block 128   6.21 -> 2.43 ms (kOnePass; exponential unit busy 73 % of the time on average over
-//                                        the SMs and 84 % on the busiest, at 4 heads: 1.73 waves)
+//   28 heads x 16384 tokens, block 128   6.21 -> 2.43 ms (kOnePass. At 1850 MHz 739 clocks a tile and SM, of which the
+//                                        exponential unit needs 512: it bounds the launch together with what its warps
+//                                        wait for. Half of the exponentials left out 523 clocks, all of them 498, but the
+//                                        clock then falls to 1.6 GHz under the power limit: 1.99 and 1.92 ms. Fold and
+//                                        ranking are 1.4 %. No step at whole waves: 203-206 us a wave, 14 to 36 heads)
 //   32 heads x 8192 tokens, block 128    1.79 -> 0.72 ms (kOnePass)
 //   28 heads x 16384 tokens, block 64    6.24 -> 3.00 ms (kOnePassWide; in two passes 5.0)
 //   8 heads x 65536 tokens, block 128    27.4 -> 12.8 ms (kOnePassMost; in two passes 22.3)
@@ -64,8 +67,10 @@ __host__ __device__ constexpr int block_sums(int mode) { return tmem_sums(mode) 
 
 // Of 16 pairs of exponentials, how many are taken off the exponential unit (exp2_by_polynomial, 16 instructions a pair).
 // Only where one CTA per SM leaves issue slots: 28 x 16384 block 64 3292 -> 2996 us with two, 3078 with three, 2982 with
-// four; 8 x 65536 block 128 14040 -> 13266, 12800, 13108. With two CTAs per SM the launch is at its power limit instead
-// (28 x 16384 block 128 2458, 2460, 2443, 2493), or short of work (2 x 1024 13.9, 13.9, 14.8, 14.6).
+// four; 8 x 65536 block 128 14040 -> 13266, 12800, 13108. As chosen, 32 x 24576 block 64 8190 -> 7445, 28 x 8704 block 64
+// 950 -> 869, 16 x 8192 block 32 498 -> 459, 8 x 49152 block 128 7966 -> 7268, 2 x 16384 block 32 (512 key blocks) 282 ->
+// 257. With two CTAs per SM there is nothing to gain (28 x 16384 block 128 2458, 2460, 2443, 2493; 2 x 1024 13.9, 13.9,
+// 14.8, 14.6): fewer clocks there run at a lower clock, see above.
 __host__ __device__ constexpr int poly_pairs(int mode) { return mode == kOnePassMost ? 3 : mode == kOnePassWide ? 2 : 0; }
 
 // A row's reference is the maximum of both groups' first 64-key tiles, and stays until the sum of a later tile outgrows
